@@ -167,9 +167,7 @@ static void free_tables(pat_geometry* g) {
     cudaFree(g->pc.krow);
     cudaFree(g->pc.kcol);
     cudaFree(g->pc.tile_kmax);
-    cudaFree(g->adj_rays);
-    cudaFree(g->adj_ray_geo);
-    g->adj_ray_geo = nullptr;
+    cudaFree(g->adj_rec);
     cudaFree(g->adj_item);
     cudaFree(g->fwd_units);
     cudaFree(g->fwd_ctas);
@@ -179,7 +177,7 @@ static void free_tables(pat_geometry* g) {
     g->fwd_ctas = nullptr;
     g->fwd_roff = nullptr;
     g->fwd_rgs = nullptr;
-    g->adj_rays = nullptr;
+    g->adj_rec = nullptr;
     g->adj_item = nullptr;
     g->pc.tile_kmax = nullptr;
     g->det = nullptr;
@@ -525,27 +523,28 @@ struct AdjWork {
     std::vector<float> cost;
 };
 
-// The K^T work list of geometry d for a GPU that holds `slots` K^T CTAs at once.
+// The K^T work list of geometry d for a GPU that holds `slots` K^T CTAs at once: tiles of
+// `side` pixels, work items of at least `min_piece` candidates.
 static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, double slots, AdjWork& w,
-                            int waves = ADJ_WAVES) {
+                            int side, long long min_piece, int waves = ADJ_WAVES) {
     const int N = d.n, D = d.n_det, T = d.n_t, M = d.quad_m;
     const double hx = (d.xmax - d.xmin) / N, hy = (d.ymax - d.ymin) / N;
     const double ex = 1e-3 * hx, ey = 1e-3 * hy;
     const std::vector<float2>& det = pt.det;
     const std::vector<float2>& cs = pt.cs;
-    // K^T candidate boxes: for every WTILE x WTILE work tile and detector, the (k, m)
-    // polar box of the tile's tap region (points with i0 in [x0-1, x0+WTILE-1], same in
+    // K^T candidate boxes: for every side x side work tile and detector, the (k, m)
+    // polar box of the tile's tap region (points with i0 in [x0-1, x0+side-1], same in
     // y), with one index of margin on every side; FP64 on the host
     w.tiles_x = (N + ATILE - 1) / ATILE;
     w.tiles = w.tiles_x * w.tiles_x;
-    const int tiles_x = (N + WTILE - 1) / WTILE, tiles = tiles_x * tiles_x;
+    const int tiles_x = (N + side - 1) / side, tiles = tiles_x * tiles_x;
     w.wtiles_x = tiles_x;
     w.wtiles = tiles;
     std::vector<int4> box((size_t)tiles * D);
     for (int t = 0; t < tiles; ++t) {
-        const int x0 = (t % tiles_x) * WTILE, y0 = (t / tiles_x) * WTILE;
-        const double rx0 = d.xmin + (x0 - 0.5) * hx - ex, rx1 = d.xmin + (x0 + WTILE + 0.5) * hx + ex;
-        const double ry0 = d.ymin + (y0 - 0.5) * hy - ey, ry1 = d.ymin + (y0 + WTILE + 0.5) * hy + ey;
+        const int x0 = (t % tiles_x) * side, y0 = (t / tiles_x) * side;
+        const double rx0 = d.xmin + (x0 - 0.5) * hx - ex, rx1 = d.xmin + (x0 + side + 0.5) * hx + ex;
+        const double ry0 = d.ymin + (y0 - 0.5) * hy - ey, ry1 = d.ymin + (y0 + side + 0.5) * hy + ey;
         for (int di = 0; di < D; ++di) {
             const double dx = d.det_xy_host[2 * di], dy = d.det_xy_host[2 * di + 1];
             const double cx = std::min(std::max(dx, rx0), rx1), cy = std::min(std::max(dy, ry0), ry1);
@@ -583,7 +582,7 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
 
     // K^T work list.  Every ray (detector d, angle m) of a tile's polar box is cut to the
     // radius interval where its points can have taps in the tile's window [x0 - 1, x0 +
-    // WTILE) x [y0 - 1, y0 + WTILE) (the window is convex, so the interval is one
+    // side) x [y0 - 1, y0 + side) (the window is convex, so the interval is one
     // segment).  The cut is FP64 arithmetic on the same FP32 tables the kernels read, on
     // the window widened by 1e-3 pixel, far beyond the FP32 rounding of a point's position
     // (about 1e-5 pixel); the kernel still tests every candidate exactly.  A tile's non-empty segments, concatenated, are its
@@ -598,9 +597,9 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
         std::vector<long long> tile_base(tiles + 1, 0), tile_total(tiles, 0);
         for (int t = 0; t < tiles; ++t) {
             tile_base[t] = (long long)rays.size();
-            const int x0 = (t % tiles_x) * WTILE, y0 = (t / tiles_x) * WTILE;
-            const double wx0 = x0 - 1.001, wx1 = x0 + WTILE + 0.001;
-            const double wy0 = y0 - 1.001, wy1 = y0 + WTILE + 0.001;
+            const int x0 = (t % tiles_x) * side, y0 = (t / tiles_x) * side;
+            const double wx0 = x0 - 1.001, wx1 = x0 + side + 0.001;
+            const double wy0 = y0 - 1.001, wy1 = y0 + side + 0.001;
             long long pre = 0;
             for (int di = 0; di < D; ++di) {
                 const int4 bx = box[(size_t)t * D + di];
@@ -645,10 +644,10 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
         long long total = 0;
         for (int t = 0; t < tiles; ++t) total += tile_total[t];
         w.candidates = total;
-        // pieces per tile: `waves` waves of resident CTAs (at least 1024 candidates a piece),
+        // pieces per tile: `waves` waves of resident CTAs (at least min_piece candidates a piece),
         // each piece going to the tile whose pieces are largest at that point, which
         // minimises the largest piece
-        const long long Q = std::max(1LL, std::min((long long)(waves * slots), total / 1024));
+        const long long Q = std::max(1LL, std::min((long long)(waves * slots), total / min_piece));
         std::vector<long long> n_piece(tiles, 0);
         {
             std::priority_queue<std::pair<double, int>> heap;   // (piece size, tile)
@@ -712,6 +711,38 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
         }
     }
     return PAT_OK;
+}
+
+// The device records of a work list: an item takes the ray segments whose first candidate
+// lies in its share [c0, c1), so segments stay whole.  Neighbouring records go to the lanes
+// of one warp, so each kind is sorted longest first and the first kind is filled up to whole
+// warps with empty records.
+static void adjoint_records(const pat_geometry_desc& d, const PointTables& pt, const AdjWork& w,
+                            std::vector<AdjRec>& recs, std::vector<AdjWorkItem>& items) {
+    const int Tp = row_stride(d.n_t);
+    auto longest = [](const AdjRec& a, const AdjRec& b) { return a.n > b.n; };
+    recs.reserve(w.rays.size() + w.items.size() * AROWS);
+    std::vector<AdjRec> kind[2];
+    for (const AdjItem& it : w.items) {
+        kind[0].clear();
+        kind[1].clear();
+        for (int r = it.ray0; r < it.ray0 + it.nray; ++r) {
+            const int4 ray = w.rays[r];
+            if (ray.w < it.c0) continue;   // begins in the item before
+            const float2 det = pt.det[ray.x], cs = pt.cs[ray.y];
+            const bool fast_y = std::fabs(cs.y) > std::fabs(cs.x);
+            const int k0 = ray.z & ~1, n = ray.z - k0 + w.rays[r + 1].w - ray.w;
+            AdjRec q{fast_y ? det.y : det.x, fast_y ? det.x : det.y, fast_y ? cs.y : cs.x, fast_y ? cs.x : cs.y,
+                     (unsigned)((long long)ray.x * Tp + k0), (unsigned)((long long)ray.x * d.n_t + k0), (float)k0, n};
+            kind[fast_y].push_back(q);
+        }
+        std::stable_sort(kind[0].begin(), kind[0].end(), longest);
+        std::stable_sort(kind[1].begin(), kind[1].end(), longest);
+        while (kind[0].size() % AROWS) kind[0].push_back(AdjRec{});
+        items.push_back(AdjWorkItem{it.tile, (int)recs.size(), (int)(kind[0].size() + kind[1].size()), (int)kind[0].size()});
+        recs.insert(recs.end(), kind[0].begin(), kind[0].end());
+        recs.insert(recs.end(), kind[1].begin(), kind[1].end());
+    }
 }
 
 // Angular windows of every (detector, group of KGRP radii): the smallest circular interval
@@ -815,40 +846,32 @@ static int install_adjoint_plan(pat_geometry* g, const PointTables& pt, int wave
     pat_geometry_desc dd = g->desc;
     dd.det_xy_host = g->det_xy.data();
     AdjWork aw;
-    const int rc = adjoint_worklist(dd, pt, (double)sm_count() * adjoint_blocks_per_sm(), aw, waves);
+    // (every item zeroes and flushes a copy of its tile, so it should have candidates enough)
+    const int side = work_tile_side(dd.n, dd.n_det, dd.n_t, dd.quad_m);
+    const int rc = adjoint_worklist(dd, pt, (double)sm_count() * adjoint_blocks_per_sm(), aw, side,
+                                    side == WTILE_SMALL ? 1024 : 4096, waves);
     if (rc) return rc;
-    const std::vector<int4>& rays = aw.rays;
-    const std::vector<AdjItem>& items = aw.items;
-    // each segment's detector and direction next to it, so the K^T staging reads them in
-    // one coalesced pass (sentinels get zeros)
-    std::vector<float4> geo(rays.size());
-    for (size_t i = 0; i < rays.size(); ++i)
-        geo[i] = rays[i].x >= 0
-                     ? make_float4(pt.det[rays[i].x].x, pt.det[rays[i].x].y, pt.cs[rays[i].y].x, pt.cs[rays[i].y].y)
-                     : make_float4(0.f, 0.f, 0.f, 0.f);
-    int4* r_dev = nullptr;
-    float4* geo_dev = nullptr;
-    AdjItem* it_dev = nullptr;
-    cudaError_t e = cudaMalloc(&r_dev, sizeof(int4) * std::max<size_t>(rays.size(), 1));
-    if (e == cudaSuccess) e = cudaMemcpy(r_dev, rays.data(), sizeof(int4) * rays.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&geo_dev, sizeof(float4) * std::max<size_t>(geo.size(), 1));
-    if (e == cudaSuccess) e = cudaMemcpy(geo_dev, geo.data(), sizeof(float4) * geo.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&it_dev, sizeof(AdjItem) * std::max<size_t>(items.size(), 1));
-    if (e == cudaSuccess) e = cudaMemcpy(it_dev, items.data(), sizeof(AdjItem) * items.size(), cudaMemcpyHostToDevice);
+    std::vector<AdjRec> recs;
+    std::vector<AdjWorkItem> items;
+    adjoint_records(dd, pt, aw, recs, items);
+    AdjRec* r_dev = nullptr;
+    AdjWorkItem* it_dev = nullptr;
+    cudaError_t e = cudaMalloc(&r_dev, sizeof(AdjRec) * std::max<size_t>(recs.size(), 1));
+    if (e == cudaSuccess) e = cudaMemcpy(r_dev, recs.data(), sizeof(AdjRec) * recs.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&it_dev, sizeof(AdjWorkItem) * items.size());
+    if (e == cudaSuccess) e = cudaMemcpy(it_dev, items.data(), sizeof(AdjWorkItem) * items.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         cudaFree(r_dev);
-        cudaFree(geo_dev);
         cudaFree(it_dev);
         return cuda_fail(e, "K^T work list upload");
     }
-    cudaFree(g->adj_rays);
-    cudaFree(g->adj_ray_geo);
+    cudaFree(g->adj_rec);
     cudaFree(g->adj_item);
-    g->adj_rays = r_dev;
-    g->adj_ray_geo = geo_dev;
+    g->adj_rec = r_dev;
     g->adj_item = it_dev;
     g->adj_tiles_x = aw.tiles_x;
     g->adj_tiles = aw.tiles;
+    g->adj_side = side;
     g->adj_wtiles_x = aw.wtiles_x;
     g->adj_candidates = aw.candidates;
     g->adj_item_cost = aw.cost;
@@ -1014,7 +1037,7 @@ extern "C" int pat_adjoint_worklist(const pat_geometry_desc* desc, int slots, in
         s = (double)sms * adjoint_blocks_per_sm();
     }
     AdjWork aw;
-    const int rc = adjoint_worklist(*desc, point_tables(*desc), s, aw);
+    const int rc = adjoint_worklist(*desc, point_tables(*desc), s, aw, WTILE_ABI, 1024);
     if (rc) return rc;
     counts3_host[0] = (long long)aw.rays.size();
     counts3_host[1] = (long long)aw.items.size();

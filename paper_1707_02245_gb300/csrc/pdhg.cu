@@ -832,7 +832,7 @@ static int alloc_workspace(const pat_geometry* g, int reg, Workspace& ws, cudaSt
     size_t sz[17] = {nx * 4, nx * 4, ny * 4, ny * 4, S * 4, NN * 4, NN * 4 * 2,
                      (reg == PAT_TGV ? 2 * NN : 1) * 4,
                      NN * 4, S * 4, NN * 4, (size_t)ws.n_data * GAP_DATA_TERMS * 8, (size_t)ws.n_pix * GAP_PIX_TERMS * 8, sizeof(InfoDev),
-                     S * 4, nx * 2, nx * 2};
+                     (size_t)g->desc.n_det * row_stride(g->desc.n_t) * 4, nx * 2, nx * 2};
     size_t total = 0;
     for (int i = 0; i < 17; ++i) {
         off[i] = total;
@@ -1520,11 +1520,12 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
     if (int mrc = wav_model(g[0], &p[0], wm)) return mrc;
     const bool cwt = wm.kind == PAT_WAVELET_DTCWT;
     const long long NR = wm.nr;   // coefficients of W u
-    long long S = 0;              // the largest data size and K CTA count of the batch
+    long long S = 0, Sp = 0;      // the largest data size, padded data size and K CTA count of the batch
     int n_data = 0;
     for (int b = 0; b < B; ++b) {
         if (g[b]->desc.n != N) return fail(PAT_ERR_INVALID_ARG, std::string(who) + ": a wavelet batch needs one N");
         S = std::max(S, (long long)g[b]->desc.n_det * g[b]->desc.n_t);
+        Sp = std::max(Sp, (long long)g[b]->desc.n_det * row_stride(g[b]->desc.n_t));
         n_data = std::max(n_data, g[b]->fwd_n_ctas);
     }
     // one workspace block per problem (DT-CWT: R, WB, WU and SIGR hold 4 planes, SCRT the
@@ -1533,7 +1534,7 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
            NBUF };
     // SCR, SCR2: transform scratch (DT-CWT: the LL blocks passed between levels, 5 N^2 / 4)
     const size_t nn4 = (size_t)NN * 4, nr4 = (size_t)NR * 4, scr4 = cwt ? nn4 + nn4 / 4 : nn4;
-    const size_t sz[NBUF] = {nn4, nn4, nn4, (size_t)S * 4, (size_t)S * 4, (size_t)NN * 8, nr4, nr4, nn4, scr4, scr4,
+    const size_t sz[NBUF] = {nn4, nn4, nn4, (size_t)S * 4, (size_t)Sp * 4, (size_t)NN * 8, nr4, nr4, nn4, scr4, scr4,
                              nr4, nn4, nr4, (size_t)S * 4, (size_t)n_data * GAP_DATA_TERMS * 8,
                              (size_t)n_pix * GAP_PIX_TERMS * 8, sizeof(InfoDev), cwt ? nr4 : 16, 2 * sizeof(float),
                              (size_t)g[0]->adj_tiles * sizeof(float)};
