@@ -371,10 +371,10 @@ const char* pat_last_error(void);
 int  pat_geometry_info(const pat_geometry* g, long long* out6_host);
 
 /* Host only: the work list of the K^T kernel (Sec. 3.3.1's adjoint, evaluated by pixel
- * tiles) with tiles of 32 pixels, for a GPU that holds `slots` K^T CTAs at once.
- * pat_create_geometry builds its list with the same function (tiles of 32 or 64 pixels by
- * the amount of work) and gives an item the whole segments that begin in its share.  With
- * slots > 0 no CUDA call is made; slots <= 0 sizes it for the current device.  counts3_host = {ray segments, work items, candidate points}.
+ * tiles), for a GPU that holds `slots` K^T CTAs at once.  pat_create_geometry builds its list
+ * with the same function (without the limit of 1024 segments per item) and gives an item the
+ * whole segments that begin in its share.  With slots > 0 no CUDA call is made; slots <= 0
+ * sizes it for the current device.  counts3_host = {ray segments, work items, candidate points}.
  * rays_host (4 ints per segment: detector, angle index m, first radius index k,
  * exclusive prefix within its tile; after each tile a sentinel {-1, 0, 0, tile total})
  * and items_host (5 ints per item: tile, first segment, segment count, first and end

@@ -9,11 +9,11 @@ namespace pat {
 // ---------------------------------------------------------------------------------
 // K^T by pixel tiles with exact fixed-point accumulation.
 //
-// A CTA owns a share of one WTILE x WTILE pixel tile's candidate points (WTILE: see
-// work_tile_side).  Its shared accumulator (with a one-pixel ring, so every point whose taps
-// touch the tile can add all four weights) holds int32 fixed-point values: every pixel satisfies
+// A CTA owns a share of one WTILE x WTILE pixel tile's candidate points.  Its shared
+// accumulators (with a one-pixel ring, so every point whose taps touch the tile can add
+// all four weights) hold int32 fixed-point values: every pixel satisfies
 //   |(K^T y)(p)| <= max|y| * (K^T 1)(p)        (all entries of K are >= 0),
-// so with the scale S = 2^30 / (max|y| * max over the work tile of K^T 1) no partial sum
+// so with the scale S = 2^30 / (max|y| * max over the ATILE tile of K^T 1) no partial sum
 // of a tile pixel exceeds 2^30 and integer addition (native shared atomics, associative,
 // hence deterministic) replaces floating-point atomics.  The resolution 2^-30 of that
 // bound is finer than FP32 accumulation of the same terms.  Ring cells are dropped.
@@ -23,22 +23,27 @@ namespace pat {
 // into the tile's candidate list, and cuts the lists into nearly equal work items of whole
 // segments that fill one wave of resident CTAs.  Every candidate uses the forward projector's
 // FP32 position and tap arithmetic, so the CTA adds exactly the entries of K^T that belong to
-// its pixels.  Items of one tile share its scale, so their fixed-point tiles add exactly (in
-// any order) into one image with integer atomics.
+// its pixels.  Items of one scale tile share its scale, so their fixed-point tiles add exactly
+// (in any order) into one image with integer atomics.
 //
 // Bound: issue slots and the shared-memory atomics together.  At 256^2 with 256 detectors
-// (8.4 M points): 19.2 us per launch, 2.0 wavefronts per atomic and 14 M warp instructions,
-// against 26.5 us, 3.6 and 19 M for a kernel whose threads walked contiguous runs of the
-// candidate list one point at a time: there nearly every step of a warp held some lane's
-// segment change, and its lanes' pixels lay on random banks.
+// (8.4 M points): 18.8 us per launch, against 26.5 us for a kernel whose threads walked
+// contiguous runs of the candidate list one point at a time: there nearly every step of a
+// warp held some lane's segment change, and its lanes' pixels lay on random banks (3.6
+// wavefronts per atomic, 19 M warp instructions).  64^2 with 64 detectors: 6.0 -> 5.2 us;
+// an uneven batch of 8: 77 -> 63 us.  Tiles of 64 pixels with 16 lanes to a segment: 19.2 us.
 // ---------------------------------------------------------------------------------
 // Threads of a K^T CTA and resident CTAs per SM.  Fewer, larger CTAs zero and flush fewer tile
-// copies; the 64 registers of 2 x 512 threads hold the loop without spills (measured at 256^2:
-// 2 x 512 19.2 us, 1 x 1024 19.9, 4 x 256 20.5, 3 x 512 with spills 30).
+// copies; the 64 registers of 2 x 512 threads hold the loop without spills (measured at 256^2
+// on 64-pixel tiles: 2 x 512 19.2 us, 1 x 1024 19.9, 4 x 256 20.5, 3 x 512 with spills 30).
 constexpr int ATHREADS = 512;
 constexpr int ADJ_MIN_BLOCKS = 2;
-constexpr int acell(int side) { return side + 3; }   // cells per axis: the tile, its ring and one more for points outside
-constexpr int astride(int side) { return (2 * acell(side) + 31) / 32 * 32; }   // row stride of the accumulators: a cell's bank is its column mod 32
+constexpr int ACELL = WTILE + 3;     // cells per axis: the tile, its ring and one more for points outside
+constexpr int ACOPY = 48;            // columns from an accumulator to its second copy (16 banks on)
+constexpr int AKIND = 96;            // columns to the accumulators of the other kind of segment (0 banks on)
+constexpr int ASTRIDE = 192;         // row stride: a multiple of 32 words, so a cell's column alone is its bank
+static_assert(ACELL <= ACOPY && ACOPY + ACELL <= AKIND && AKIND + ACOPY + ACELL <= ASTRIDE, "accumulators side by side");
+static_assert(ASTRIDE % 32 == 0 && ACOPY % 32 == 16 && AKIND % 32 == 0, "banks of the accumulators");
 
 // One work item of K^T: the ray segments of its records.  ALANES lanes share a segment, each
 // with two neighbouring points at a time (their data are one aligned 8-byte load), so a warp
@@ -47,104 +52,135 @@ constexpr int astride(int side) { return (2 * acell(side) + 31) / 32 * 32; }   /
 // instruction; a point whose taps fall outside the tile window adds to the cells past the
 // ring, which are dropped with it, so the loop has no branch.
 //
-// Two accumulators hold the tile: the first with x along a row, the second with y along a
-// row.  A segment adds to the one whose rows run along its fast axis: its lanes then stand in
-// different columns, and with a row stride of a multiple of 32 words the column alone is the
-// bank.  Both are added before the tile leaves the CTA.
-template <bool PREMUL, int WTILE>
-__device__ __forceinline__ void adjoint_tile(const AdjArgs& a, int item_index, int* acc) {
-    constexpr int ACELL = acell(WTILE), ASTRIDE = astride(WTILE);
-    const AdjGeom& g = a.g;
-    const int N = g.n;
+// Banks: segments that advance fastest along x add to accumulators with x along a row, the
+// others to accumulators with y along a row, so the lanes of a segment stand in different
+// columns, and with a row stride of a multiple of 32 words the column alone is the bank.
+// Every second segment of a warp adds to a copy 16 banks on.  All four accumulators are added
+// before the tile leaves the CTA.  Wavefronts per atomic and lanes in use at 256^2: 3.1 and
+// 26.6 of 32 without the copies, 2.1 with them (16 lanes to a segment: 1.6 and 23.8).
+//
+// The order of the products of a tap is that of the axes, not of the kind of segment, so
+// tiles and work items of any shape give the same bits.
+struct AdjConst {
+    float2 dr, rh, scale;
+    const float* wk;
+    int T;
+};
+
+// The points of one segment that this lane takes.  FAST_Y: the row of the accumulator runs
+// along y.
+template <bool PREMUL, bool FAST_Y>
+__device__ __forceinline__ void adjoint_segment(const AdjConst& a, const float4 geo, const float4 seg, const float* __restrict__ y,
+                                                int sub2, int bm, int bs, int* cells) {
+    const float2 magic = make_float2(FLOOR_MAGIC, FLOOR_MAGIC), nmagic = make_float2(-FLOOR_MAGIC, -FLOOR_MAGIC);
+    const float2 one = make_float2(1.f, 1.f), mone = make_float2(-1.f, -1.f);
+    const int n = __float_as_int(seg.w);
+    const float2 dm = make_float2(geo.x, geo.x), ds = make_float2(geo.y, geo.y);
+    const float2 cm = make_float2(geo.z, geo.z), cs = make_float2(geo.w, geo.w);
+    const float* __restrict__ yp = y + (size_t)__float_as_uint(PREMUL ? seg.x : seg.y);
+    const float k0 = seg.z + (float)sub2;
+    float2 kf = make_float2(k0, k0 + 1.f);
+    for (int p = sub2; p < n; p += 2 * ALANES) {
+        float2 yv;
+        if (PREMUL) {
+            yv = __ldg(reinterpret_cast<const float2*>(yp + p));
+        } else {   // (the caller's array may lie on any 4-byte boundary and its rows have no padding)
+            const int k = (int)seg.z + p;
+            yv = make_float2(__ldg(yp + p) * __ldg(a.wk + k), k + 1 < a.T ? __ldg(yp + p + 1) * __ldg(a.wk + k + 1) : 0.f);
+        }
+        const float2 c = __fmul2_rn(yv, a.scale);
+        const float2 r = __ffma2_rn(kf, a.dr, a.rh);   // = rk[k], bit for bit (see radius())
+        kf = __fadd2_rn(kf, make_float2(2.f * ALANES, 2.f * ALANES));
+        const float2 fm = __ffma2_rn(r, cm, dm), fs = __ffma2_rn(r, cs, ds);
+        const float2 tm = __fadd2_rd(fm, magic), ts = __fadd2_rd(fs, magic);   // floor + 1.5 * 2^23, exactly
+        const float2 frm = __ffma2_rn(__fadd2_rn(tm, nmagic), mone, fm), frs = __ffma2_rn(__fadd2_rn(ts, nmagic), mone, fs);
+        const float2 omm = __ffma2_rn(frm, mone, one), oms = __ffma2_rn(frs, mone, one);
+        // taps (c (1 - ay)) (1 - ax), ...
+        const float2 c0 = __fmul2_rn(c, FAST_Y ? omm : oms), c1 = __fmul2_rn(c, FAST_Y ? frm : frs);
+        const float2 wl = FAST_Y ? oms : omm, wh = FAST_Y ? frs : frm;
+        const float2 v00 = __fmul2_rn(c0, wl), v11 = __fmul2_rn(c1, wh);
+        const float2 vx = __fmul2_rn(c0, wh), vy = __fmul2_rn(c1, wl);   // the tap further along x, along y
+        const float2 v10 = FAST_Y ? vy : vx, v01 = FAST_Y ? vx : vy;     // along the row, across rows
+        // tile-local cells straight from the floors' bits
+        {
+            const unsigned lm = min((unsigned)(__float_as_int(tm.x) - bm), (unsigned)(WTILE + 1));
+            const unsigned ls = min((unsigned)(__float_as_int(ts.x) - bs), (unsigned)(WTILE + 1));
+            int* t = cells + ls * ASTRIDE + lm;
+            atomicAdd(t, __float2int_rn(v00.x));
+            atomicAdd(t + 1, __float2int_rn(v10.x));
+            atomicAdd(t + ASTRIDE, __float2int_rn(v01.x));
+            atomicAdd(t + ASTRIDE + 1, __float2int_rn(v11.x));
+        }
+        {
+            const unsigned lm = min((unsigned)(__float_as_int(tm.y) - bm), (unsigned)(WTILE + 1));
+            const unsigned ls = min((unsigned)(__float_as_int(ts.y) - bs), (unsigned)(WTILE + 1));
+            int* t = cells + ls * ASTRIDE + lm;
+            atomicAdd(t, __float2int_rn(v00.y));
+            atomicAdd(t + 1, __float2int_rn(v10.y));
+            atomicAdd(t + ASTRIDE, __float2int_rn(v01.y));
+            atomicAdd(t + ASTRIDE + 1, __float2int_rn(v11.y));
+        }
+    }
+}
+
+template <bool PREMUL>
+__device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index) {
+    const int N = a.g.n;
     const int4 item = __ldg(reinterpret_cast<const int4*>(a.items + item_index));
     const int tile = item.x, nrec = item.z, split = item.w;
     const int x0 = (tile % a.wtiles_x) * WTILE, y0 = (tile / a.wtiles_x) * WTILE;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __shared__ __align__(16) int acc[ACELL * ASTRIDE];
     for (int c = tid; c < ACELL * ASTRIDE / 4; c += ATHREADS) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
     // the scale of the ATILE tile that holds this work tile
     const float bound = __uint_as_float(*a.ymax_bits) * __ldg(&a.tile_kmax[(y0 / ATILE) * a.tiles_x + x0 / ATILE]);
     const float scale = 1073741824.0f / bound;  // 2^30 / bound
-    const float* __restrict__ wk = g.wk;
     const float* __restrict__ y = a.y;
-    const int T = g.n_t;
     const float4* __restrict__ recs = reinterpret_cast<const float4*>(a.recs + item.y);
+    const AdjConst ac{make_float2(a.g.dr_f, a.g.dr_f), make_float2(a.g.rh_f, a.g.rh_f), make_float2(scale, scale), a.g.wk, a.g.n_t};
     constexpr int STEP = ATHREADS / ALANES;      // segments the CTA walks at once
     const int sub2 = 2 * (lane % ALANES);
-    const float sub2f = (float)sub2;
-    int j = warp * AROWS + lane / ALANES;
+    int first = warp * AROWS, j = first + lane / ALANES;
     const bool run = bound > 0.f && isfinite(bound);
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f), s = q;
     if (run && j < nrec) {
         q = __ldg(recs + 2 * j);
         s = __ldg(recs + 2 * j + 1);
     }
-    const float2 dr2 = make_float2(g.dr_f, g.dr_f), rh2 = make_float2(g.rh_f, g.rh_f);
-    const float2 magic = make_float2(FLOOR_MAGIC, FLOOR_MAGIC), nmagic = make_float2(-FLOOR_MAGIC, -FLOOR_MAGIC);
-    const float2 one = make_float2(1.f, 1.f), mone = make_float2(-1.f, -1.f), scale2 = make_float2(scale, scale);
     __syncthreads();
     if (run) {
-        for (int first = warp * AROWS; first < nrec; first += STEP) {
-            const float4 geo = q, seg = s;
+        int* cells = acc + (lane / ALANES % 2) * ACOPY;
+        const int bx = FLOOR_MAGIC_BITS + x0 - 1, by = FLOOR_MAGIC_BITS + y0 - 1;
+        // the next segment is loaded while this one is walked
+        auto advance = [&](float4& geo, float4& seg) {
+            geo = q;
+            seg = s;
             j += STEP;
+            first += STEP;
             s.w = 0.f;
-            if (j < nrec) {   // the next segment, while this one is walked
+            if (j < nrec) {
                 q = __ldg(recs + 2 * j);
                 s = __ldg(recs + 2 * j + 1);
             }
-            const int n = __float_as_int(seg.w);
-            const float2 dm = make_float2(geo.x, geo.x), ds = make_float2(geo.y, geo.y);
-            const float2 cm = make_float2(geo.z, geo.z), cs = make_float2(geo.w, geo.w);
-            // tile-local cells straight from the floors' bits
-            const bool fast_y = first >= split;
-            const int bm = FLOOR_MAGIC_BITS + (fast_y ? y0 : x0) - 1, bs = FLOOR_MAGIC_BITS + (fast_y ? x0 : y0) - 1;
-            int* cells = acc + (fast_y ? ACELL : 0);
-            const float* __restrict__ yp = y + (size_t)__float_as_uint(PREMUL ? seg.x : seg.y);
-            float2 kf = make_float2(seg.z + sub2f, seg.z + sub2f + 1.f);
-            for (int p = sub2; p < n; p += 2 * ALANES) {
-                float2 yv;
-                if (PREMUL) {
-                    yv = __ldg(reinterpret_cast<const float2*>(yp + p));
-                } else {   // (the caller's array may lie on any 4-byte boundary and its rows have no padding)
-                    const int k = (int)seg.z + p;
-                    yv = make_float2(__ldg(yp + p) * __ldg(wk + k), k + 1 < T ? __ldg(yp + p + 1) * __ldg(wk + k + 1) : 0.f);
-                }
-                const float2 c = __fmul2_rn(yv, scale2);
-                const float2 r = __ffma2_rn(kf, dr2, rh2);   // = rk[k], bit for bit (see radius())
-                kf = __fadd2_rn(kf, make_float2(2.f * ALANES, 2.f * ALANES));
-                const float2 fm = __ffma2_rn(r, cm, dm), fs = __ffma2_rn(r, cs, ds);
-                const float2 tm = __fadd2_rd(fm, magic), ts = __fadd2_rd(fs, magic);   // floor + 1.5 * 2^23, exactly
-                const float2 frm = __ffma2_rn(__fadd2_rn(tm, nmagic), mone, fm), frs = __ffma2_rn(__fadd2_rn(ts, nmagic), mone, fs);
-                const float2 omm = __ffma2_rn(frm, mone, one), oms = __ffma2_rn(frs, mone, one);
-                const float2 c0 = __fmul2_rn(c, oms), c1 = __fmul2_rn(c, frs);
-                const float2 v00 = __fmul2_rn(c0, omm), v10 = __fmul2_rn(c0, frm);
-                const float2 v01 = __fmul2_rn(c1, omm), v11 = __fmul2_rn(c1, frm);
-                {
-                    const unsigned lm = min((unsigned)(__float_as_int(tm.x) - bm), (unsigned)(WTILE + 1));
-                    const unsigned ls = min((unsigned)(__float_as_int(ts.x) - bs), (unsigned)(WTILE + 1));
-                    int* t = cells + ls * ASTRIDE + lm;
-                    atomicAdd(t, __float2int_rn(v00.x));
-                    atomicAdd(t + 1, __float2int_rn(v10.x));
-                    atomicAdd(t + ASTRIDE, __float2int_rn(v01.x));
-                    atomicAdd(t + ASTRIDE + 1, __float2int_rn(v11.x));
-                }
-                {
-                    const unsigned lm = min((unsigned)(__float_as_int(tm.y) - bm), (unsigned)(WTILE + 1));
-                    const unsigned ls = min((unsigned)(__float_as_int(ts.y) - bs), (unsigned)(WTILE + 1));
-                    int* t = cells + ls * ASTRIDE + lm;
-                    atomicAdd(t, __float2int_rn(v00.y));
-                    atomicAdd(t + 1, __float2int_rn(v10.y));
-                    atomicAdd(t + ASTRIDE, __float2int_rn(v01.y));
-                    atomicAdd(t + ASTRIDE + 1, __float2int_rn(v11.y));
-                }
-            }
+        };
+        float4 geo, seg;
+        while (first < split) {
+            advance(geo, seg);
+            adjoint_segment<PREMUL, false>(ac, geo, seg, y, sub2, bx, by, cells);
+        }
+        cells += AKIND;
+        while (first < nrec) {
+            advance(geo, seg);
+            adjoint_segment<PREMUL, true>(ac, geo, seg, y, sub2, by, bx, cells);
         }
     }
     __syncthreads();
-    // the first accumulator += the second transposed, along diagonals: a warp's cells lie in
-    // 32 different columns of both
+    // the accumulators with x along a row += those with y along a row, along diagonals: a
+    // warp's cells lie in 32 different columns of each
     for (int c = tid; c < WTILE * WTILE; c += ATHREADS) {
-        const int lx = c & (WTILE - 1), ly = (lx + c / WTILE) & (WTILE - 1);
-        acc[(ly + 1) * ASTRIDE + lx + 1] += acc[(lx + 1) * ASTRIDE + ACELL + ly + 1];
+        const int lx = c % WTILE, ly = (lx + c / WTILE) % WTILE;
+        const int* ty = acc + (lx + 1) * ASTRIDE + AKIND + ly + 1;
+        acc[(ly + 1) * ASTRIDE + lx + 1] += ty[0] + ty[ACOPY];
     }
     __syncthreads();
     // work items of one tile share its scale, so their fixed-point partial sums add
@@ -153,18 +189,10 @@ __device__ __forceinline__ void adjoint_tile(const AdjArgs& a, int item_index, i
         const int lx = c % WTILE, ly = c / WTILE;
         const int gx = x0 + lx, gy = y0 + ly;
         if (gx >= N || gy >= N) continue;
-        const int v = acc[(ly + 1) * ASTRIDE + lx + 1];
+        const int* t = acc + (ly + 1) * ASTRIDE + lx + 1;
+        const int v = t[0] + t[ACOPY];
         if (v) atomicAdd(&a.acc_out[(size_t)gy * N + gx], v);
     }
-}
-
-template <bool PREMUL>
-__device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index) {
-    __shared__ __align__(16) int acc[acell(WTILE_LARGE) * astride(WTILE_LARGE)];
-    if (a.side == WTILE_SMALL)
-        adjoint_tile<PREMUL, WTILE_SMALL>(a, item_index, acc);
-    else
-        adjoint_tile<PREMUL, WTILE_LARGE>(a, item_index, acc);
 }
 
 __global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles(AdjArgs a) {
@@ -210,7 +238,6 @@ AdjArgs make_adj_args(const pat_geometry* g, const float* y, const float* premul
     a.items = g->adj_item;
     a.acc_out = acc;
     a.tiles_x = g->adj_tiles_x;
-    a.side = g->adj_side;
     a.wtiles_x = g->adj_wtiles_x;
     a.stop = stop;
     return a;

@@ -523,28 +523,28 @@ struct AdjWork {
     std::vector<float> cost;
 };
 
-// The K^T work list of geometry d for a GPU that holds `slots` K^T CTAs at once: tiles of
-// `side` pixels, work items of at least `min_piece` candidates.
+// The K^T work list of geometry d for a GPU that holds `slots` K^T CTAs at once, with at most
+// `max_rays` segments per work item.
 static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, double slots, AdjWork& w,
-                            int side, long long min_piece, int waves = ADJ_WAVES) {
+                            int max_rays, int waves = ADJ_WAVES) {
     const int N = d.n, D = d.n_det, T = d.n_t, M = d.quad_m;
     const double hx = (d.xmax - d.xmin) / N, hy = (d.ymax - d.ymin) / N;
     const double ex = 1e-3 * hx, ey = 1e-3 * hy;
     const std::vector<float2>& det = pt.det;
     const std::vector<float2>& cs = pt.cs;
-    // K^T candidate boxes: for every side x side work tile and detector, the (k, m)
-    // polar box of the tile's tap region (points with i0 in [x0-1, x0+side-1], same in
-    // y), with one index of margin on every side; FP64 on the host
+    // K^T candidate boxes: for every WTILE x WTILE work tile and detector, the (k, m)
+    // polar box of the tile's tap region (points with i0 in [x0-1, x0+WTILE-1], same in
+    // y), with one index of margin on every WTILE; FP64 on the host
     w.tiles_x = (N + ATILE - 1) / ATILE;
     w.tiles = w.tiles_x * w.tiles_x;
-    const int tiles_x = (N + side - 1) / side, tiles = tiles_x * tiles_x;
+    const int tiles_x = (N + WTILE - 1) / WTILE, tiles = tiles_x * tiles_x;
     w.wtiles_x = tiles_x;
     w.wtiles = tiles;
     std::vector<int4> box((size_t)tiles * D);
     for (int t = 0; t < tiles; ++t) {
-        const int x0 = (t % tiles_x) * side, y0 = (t / tiles_x) * side;
-        const double rx0 = d.xmin + (x0 - 0.5) * hx - ex, rx1 = d.xmin + (x0 + side + 0.5) * hx + ex;
-        const double ry0 = d.ymin + (y0 - 0.5) * hy - ey, ry1 = d.ymin + (y0 + side + 0.5) * hy + ey;
+        const int x0 = (t % tiles_x) * WTILE, y0 = (t / tiles_x) * WTILE;
+        const double rx0 = d.xmin + (x0 - 0.5) * hx - ex, rx1 = d.xmin + (x0 + WTILE + 0.5) * hx + ex;
+        const double ry0 = d.ymin + (y0 - 0.5) * hy - ey, ry1 = d.ymin + (y0 + WTILE + 0.5) * hy + ey;
         for (int di = 0; di < D; ++di) {
             const double dx = d.det_xy_host[2 * di], dy = d.det_xy_host[2 * di + 1];
             const double cx = std::min(std::max(dx, rx0), rx1), cy = std::min(std::max(dy, ry0), ry1);
@@ -582,7 +582,7 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
 
     // K^T work list.  Every ray (detector d, angle m) of a tile's polar box is cut to the
     // radius interval where its points can have taps in the tile's window [x0 - 1, x0 +
-    // side) x [y0 - 1, y0 + side) (the window is convex, so the interval is one
+    // WTILE) x [y0 - 1, y0 + WTILE) (the window is convex, so the interval is one
     // segment).  The cut is FP64 arithmetic on the same FP32 tables the kernels read, on
     // the window widened by 1e-3 pixel, far beyond the FP32 rounding of a point's position
     // (about 1e-5 pixel); the kernel still tests every candidate exactly.  A tile's non-empty segments, concatenated, are its
@@ -597,9 +597,9 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
         std::vector<long long> tile_base(tiles + 1, 0), tile_total(tiles, 0);
         for (int t = 0; t < tiles; ++t) {
             tile_base[t] = (long long)rays.size();
-            const int x0 = (t % tiles_x) * side, y0 = (t / tiles_x) * side;
-            const double wx0 = x0 - 1.001, wx1 = x0 + side + 0.001;
-            const double wy0 = y0 - 1.001, wy1 = y0 + side + 0.001;
+            const int x0 = (t % tiles_x) * WTILE, y0 = (t / tiles_x) * WTILE;
+            const double wx0 = x0 - 1.001, wx1 = x0 + WTILE + 0.001;
+            const double wy0 = y0 - 1.001, wy1 = y0 + WTILE + 0.001;
             long long pre = 0;
             for (int di = 0; di < D; ++di) {
                 const int4 bx = box[(size_t)t * D + di];
@@ -644,10 +644,10 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
         long long total = 0;
         for (int t = 0; t < tiles; ++t) total += tile_total[t];
         w.candidates = total;
-        // pieces per tile: `waves` waves of resident CTAs (at least min_piece candidates a piece),
+        // pieces per tile: `waves` waves of resident CTAs (at least 1024 candidates a piece),
         // each piece going to the tile whose pieces are largest at that point, which
         // minimises the largest piece
-        const long long Q = std::max(1LL, std::min((long long)(waves * slots), total / min_piece));
+        const long long Q = std::max(1LL, std::min((long long)(waves * slots), total / 1024));
         std::vector<long long> n_piece(tiles, 0);
         {
             std::priority_queue<std::pair<double, int>> heap;   // (piece size, tile)
@@ -677,8 +677,8 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
                 while (rays[r + 1].w <= b0) ++r;
                 long long r_last = r;                    // segment holding b1 - 1
                 while (rays[r_last + 1].w <= b1 - 1) ++r_last;
-                while (b0 < b1) {                        // at most ARAYS segments per item
-                    const long long re = std::min(r_last, r + ARAYS - 1);
+                while (b0 < b1) {                        // at most max_rays segments per item
+                    const long long re = std::min(r_last, r + max_rays - 1);
                     const long long e1 = re == r_last ? b1 : rays[re + 1].w;
                     AdjItem it{};
                     it.tile = t;
@@ -846,10 +846,7 @@ static int install_adjoint_plan(pat_geometry* g, const PointTables& pt, int wave
     pat_geometry_desc dd = g->desc;
     dd.det_xy_host = g->det_xy.data();
     AdjWork aw;
-    // (every item zeroes and flushes a copy of its tile, so it should have candidates enough)
-    const int side = work_tile_side(dd.n, dd.n_det, dd.n_t, dd.quad_m);
-    const int rc = adjoint_worklist(dd, pt, (double)sm_count() * adjoint_blocks_per_sm(), aw, side,
-                                    side == WTILE_SMALL ? 1024 : 4096, waves);
+    const int rc = adjoint_worklist(dd, pt, (double)sm_count() * adjoint_blocks_per_sm(), aw, 1 << 30, waves);
     if (rc) return rc;
     std::vector<AdjRec> recs;
     std::vector<AdjWorkItem> items;
@@ -871,7 +868,6 @@ static int install_adjoint_plan(pat_geometry* g, const PointTables& pt, int wave
     g->adj_item = it_dev;
     g->adj_tiles_x = aw.tiles_x;
     g->adj_tiles = aw.tiles;
-    g->adj_side = side;
     g->adj_wtiles_x = aw.wtiles_x;
     g->adj_candidates = aw.candidates;
     g->adj_item_cost = aw.cost;
@@ -1037,7 +1033,7 @@ extern "C" int pat_adjoint_worklist(const pat_geometry_desc* desc, int slots, in
         s = (double)sms * adjoint_blocks_per_sm();
     }
     AdjWork aw;
-    const int rc = adjoint_worklist(*desc, point_tables(*desc), s, aw, WTILE_ABI, 1024);
+    const int rc = adjoint_worklist(*desc, point_tables(*desc), s, aw, ARAYS);
     if (rc) return rc;
     counts3_host[0] = (long long)aw.rays.size();
     counts3_host[1] = (long long)aw.items.size();

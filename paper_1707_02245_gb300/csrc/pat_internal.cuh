@@ -99,25 +99,11 @@ constexpr int FWD_MAX_CLUSTER = 16;              // largest (non-portable) clust
 constexpr int FWD_ROUND = 256;                   // row groups of a cluster per round
 constexpr int FWD_STAGE_MAX = 1024;              // slabs need the cs and det tables staged: M, D <= this
 constexpr int MAX_QUAD_M = 8192;
-constexpr int ATILE = 32;      // side of the pixel tiles that the readers of a K^T image look a scale up for
-// Sides of the pixel tiles one K^T work item accumulates (one scale each).  Large tiles have
-// longer ray segments; small ones leave less to zero and to flush per work item, which
-// counts where a work item has little to add (us per launch with small / large tiles: 64^2
-// image with 64 detectors 5.9 / 7.2, 128^2 with 64 6.9 / 7.6, 192^2 with 64 8.0 / 8.3, but
-// 128^2 with 512 24.7 / 19.9, 192^2 with 256 20.0 / 15.9, 256^2 with 256 23.6 / 19.2).
-constexpr int WTILE_LARGE = 64, WTILE_SMALL = 32;
-inline int work_tile_side(int n, int n_det, int n_t, int quad_m) {
-    return n <= 192 && (double)n_det * n_t * quad_m <= 8e6 ? WTILE_SMALL : WTILE_LARGE;
-}
-constexpr int WTILE_ABI = 32;  // tile side of the work list that pat_adjoint_worklist describes
-static_assert(WTILE_LARGE % ATILE == 0 && WTILE_SMALL % ATILE == 0, "scale tiles nest in work tiles");
-constexpr int ARAYS = 1024;    // most ray segments one K^T work item holds
-// Lanes of a warp that share one K^T ray segment, two neighbouring points each.  Fewer lanes
-// waste fewer steps on short segments, but more segments a warp put more lanes on one bank
-// (wavefronts per shared atomic at 256^2 on 64-pixel tiles: 3.3 with 8 lanes, 2.0 with 16,
-// 1.4 with 32; measured per launch: 23.6, 19.2 and 26.7 us; 32-pixel tiles: 26.5 and 23.6 us
-// with 8 and 16).
-constexpr int ALANES = 16;
+constexpr int ATILE = 32;      // side of the pixel tiles that share one K^T fixed-point scale
+constexpr int WTILE = 32;      // side of the pixel tiles one K^T work item accumulates
+static_assert(ATILE % WTILE == 0, "work tiles nest in scale tiles");
+constexpr int ARAYS = 1024;    // most ray segments a work item of the exported work list holds
+constexpr int ALANES = 8;            // lanes of a warp that share one K^T ray segment (8: 18.8 us per launch, 16: 22.3)
 constexpr int AROWS = 32 / ALANES;   // ray segments a warp walks at once
 #ifndef PAT_ADJ_WAVES
 #define PAT_ADJ_WAVES 1
@@ -179,7 +165,7 @@ struct pat_geometry {
     pat::AdjRec* adj_rec = nullptr;        // K^T ray segments of the work items
     pat::AdjWorkItem* adj_item = nullptr;  // K^T work items, one CTA each
     int adj_tiles_x = 0, adj_tiles = 0, adj_items = 0;   // scale tiles (ATILE) per row, in all; items
-    int adj_side = 0, adj_wtiles_x = 0;   // side of the work tiles, work tiles per row
+    int adj_wtiles_x = 0;              // work tiles (WTILE) per row
     long long adj_candidates = 0;     // candidate points of one K^T application
     std::vector<float> adj_item_cost;  // estimated cost per work item (host)
     int4* fwd_units = nullptr;         // K work units (see GeomView)
@@ -333,7 +319,7 @@ struct AdjArgs {       // fixed-point K^T y, one work item per block
     const AdjWorkItem* items;
     int* acc_out;            // N*N fixed-point image, added to with integer atomics
     int tiles_x;             // scale tiles per row
-    int side, wtiles_x;      // side of the work tiles, work tiles per row
+    int wtiles_x;            // work tiles per row
     const int* stop;
 };
 

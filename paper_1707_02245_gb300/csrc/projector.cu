@@ -364,15 +364,12 @@ __global__ void k_absmax(const float* __restrict__ y, long long n, unsigned* __r
     if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
 }
 
-// max of K^T 1 over the work tile that holds each ATILE tile: all the ATILE tiles of a work
-// tile get one value, so its work items accumulate with one scale
-__global__ void k_tile_kmax(const float* __restrict__ kcol, int N, int tiles_x, int side,
-                            float* __restrict__ tile_kmax) {
+__global__ void k_tile_kmax(const float* __restrict__ kcol, int N, int tiles_x, float* __restrict__ tile_kmax) {
     const int t = blockIdx.x;
-    const int x0 = (t % tiles_x) * ATILE / side * side, y0 = (t / tiles_x) * ATILE / side * side;
+    const int x0 = (t % tiles_x) * ATILE, y0 = (t / tiles_x) * ATILE;
     float m = 0.f;
-    for (int c = threadIdx.x; c < side * side; c += blockDim.x) {
-        const int gx = x0 + c % side, gy = y0 + c / side;
+    for (int c = threadIdx.x; c < ATILE * ATILE; c += blockDim.x) {
+        const int gx = x0 + c % ATILE, gy = y0 + c / ATILE;
         if (gx < N && gy < N) m = fmaxf(m, kcol[(size_t)gy * N + gx]);
     }
 #pragma unroll
@@ -567,7 +564,7 @@ int ensure_precond(const pat_geometry* gc, cudaStream_t st) {
     k_double_to_float<<<ceil_div((long long)N * N, 256), 256, 0, st>>>(tmp, g->pc.kcol, N * N);
     PAT_LAUNCH_CHECK("k_double_to_float");
     if (!g->pc.tile_kmax) PAT_CUDA(cudaMalloc(&g->pc.tile_kmax, (size_t)g->adj_tiles * sizeof(float)));
-    k_tile_kmax<<<g->adj_tiles, 256, 0, st>>>(g->pc.kcol, N, g->adj_tiles_x, g->adj_side, g->pc.tile_kmax);
+    k_tile_kmax<<<g->adj_tiles, 256, 0, st>>>(g->pc.kcol, N, g->adj_tiles_x, g->pc.tile_kmax);
     PAT_LAUNCH_CHECK("k_tile_kmax");
     PAT_CUDA(cudaFreeAsync(tmp, st));
     PAT_CUDA(cudaStreamSynchronize(st));

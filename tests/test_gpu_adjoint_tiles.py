@@ -1,8 +1,8 @@
 """K^T at the edges of its pixel tiles and ray segments, against the FP64 oracle.
 
-Tiles have a side of 32 or 64 pixels by the amount of work, a warp walks two segments in
-pairs of points, and the data rows inside a reconstruction are padded to an even length.  So:
-image sides around multiples of both tiles, odd numbers of samples (the last pair is half
+Tiles have a side of 32 pixels, a warp walks four segments in pairs of points, and the data
+rows inside a reconstruction are padded to an even length.  So: image sides around multiples
+of the tile, odd numbers of samples (the last pair is half
 padding), segments shorter and longer than a warp's step, detectors inside the image (rays
 in every direction through one tile) and a single datum.
 
@@ -34,8 +34,7 @@ def _lib():
     P.load()
 
 
-# n, detectors, radius of their circle, samples, angles: small tiles, then large ones (a side
-# above 192, or more than 8e6 points)
+# n, detectors, radius of their circle, samples, angles
 CASES = [(2, 1, 1.2, 1, 16), (31, 3, 1.2, 17, 48), (32, 5, 1.2, 33, 64), (33, 4, 0.5, 21, 200), (65, 2, 1.2, 301, 96),
          (192, 3, 1.2, 95, 64), (193, 3, 1.2, 385, 64), (200, 2, 0.4, 51, 128), (64, 140, 1.2, 255, 256),
          (96, 330, 0.9, 97, 256)]
