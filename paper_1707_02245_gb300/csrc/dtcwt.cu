@@ -273,12 +273,12 @@ __global__ void __launch_bounds__(256) k_cwt_gap_pixels(CwtGapArgs a, long long 
         double s[4] = {0, 0, 0, 0};
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
             for (int c = 0; c < 4; ++c) s[c] += sh[c][w];
-        double* o = a.partials + (size_t)a.terms * blockIdx.x;
-        for (int c = 0; c < a.terms; ++c) o[c] = 0.0;
+        double* o = a.partials + blockIdx.x;   // term c of block b at [c * blocks + b]
+        for (int c = 0; c < a.terms; ++c) o[(size_t)c * gridDim.x] = 0.0;
         o[0] = s[0];
-        o[2] = s[1];
-        o[4] = s[2];
-        o[5] = s[3];
+        o[(size_t)2 * gridDim.x] = s[1];
+        o[(size_t)4 * gridDim.x] = s[2];
+        o[(size_t)5 * gridDim.x] = s[3];
     }
 }
 

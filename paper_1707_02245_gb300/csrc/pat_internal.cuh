@@ -297,7 +297,8 @@ struct FwdArgs {
     const float* step_mul; // {tau multiplier s, sigma multiplier 1/s} (device) or NULL
     float* qw;             // rows of row_stride(T)
     unsigned* qmax_bits;
-    double* partials;      // FWD_GAP: one GAP_DATA_TERMS block of sums per K CTA
+    double* partials;      // FWD_GAP: term c of K CTA i at [c * n_part + i]
+    int n_part;            // K CTAs of the problem
     const int* stop;
 };
 
@@ -330,8 +331,12 @@ AdjArgs make_adj_args(const pat_geometry* g, const float* y, const float* premul
 // K launch over a map of (problem, CTA) pairs: cluster-major, the S ranks of a cluster
 // consecutive; every problem of one launch has the same S (cluster size).  smem: dynamic
 // shared memory of the launch (the largest plan of its problems).
+// FWD_GAP with gap and fin (per-problem arrays, or both NULL: data terms only): the CTAs also
+// sum the pixel terms, and the last one evaluates the gap.
+struct GapArgs;
+struct FinalArgs;
 int launch_forward_b(int epi, const FwdArgs* args, const int2* map, int nblocks, int cluster, int smem,
-                     cudaStream_t st);
+                     cudaStream_t st, const GapArgs* gap = nullptr, const FinalArgs* fin = nullptr);
 int forward_smem_bytes(int rows, int stride, int M, int D, bool staged);
 int forward_clusters_per_gpu(int cluster, int smem);   // K clusters the GPU holds at once
 int forward_threads(int smem);                         // threads of a K CTA with this shared memory

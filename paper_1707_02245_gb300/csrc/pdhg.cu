@@ -20,6 +20,7 @@
 #include <cstring>
 #include <vector>
 
+#include "gap.cuh"
 #include "pat_internal.cuh"
 #include "reduce.cuh"
 #include "stencil.cuh"
@@ -367,287 +368,15 @@ __global__ void k_dual_step(DualArgs a) {
     }
 }
 
-// ---------------------------------------------------------------------------------
-// FP64 duality gap over pixels (Sec. 3.3.3, box-restricted reading)
-// partials per block: {R1, R2, |K^T q - div r|_1, |E^T s - r|_1, |x - x_old|^2, |x_old|^2}
-// ---------------------------------------------------------------------------------
-constexpr int GAP_PIX_TERMS = 7;   // per-block sums of the pixel pass
-constexpr int GAP_TERMS = GAP_DATA_TERMS + GAP_PIX_TERMS;
-
-// Distance of g from the normal cone of the radius-ball at p: the cone is {0} inside the
-// ball and the ray through p on its sphere (the dual residual of a ball-constrained dual).
-__device__ __forceinline__ float cone_distance2(float g0, float g1, float p0, float p1, float radius) {
-    const float np = sqrtf(p0 * p0 + p1 * p1);
-    const float lam = np >= radius * (1.f - 1e-6f) && np > 0.f ? fmaxf(0.f, (g0 * p0 + g1 * p1) / np) : 0.f;
-    return sqrtf(fmaxf(g0 * g0 + g1 * g1 - lam * lam, 0.f));
-}
-__device__ __forceinline__ float cone_distance3(float g0, float g1, float g2, float p0, float p1, float p2,
-                                                float radius) {
-    const float np = sqrtf(p0 * p0 + p1 * p1 + p2 * p2);
-    const float lam =
-        np >= radius * (1.f - 1e-6f) && np > 0.f ? fmaxf(0.f, (g0 * p0 + g1 * p1 + g2 * p2) / np) : 0.f;
-    return sqrtf(fmaxf(g0 * g0 + g1 * g1 + g2 * g2 - lam * lam, 0.f));
-}
-
-struct GapArgs {
-    int n;
-    float alpha, ab;      // ball radii of r and s
-    double gamma;
-    const float* xi;
-    const float* x;       // x^{n+1}
-    const float* x_old;   // x^n (NULL: residual terms are zero)
-    const float* y;       // r, s at the same evaluation (y^{n+1})
-    KtView kt;            // K^T q^{n+1} (fixed point)
-    double* partials;
-    const int* stop;
-    int nblocks;          // blocks of this problem's pixel pass
-};
-
-template <int REG>
-__device__ __forceinline__ void gap_pixels_block(const GapArgs& a, const int lb) {
-    const int N = a.n;
-    const size_t NN = (size_t)N * N;
-    const float gam = (float)a.gamma;
-    const float alpha = a.alpha, ab = a.ab;
-    // per-thread terms in FP32 (each thread covers few pixels); warp sums as FP32 pairs and
-    // block sums in FP64: GB300's FP64 pipe runs at 1/64 of FP32, so FP64 is kept to one
-    // warp per block
-    // + the dual residual of the regulariser duals (distance of their argument from the
-    // normal cone of the ball at r and s), for the adaptive balance
-    float acc[GAP_PIX_TERMS] = {0, 0, 0, 0, 0, 0, 0};
-    const int nthreads = a.nblocks * blockDim.x;
-    auto X = [&](int c, int x, int y) -> float { return __ldg(a.x + c * NN + (size_t)y * N + x); };
-    auto Yf = [&](int c, int x, int y) -> float { return __ldg(a.y + c * NN + (size_t)y * N + x); };
-    // r masked for div (dTV: D_xi r), zero outside the grid
-    auto rm = [&](int c, int x, int y) -> float {
-        if (x < 0 || y < 0 || (c == 0 && x >= N - 1) || (c == 1 && y >= N - 1)) return 0.f;
-        float r0 = Yf(0, x, y), r1 = Yf(1, x, y);
-        if (REG == PAT_DTV) {
-            float o0, o1;
-            dxi_apply(__ldg(a.xi + (size_t)y * N + x), __ldg(a.xi + NN + (size_t)y * N + x), gam, r0, r1, o0, o1);
-            r0 = o0;
-            r1 = o1;
-        }
-        return c == 0 ? r0 : r1;
-    };
-    for (long long p = (long long)lb * blockDim.x + threadIdx.x; p < (long long)NN; p += nthreads) {
-        const int gx = (int)(p % N), gy = (int)(p / N);
-        const bool ax = gx < N - 1, by = gy < N - 1;
-        const float u = X(0, gx, gy);
-        float g0 = ax ? X(0, gx + 1, gy) - u : 0.f;
-        float g1 = by ? X(0, gx, gy + 1) - u : 0.f;
-        if (REG == PAT_DTV) {
-            float o0, o1;
-            dxi_apply(__ldg(a.xi + p), __ldg(a.xi + NN + p), gam, g0, g1, o0, o1);
-            g0 = o0;
-            g1 = o1;
-        }
-        if (REG == PAT_TGV) {
-            g0 -= X(1, gx, gy);
-            g1 -= X(2, gx, gy);
-        }
-        acc[0] += sqrtf(g0 * g0 + g1 * g1);
-        acc[6] += cone_distance2(g0, g1, Yf(0, gx, gy), Yf(1, gx, gy), alpha);
-        // box term of u: |K^T q - div r|; near convergence the two sides agree closely and
-        // their FP32 difference is exact (Sterbenz), so FP32 keeps the term's precision
-        const float divr = (rm(0, gx, gy) - rm(0, gx - 1, gy)) + (rm(1, gx, gy) - rm(1, gx, gy - 1));
-        const float atu = a.kt.at(gx, gy, N) - divr;
-        acc[2] += fabsf(atu);
-        if (REG == PAT_TGV) {
-            auto vm = [&](int c, int x, int y, bool mx) -> float {  // masked v for d^-
-                if (x < 0 || y < 0 || (mx ? (x >= N - 1) : (y >= N - 1))) return 0.f;
-                return X(1 + c, x, y);
-            };
-            const float e11 = vm(0, gx, gy, true) - vm(0, gx - 1, gy, true);
-            const float e22 = vm(1, gx, gy, false) - vm(1, gx, gy - 1, false);
-            const float e12 = ((vm(0, gx, gy, false) - vm(0, gx, gy - 1, false)) +
-                               (vm(1, gx, gy, true) - vm(1, gx - 1, gy, true))) * kInvSqrt2f;
-            acc[1] += sqrtf(e11 * e11 + e22 * e22 + e12 * e12);
-            const float s11 = Yf(2, gx, gy), s22 = Yf(3, gx, gy), s12 = Yf(4, gx, gy);
-            acc[6] += cone_distance3(e11, e22, e12, s11, s22, s12, ab);
-            const float dx11 = ax ? Yf(2, gx + 1, gy) - s11 : 0.f;
-            const float dy12 = by ? Yf(4, gx, gy + 1) - s12 : 0.f;
-            const float dy22 = by ? Yf(3, gx, gy + 1) - s22 : 0.f;
-            const float dx12 = ax ? Yf(4, gx + 1, gy) - s12 : 0.f;
-            const float et1 = -dx11 - dy12 * kInvSqrt2f, et2 = -dy22 - dx12 * kInvSqrt2f;
-            acc[3] += fabsf(et1 - Yf(0, gx, gy)) + fabsf(et2 - Yf(1, gx, gy));
-        }
-        if (a.x_old) {
-            const int nc = REG == PAT_TGV ? 3 : 1;
-            for (int c = 0; c < nc; ++c) {
-                const float xn = X(c, gx, gy), xo = __ldg(a.x_old + c * NN + p);
-                acc[4] += (xn - xo) * (xn - xo);
-                acc[5] += xo * xo;
-            }
-        }
-    }
-    double dacc[GAP_PIX_TERMS];
-    block_sum_pair<GAP_PIX_TERMS>(acc, dacc);
-    if (threadIdx.x == 0)
-        for (int c = 0; c < GAP_PIX_TERMS; ++c) a.partials[GAP_PIX_TERMS * lb + c] = dacc[c];
-}
-
-
-constexpr int GAP_FINAL_BLOCKS = 32;
-constexpr int GAP_FINAL_THREADS = 32;   // one warp: the final sums are FP64, kept to few lanes
-
-struct InfoDev {
-    double primal, dual, gap, rel_gap, residual;
-    int iters_done, status, stop, iter;
-    unsigned qmax_bits[2];  // max |q| of iterations of each parity (float bits)
-    unsigned final_ticket;  // blocks of k_gap_final done (the last one resets it)
-    float step_mul[2];      // {s, 1/s}: primal and dual step multipliers
-    int n_adjust;           // adaptive-balance adjustments so far
-    double level2[GAP_FINAL_BLOCKS][GAP_TERMS];
-};
-
-struct FinalArgs {
-    const double* data_part;
-    int n_data;
-    const double* pix_part;
-    int n_pix;
-    double alpha, beta, box_u, box_v, tol;
-    int reg, adapt;
-    InfoDev* info;
-    int* batch_stopped;    // problems of the batch that have stopped (the host polls it)
-};
-
-// Adaptive primal-dual balance (residual balancing after Goldstein, Li, Yuan, Esser and
-// Baraniuk 2015), in L1 norms at the evaluated state:
-//  - primal residual |A^T y|_1 (G = 0, so A^T y = 0 at a solution);
-//  - dual residual: |q - (Ku - f)|_1, plus the distance of grad u - v (dTV: D_xi grad u)
-//    and of E v from the normal cones of the r- and s-balls.
-// When one exceeds the other by more than BAL_DEAD, s (the primal step multiplier) moves
-// toward balance by the square root of their ratio, clamped to a factor BAL_MAX_STEP.  The
-// exponent decays by BAL_DECAY per adjustment, so s settles.
-constexpr double BAL_DEAD = 2.0, BAL_MAX_STEP = 2.0, BAL_DECAY = 0.97, BAL_MIN = 1e-3, BAL_MAX = 1e3;
-
-__device__ void balance_update(InfoDev* in, double primal_res, double dual_res) {
-    if (!(primal_res > 0 && dual_res > 0)) return;
-    const double rho = primal_res / dual_res;
-    if (rho >= 1.0 / BAL_DEAD && rho <= BAL_DEAD) return;
-    const double f = fmin(fmax(sqrt(rho), 1.0 / BAL_MAX_STEP), BAL_MAX_STEP);
-    double s = (double)in->step_mul[0] * pow(f, pow(BAL_DECAY, (double)in->n_adjust));
-    s = fmin(fmax(s, BAL_MIN), BAL_MAX);
-    in->step_mul[0] = (float)s;
-    in->step_mul[1] = (float)(1.0 / s);
-    in->n_adjust += 1;
-}
-
-__device__ __forceinline__ void gap_evaluate(const FinalArgs& a, const double (&t)[GAP_TERMS]);
-
-// Two-level FP64 reduction in a fixed order: each of GAP_FINAL_BLOCKS blocks sums a fixed
-// strided subset of the partials, the last block to finish adds the block sums in index
-// order and evaluates the gap, the residual and the stopping test.
-__device__ __forceinline__ void gap_final_block(const FinalArgs& a, const int lb) {
-    double acc[GAP_TERMS];
-    for (int c = 0; c < GAP_TERMS; ++c) acc[c] = 0.0;
-    const int stride = GAP_FINAL_BLOCKS * blockDim.x;
-    for (int b = lb * blockDim.x + threadIdx.x; b < a.n_data; b += stride)
-        for (int c = 0; c < GAP_DATA_TERMS; ++c) acc[c] += a.data_part[GAP_DATA_TERMS * b + c];
-    for (int b = lb * blockDim.x + threadIdx.x; b < a.n_pix; b += stride)
-        for (int c = 0; c < GAP_PIX_TERMS; ++c) acc[GAP_DATA_TERMS + c] += a.pix_part[GAP_PIX_TERMS * b + c];
-    block_sum<GAP_TERMS>(acc);
-    __shared__ bool s_last;
-    InfoDev* in = a.info;
-    if (threadIdx.x == 0) {
-        for (int c = 0; c < GAP_TERMS; ++c) in->level2[lb][c] = acc[c];
-        __threadfence();
-        s_last = atomicAdd(&in->final_ticket, 1u) == GAP_FINAL_BLOCKS - 1;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    // warp c adds the block sums of component c with a shuffle tree (fixed order)
-    __shared__ double s_tot[GAP_TERMS];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int c = warp; c < GAP_TERMS; c += blockDim.x >> 5) {
-        double v = lane < GAP_FINAL_BLOCKS ? *(volatile double*)&in->level2[lane][c] : 0.0;
-        v = warp_sum(v);
-        if (lane == 0) s_tot[c] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    in->final_ticket = 0;
-    double t[GAP_TERMS];
-    for (int c = 0; c < GAP_TERMS; ++c) t[c] = s_tot[c];
-    gap_evaluate(a, t);
-}
-
-// The gap, the residual and the stopping test from the summed terms (one thread).
-__device__ __forceinline__ void gap_evaluate(const FinalArgs& a, const double (&t)[GAP_TERMS]) {
-    InfoDev* in = a.info;
-    const double res2 = t[0], q2 = t[1], qf = t[2], dres_q = t[3];
-    const double r1 = t[4], r2 = t[5], bu = t[6], bv = t[7], dx2 = t[8], x2 = t[9], dres_rs = t[10];
-    const double reg = a.reg == PAT_TGV ? r1 + a.beta * r2 : r1;
-    const double primal = 0.5 * res2 + a.alpha * reg;
-    const double dual = -(0.5 * q2 + qf) - a.box_u * bu - (a.reg == PAT_TGV ? a.box_v * bv : 0.0);
-    const double gap = primal - dual;
-    const double rel = primal > 0 ? gap / primal : (gap == 0 ? 0.0 : INFINITY);
-    const double resid = x2 > 0 ? sqrt(dx2 / x2) : (dx2 == 0 ? 0.0 : INFINITY);
-    in->primal = primal;
-    in->dual = dual;
-    in->gap = gap;
-    in->rel_gap = rel;
-    in->residual = resid;
-    in->iters_done = in->iter;
-    if (!isfinite(gap) || !isfinite(primal)) {
-        in->status = PAT_STATUS_DIVERGED;
-        in->stop = 1;
-        if (a.batch_stopped) atomicAdd(a.batch_stopped, 1);
-    } else if (a.tol > 0 && rel <= a.tol) {
-        in->status = PAT_STATUS_CONVERGED;
-        in->stop = 1;
-        if (a.batch_stopped) atomicAdd(a.batch_stopped, 1);
-    } else if (a.adapt == PAT_ADAPT_BALANCE) {
-        balance_update(in, bu + (a.reg == PAT_TGV ? bv : 0.0), dres_q + dres_rs);
-    }
-}
-
-__global__ void __launch_bounds__(GAP_FINAL_THREADS) k_gap_final_b(const FinalArgs* __restrict__ args, const int2* __restrict__ map) {
-    const int2 pm = map[blockIdx.x];
+// The wavelet model's final sums: one block per problem.
+constexpr int GAP_FINAL_THREADS = 256;
+__global__ void __launch_bounds__(GAP_FINAL_THREADS) k_gap_final_b(const FinalArgs* __restrict__ args) {
     __shared__ FinalArgs sa;
-    const FinalArgs& a = stage_args(args, pm.x, sa);
+    __shared__ double s_tot[GAP_TERMS];
+    const FinalArgs& a = stage_args(args, blockIdx.x, sa);
     if (*(volatile const int*)&a.info->stop) return;
-    gap_final_block(a, pm.y);
-}
-
-// The gap's pixel pass with the final reduction in its last block: every block writes its
-// partial sums; the last of a problem's blocks to finish (a ticket) adds all the problem's
-// data and pixel partials in FP64 in a fixed order (thread t takes rows t, t + 256, ...,
-// then a fixed shuffle and warp tree) and evaluates the gap and the stopping test.
-template <int REG>
-__global__ void __launch_bounds__(256) k_gap_pixels_final_b(const GapArgs* __restrict__ args,
-                                                            const FinalArgs* __restrict__ fin,
-                                                            const int2* __restrict__ map) {
-    const int2 pm = map[blockIdx.x];
-    __shared__ GapArgs sa;
-    const GapArgs& a = stage_args(args, pm.x, sa);
-    if (a.stop && *(volatile const int*)a.stop) return;
-    gap_pixels_block<REG>(a, pm.y);
-    __shared__ bool s_last;
-    InfoDev* in = fin[pm.x].info;
-    if (threadIdx.x == 0) {
-        __threadfence();   // this block's partials before its ticket
-        s_last = atomicAdd(&in->final_ticket, 1u) == (unsigned)(a.nblocks - 1);
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    const FinalArgs f = fin[pm.x];
-    double acc[GAP_TERMS];
-#pragma unroll
-    for (int c = 0; c < GAP_TERMS; ++c) acc[c] = 0.0;
-    for (int b = threadIdx.x; b < f.n_data; b += blockDim.x)
-#pragma unroll
-        for (int c = 0; c < GAP_DATA_TERMS; ++c) acc[c] += __ldcg(f.data_part + GAP_DATA_TERMS * b + c);
-    for (int b = threadIdx.x; b < f.n_pix; b += blockDim.x)
-#pragma unroll
-        for (int c = 0; c < GAP_PIX_TERMS; ++c) acc[GAP_DATA_TERMS + c] += __ldcg(f.pix_part + GAP_PIX_TERMS * b + c);
-    block_sum<GAP_TERMS>(acc);
-    if (threadIdx.x != 0) return;
-    in->final_ticket = 0;
-    gap_evaluate(f, acc);
+    gap_sum_terms(a, s_tot);
+    gap_evaluate(a, s_tot);
 }
 
 // ---------------------------------------------------------------------------------
@@ -816,9 +545,9 @@ struct Workspace {
     float *q = nullptr, *ubar = nullptr, *vbar0 = nullptr;
     int* kt[2] = {nullptr, nullptr};   // fixed-point K^T q, by iteration parity
     float *tau_u = nullptr, *sig_q = nullptr, *sig_r = nullptr, *qw = nullptr;
-    double *data_part = nullptr, *pix_part = nullptr;
+    double* part = nullptr;   // the gap's partial sums
     InfoDev* info = nullptr;
-    int n_data = 0, n_pix = 0;
+    int n_data = 0;
 };
 
 static int pix_blocks(int N) { return std::min(4 * sm_count(), ceil_div((long long)N * N, 256)); }
@@ -826,15 +555,14 @@ static int pix_blocks(int N) { return std::min(4 * sm_count(), ceil_div((long lo
 static int alloc_workspace(const pat_geometry* g, int reg, Workspace& ws, cudaStream_t st) {
     const size_t N = g->desc.n, NN = N * N, S = (size_t)g->desc.n_det * g->desc.n_t;
     const size_t nx = NN * (reg == PAT_TGV ? 3 : 1), ny = NN * (reg == PAT_TGV ? 5 : 2);
-    ws.n_data = g->fwd_n_ctas;   // one block of data-term sums per K CTA
-    ws.n_pix = pix_blocks((int)N);
-    size_t off[17];
-    size_t sz[17] = {nx * 4, nx * 4, ny * 4, ny * 4, S * 4, NN * 4, NN * 4 * 2,
+    ws.n_data = g->fwd_n_ctas;   // one set of gap sums per K CTA
+    size_t off[16];
+    size_t sz[16] = {nx * 4, nx * 4, ny * 4, ny * 4, S * 4, NN * 4, NN * 4 * 2,
                      (reg == PAT_TGV ? 2 * NN : 1) * 4,
-                     NN * 4, S * 4, NN * 4, (size_t)ws.n_data * GAP_DATA_TERMS * 8, (size_t)ws.n_pix * GAP_PIX_TERMS * 8, sizeof(InfoDev),
+                     NN * 4, S * 4, NN * 4, (size_t)ws.n_data * GAP_TERMS * 8, sizeof(InfoDev),
                      (size_t)g->desc.n_det * row_stride(g->desc.n_t) * 4, nx * 2, nx * 2};
     size_t total = 0;
-    for (int i = 0; i < 17; ++i) {
+    for (int i = 0; i < 16; ++i) {
         off[i] = total;
         total += align_up(sz[i]);
     }
@@ -853,12 +581,11 @@ static int alloc_workspace(const pat_geometry* g, int reg, Workspace& ws, cudaSt
     ws.tau_u = (float*)(b + off[8]);
     ws.sig_q = (float*)(b + off[9]);
     ws.sig_r = (float*)(b + off[10]);
-    ws.data_part = (double*)(b + off[11]);
-    ws.pix_part = (double*)(b + off[12]);
-    ws.info = (InfoDev*)(b + off[13]);
-    ws.qw = (float*)(b + off[14]);
-    ws.XL[0] = (unsigned short*)(b + off[15]);
-    ws.XL[1] = (unsigned short*)(b + off[16]);
+    ws.part = (double*)(b + off[11]);
+    ws.info = (InfoDev*)(b + off[12]);
+    ws.qw = (float*)(b + off[13]);
+    ws.XL[0] = (unsigned short*)(b + off[14]);
+    ws.XL[1] = (unsigned short*)(b + off[15]);
     return PAT_OK;
 }
 
@@ -966,8 +693,6 @@ struct FwdGroup {
 struct GapPlan {
     FwdGroup fwd[FWD_MAX_CLUSTER];
     int n_fwd_groups = 0;
-    size_t map_pix[3] = {0, 0, 0};
-    int n_pix[3] = {0, 0, 0};
 };
 
 // The K launch groups of a batch.  In each, clusters run longest first: their work differs
@@ -1000,24 +725,14 @@ static void forward_groups(const Prob* pr, int B, Arena& ar, GapPlan& gp) {
     }
 }
 
-static int launch_forward_groups(int epi, const FwdArgs* args, const GapPlan& gp, const char* base, cudaStream_t st) {
+static int launch_forward_groups(int epi, const FwdArgs* args, const GapPlan& gp, const char* base, cudaStream_t st,
+                                 const GapArgs* gap = nullptr, const FinalArgs* fin = nullptr) {
     for (int i = 0; i < gp.n_fwd_groups; ++i) {
         const FwdGroup& grp = gp.fwd[i];
-        const int rc = launch_forward_b(epi, args, (const int2*)(base + grp.map), grp.n, grp.cluster, grp.smem, st);
+        const int rc = launch_forward_b(epi, args, (const int2*)(base + grp.map), grp.n, grp.cluster, grp.smem, st, gap, fin);
         if (rc) return rc;
     }
     return PAT_OK;
-}
-
-static void build_gap_plan(const Prob* pr, int B, Arena& ar, GapPlan& gp) {
-    std::vector<int2> pix[3];
-    for (int b = 0; b < B; ++b)
-        for (int i = 0; i < pr[b].ws.n_pix; ++i) pix[pr[b].p.reg].push_back(make_int2(b, i));
-    forward_groups(pr, B, ar, gp);
-    for (int r = 0; r < 3; ++r) {
-        gp.map_pix[r] = ar.put(pix[r].data(), pix[r].size());
-        gp.n_pix[r] = (int)pix[r].size();
-    }
 }
 
 static GapArgs make_gap_args(const Prob& pr, const KtView& kt, const float* x, const float* x_old, const float* y_rs) {
@@ -1031,14 +746,12 @@ static GapArgs make_gap_args(const Prob& pr, const KtView& kt, const float* x, c
     ga.x_old = x_old;
     ga.y = y_rs;
     ga.kt = kt;
-    ga.partials = pr.ws.pix_part;
-    ga.stop = &pr.ws.info->stop;
-    ga.nblocks = pr.ws.n_pix;
+    ga.reg = pr.p.reg;
     return ga;
 }
 
 static FinalArgs make_final_args(const Prob& pr, int* batch_stopped = nullptr) {
-    FinalArgs fa{pr.ws.data_part, pr.ws.n_data, pr.ws.pix_part, pr.ws.n_pix, pr.p.alpha, pr.p.beta, pr.p.box_u,
+    FinalArgs fa{pr.ws.part, pr.ws.n_data, pr.ws.part + (size_t)pr.ws.n_data * GAP_DATA_TERMS, pr.ws.n_data, pr.p.alpha, pr.p.beta, pr.p.box_u,
                  pr.p.box_v, pr.p.tol, pr.p.reg, pr.p.adapt, pr.ws.info, batch_stopped};
     return fa;
 }
@@ -1104,19 +817,8 @@ static int launch_update_b(int reg, int tile, const UpdateArgs* args, const int2
 static int launch_gap_phase(const FwdArgs* fa, const GapArgs* ga, const FinalArgs* fi, const GapPlan& gp,
                             const char* base, cudaStream_t st) {
     prof_mark(PAT_PHASE_GAP, st, true);
-    int rc = launch_forward_groups(FWD_GAP, fa, gp, base, st);
+    const int rc = launch_forward_groups(FWD_GAP, fa, gp, base, st, ga, fi);
     if (rc) return rc;
-    for (int r = 0; r < 3; ++r) {
-        if (!gp.n_pix[r]) continue;
-        const int2* map = (const int2*)(base + gp.map_pix[r]);
-        if (r == PAT_TV)
-            k_gap_pixels_final_b<PAT_TV><<<gp.n_pix[r], 256, 0, st>>>(ga, fi, map);
-        else if (r == PAT_TGV)
-            k_gap_pixels_final_b<PAT_TGV><<<gp.n_pix[r], 256, 0, st>>>(ga, fi, map);
-        else
-            k_gap_pixels_final_b<PAT_DTV><<<gp.n_pix[r], 256, 0, st>>>(ga, fi, map);
-        PAT_LAUNCH_CHECK("k_gap_pixels_final_b");
-    }
     prof_mark(PAT_PHASE_GAP, st, false);
     return PAT_OK;
 }
@@ -1157,7 +859,8 @@ static void build_iter_plan(const Prob* pr, int B, Arena& ar, IterPlan& ip, int*
             FwdArgs ga = make_fwd_args(q.g, ws.X[1 - par]);
             ga.q = ws.q;
             ga.f = q.f;
-            ga.partials = ws.data_part;
+            ga.partials = ws.part;
+            ga.n_part = ws.n_data;
             ga.stop = &ws.info->stop;
             fg.push_back(ga);
             gpx.push_back(make_gap_args(q, kt_view(q.g, ws.kt[par], &ws.info->qmax_bits[par]), ws.X[1 - par],
@@ -1196,7 +899,7 @@ static void build_iter_plan(const Prob* pr, int B, Arena& ar, IterPlan& ip, int*
             ip.map_upd[r][t] = ar.put(upd[r][t].data(), upd[r][t].size());
             ip.n_upd[r][t] = (int)upd[r][t].size();
         }
-    build_gap_plan(pr, B, ar, ip.gp);
+    forward_groups(pr, B, ar, ip.gp);
 }
 
 static int enqueue_iteration(const IterPlan& ip, const char* base, int it, bool gap_due, cudaStream_t st) {
@@ -1585,7 +1288,7 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
     // device argument blocks: K and K^T per problem, as the batch engine's
     std::vector<char> host;
     Arena ar(host);
-    size_t fw_off[2] = {0, 0}, ad_off[2] = {0, 0}, fg_off = 0, fi_off = 0, amap_off = 0, finmap_off = 0;
+    size_t fw_off[2] = {0, 0}, ad_off[2] = {0, 0}, fg_off = 0, fi_off = 0, amap_off = 0;
     GapPlan gp;
     int n_adj = 0;
     if (!rc) {
@@ -1614,6 +1317,7 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
             ga.q = F(b, Q);
             ga.f = f[b];
             ga.partials = (double*)buf(b, DPART);
+            ga.n_part = g[b]->fwd_n_ctas;
             ga.stop = &in->stop;
             fg.push_back(ga);
             fi.push_back(FinalArgs{(double*)buf(b, DPART), g[b]->fwd_n_ctas, (double*)buf(b, PPART), n_pix, p[b].alpha,
@@ -1630,13 +1334,10 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
         forward_groups(prs.data(), B, ar, gp);
         std::stable_sort(order.begin(), order.end(),
                          [](const std::pair<float, int2>& x, const std::pair<float, int2>& y) { return x.first > y.first; });
-        std::vector<int2> am, fin;
+        std::vector<int2> am;
         for (auto& e : order) am.push_back(e.second);
         n_adj = (int)am.size();
-        for (int b = 0; b < B; ++b)
-            for (int i = 0; i < GAP_FINAL_BLOCKS; ++i) fin.push_back(make_int2(b, i));
         amap_off = ar.put(am.data(), am.size());
-        finmap_off = ar.put(fin.data(), fin.size());
         rc = ar.upload(&dev, st);
     }
     const char* base = (const char*)dev;
@@ -1693,8 +1394,7 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
                 if (!e) e = launch_wav_gap_pixels(wg, n_pix, s, B, ps);
             }
             if (!e) {
-                k_gap_final_b<<<B * GAP_FINAL_BLOCKS, GAP_FINAL_THREADS, 0, s>>>((const FinalArgs*)(base + fi_off),
-                                                                                (const int2*)(base + finmap_off));
+                k_gap_final_b<<<B, GAP_FINAL_THREADS, 0, s>>>((const FinalArgs*)(base + fi_off));
                 count_launch();
                 if (cudaGetLastError() != cudaSuccess) e = fail(PAT_ERR_CUDA, "k_gap_final_b");
             }
@@ -2620,7 +2320,7 @@ static int gap_impl(const pat_geometry* g, const float* f, const pat_params* p, 
         // one problem, one gap evaluation of (x, y): K^T q then the three gap passes
         GapPlan gp;
         Arena ar(host);
-        build_gap_plan(&pr, 1, ar, gp);
+        forward_groups(&pr, 1, ar, gp);
         AdjArgs aa = make_adj_args(g, y, nullptr, &pr.ws.info->qmax_bits[0], pr.ws.kt[0], nullptr);
         const size_t adj_off = ar.put(&aa, 1);
         std::vector<int2> amap(g->adj_items);
@@ -2629,7 +2329,8 @@ static int gap_impl(const pat_geometry* g, const float* f, const pat_params* p, 
         FwdArgs fa = make_fwd_args(g, x);
         fa.q = const_cast<float*>(y);   // read only by the gap epilogue
         fa.f = f;
-        fa.partials = pr.ws.data_part;
+        fa.partials = pr.ws.part;
+        fa.n_part = pr.ws.n_data;
         const size_t fa_off = ar.put(&fa, 1);
         GapArgs ga = make_gap_args(pr, kt_view(g, pr.ws.kt[0], &pr.ws.info->qmax_bits[0]), x, nullptr, y + S);
         const size_t ga_off = ar.put(&ga, 1);

@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "gap.cuh"
 #include "pat_internal.cuh"
 #include "reduce.cuh"
 
@@ -245,12 +246,41 @@ __device__ __forceinline__ void forward_units(const FwdArgs& a, int ub, int ue, 
     }
 }
 
+// Shared memory of the gap epilogue (over the units, once the rounds are done).
+struct GapShared {
+    FinalArgs fin;
+    double tot[GAP_TERMS];
+    bool last;
+};
+
+// The gap's pixel terms of pixels first, first + step, ... into t[GAP_DATA_TERMS..].  K's CTAs
+// take the pixels between them while their slabs are on the way, and the last CTA of the
+// problem adds up: one launch per gap evaluation.  With a pixel kernel of its own after K, an
+// evaluation took 30.0 us at 64^2 (64 detectors) and 47.0 us at 256^2 (256), now 17.4 and
+// 31.5, and 177 instead of 244 us for an uneven batch of 8.  What is left beside K is latency:
+// the ticket, the loads of the partial sums and the FP64 pipe of one SM.
+__device__ __forceinline__ void gap_pixel_share(const GapArgs& g, int first, int step, float (&t)[GAP_TERMS]) {
+    float acc[GAP_PIX_TERMS];
+#pragma unroll
+    for (int c = 0; c < GAP_PIX_TERMS; ++c) acc[c] = 0.f;
+    if (g.reg == PAT_TGV)
+        gap_pixels<PAT_TGV>(g, first, step, acc);
+    else if (g.reg == PAT_TV)
+        gap_pixels<PAT_TV>(g, first, step, acc);
+    else
+        gap_pixels<PAT_DTV>(g, first, step, acc);
+#pragma unroll
+    for (int c = 0; c < GAP_PIX_TERMS; ++c) t[GAP_DATA_TERMS + c] = acc[c];
+}
+
 // K (Sec. 3.3.1, eq. (K_def)) for the row groups of one cluster, then the epilogue on
 // their rows.  The S partial sums of a row (one per slab) are added in rank (slab) order,
 // so the result does not depend on scheduling.
 template <int EPI, int NT>
 __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdArgs* __restrict__ args,
-                                                           const int2* __restrict__ map) {
+                                                           const int2* __restrict__ map,
+                                                           const GapArgs* __restrict__ gap,
+                                                           const FinalArgs* __restrict__ fin) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ FwdArgs sa;
     __shared__ int s_next;
@@ -283,7 +313,13 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdA
     const int lane = threadIdx.x & 31;
     const float smul = (EPI == FWD_PROX && a.step_mul) ? __ldg(a.step_mul + 1) : 1.f;
     unsigned qbits = 0u;
-    float t[GAP_DATA_TERMS] = {0.f, 0.f, 0.f, 0.f};
+    float t[GAP_TERMS];
+#pragma unroll
+    for (int c = 0; c < GAP_TERMS; ++c) t[c] = 0.f;
+    if constexpr (EPI == FWD_GAP) {
+        // this CTA's share of the pixel terms, while the slab is on its way
+        if (gap) gap_pixel_share(gap[pm.x], pm.y * NT + (int)threadIdx.x, a.n_part * NT, t);
+    }
     const int n_rounds = (n_rg + FWD_ROUND - 1) / FWD_ROUND;
     for (int rd = 0; rd < n_rounds; ++rd) {
         const int ub = __ldg(&roff[rd]), ue = __ldg(&roff[rd + 1]);
@@ -346,11 +382,29 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdA
         __syncthreads();
         if (threadIdx.x == 0 && s_qmax) atomicMax(a.qmax_bits, s_qmax);
     }
-    if (EPI == FWD_GAP) {
-        double sum[GAP_DATA_TERMS];
-        block_sum_pair<GAP_DATA_TERMS>(t, sum);
-        if (threadIdx.x == 0)
-            for (int c = 0; c < GAP_DATA_TERMS; ++c) a.partials[(size_t)GAP_DATA_TERMS * pm.y + c] = sum[c];
+    if constexpr (EPI == FWD_GAP) {
+        // (the rounds are over: their accumulators and units are free)
+        static_assert(sizeof(double) * 32 * GAP_TERMS <= sizeof(float) * FWD_ROUND * KGRP, "sums fit the accumulators");
+        static_assert(sizeof(GapShared) <= 16 * FWD_ROUND, "fits the units");
+        GapShared& s_gap = *reinterpret_cast<GapShared*>(s_units);
+        if (gap) stage_args(fin, pm.x, s_gap.fin);
+        const double sum = block_sums_pair<GAP_TERMS>(t, reinterpret_cast<double(*)[32]>(s_acc));
+        const int terms = gap ? GAP_TERMS : GAP_DATA_TERMS;
+        if (threadIdx.x < 2 * terms && (lane & 1) == 0) a.partials[(size_t)(lane / 2) * a.n_part + pm.y] = sum;
+        if (!gap) return;
+        // the last of the problem's CTAs adds all partial sums and evaluates the gap
+        const FinalArgs& f = s_gap.fin;
+        if (threadIdx.x < 32) __threadfence();   // this CTA's partials before its ticket
+        __syncwarp();
+        if (threadIdx.x == 0) {
+            s_gap.last = atomicAdd(&f.info->final_ticket, 1u) == (unsigned)(a.n_part - 1);
+        }
+        __syncthreads();
+        if (!s_gap.last) return;
+        __threadfence();
+        if (threadIdx.x == 0) f.info->final_ticket = 0;
+        gap_sum_terms(f, s_gap.tot);
+        gap_evaluate(f, s_gap.tot);
     }
 }
 
@@ -497,22 +551,23 @@ int forward_clusters_per_gpu(int cluster, int smem) {
 }
 
 template <int NT>
-static cudaError_t launch_forward_nt(int epi, const cudaLaunchConfig_t& cfg, const FwdArgs* args, const int2* map) {
-    if (epi == FWD_Y) return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_Y, NT>, args, map);
-    if (epi == FWD_PROX) return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_PROX, NT>, args, map);
-    return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_GAP, NT>, args, map);
+static cudaError_t launch_forward_nt(int epi, const cudaLaunchConfig_t& cfg, const FwdArgs* args, const int2* map,
+                                     const GapArgs* gap, const FinalArgs* fin) {
+    if (epi == FWD_Y) return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_Y, NT>, args, map, gap, fin);
+    if (epi == FWD_PROX) return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_PROX, NT>, args, map, gap, fin);
+    return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_GAP, NT>, args, map, gap, fin);
 }
 
 int launch_forward_b(int epi, const FwdArgs* args, const int2* map, int nblocks, int cluster, int smem,
-                     cudaStream_t st) {
+                     cudaStream_t st, const GapArgs* gap, const FinalArgs* fin) {
     if (nblocks <= 0) return PAT_OK;
     const int arc = forward_attributes();
     if (arc) return arc;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = forward_config(nblocks, cluster, smem, st, attr);
     if (epi == FWD_PROX) prof_mark(PAT_PHASE_FORWARD_PROX, st, true);
-    const cudaError_t e = forward_threads(smem) == FWD_THREADS_WIDE ? launch_forward_nt<FWD_THREADS_WIDE>(epi, cfg, args, map)
-                                                                    : launch_forward_nt<FWD_THREADS>(epi, cfg, args, map);
+    const cudaError_t e = forward_threads(smem) == FWD_THREADS_WIDE ? launch_forward_nt<FWD_THREADS_WIDE>(epi, cfg, args, map, gap, fin)
+                                                                    : launch_forward_nt<FWD_THREADS>(epi, cfg, args, map, gap, fin);
     count_launch();
     if (e != cudaSuccess) return cuda_fail(e, "k_forward_b");
     if (epi == FWD_PROX) prof_mark(PAT_PHASE_FORWARD_PROX, st, false);
