@@ -132,21 +132,23 @@ __device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ __align__(16) int acc[ACELL * ASTRIDE];
     for (int c = tid; c < ACELL * ASTRIDE / 4; c += ATHREADS) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
-    // the scale of the ATILE tile that holds this work tile
-    const float bound = __uint_as_float(*a.ymax_bits) * __ldg(&a.tile_kmax[(y0 / ATILE) * a.tiles_x + x0 / ATILE]);
-    const float scale = 1073741824.0f / bound;  // 2^30 / bound
-    const float* __restrict__ y = a.y;
-    const float4* __restrict__ recs = reinterpret_cast<const float4*>(a.recs + item.y);
-    const AdjConst ac{make_float2(a.g.dr_f, a.g.dr_f), make_float2(a.g.rh_f, a.g.rh_f), make_float2(scale, scale), a.g.wk, a.g.n_t};
     constexpr int STEP = ATHREADS / ALANES;      // segments the CTA walks at once
     const int sub2 = 2 * (lane % ALANES);
     int first = warp * AROWS, j = first + lane / ALANES;
-    const bool run = bound > 0.f && isfinite(bound);
+    const float4* __restrict__ recs = reinterpret_cast<const float4*>(a.recs + item.y);
     float4 q = make_float4(0.f, 0.f, 0.f, 0.f), s = q;
-    if (run && j < nrec) {
+    if (j < nrec) {
         q = __ldg(recs + 2 * j);
         s = __ldg(recs + 2 * j + 1);
     }
+    await_predecessor();
+    if (a.stop && *(volatile const int*)a.stop) return;
+    // the scale of the ATILE tile that holds this work tile
+    const float bound = __uint_as_float(*after_wait(a.ymax_bits)) * __ldg(&a.tile_kmax[(y0 / ATILE) * a.tiles_x + x0 / ATILE]);
+    const float scale = 1073741824.0f / bound;  // 2^30 / bound
+    const float* __restrict__ y = after_wait(a.y);
+    const AdjConst ac{make_float2(a.g.dr_f, a.g.dr_f), make_float2(a.g.rh_f, a.g.rh_f), make_float2(scale, scale), a.g.wk, a.g.n_t};
+    const bool run = bound > 0.f && isfinite(bound);
     __syncthreads();
     if (run) {
         int* cells = acc + (lane / ALANES % 2) * ACOPY;
@@ -175,6 +177,7 @@ __device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index) {
         }
     }
     __syncthreads();
+    dependents_may_start();
     // the accumulators with x along a row += those with y along a row, along diagonals: a
     // warp's cells lie in 32 different columns of each
     for (int c = tid; c < WTILE * WTILE; c += ATHREADS) {
@@ -204,7 +207,6 @@ __global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles_b(co
                                                             const int2* __restrict__ map) {
     const int2 pm = map[blockIdx.x];
     const AdjArgs& a = args[pm.x];   // (a shared copy would be reloaded after every shared atomic)
-    if (a.stop && *(volatile const int*)a.stop) return;
     adjoint_item<PREMUL>(a, pm.y);
 }
 
@@ -255,10 +257,17 @@ int adjoint_blocks_per_sm() {
 int launch_adjoint_b(const AdjArgs* args, const int2* map, int nblocks, bool premul, cudaStream_t st) {
     if (nblocks <= 0) return PAT_OK;
     prof_mark(PAT_PHASE_ADJOINT, st, true);
-    if (premul)
-        k_adjoint_tiles_b<true><<<nblocks, ATHREADS, 0, st>>>(args, map);
-    else
-        k_adjoint_tiles_b<false><<<nblocks, ATHREADS, 0, st>>>(args, map);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nblocks);
+    cfg.blockDim = dim3(ATHREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    set_dependent_launch(attr[0]);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = premul ? cudaLaunchKernelEx(&cfg, k_adjoint_tiles_b<true>, args, map)
+                                 : cudaLaunchKernelEx(&cfg, k_adjoint_tiles_b<false>, args, map);
+    if (e != cudaSuccess) return cuda_fail(e, "k_adjoint_tiles_b");
     PAT_LAUNCH_CHECK("k_adjoint_tiles_b");
     prof_mark(PAT_PHASE_ADJOINT, st, false);
     return PAT_OK;

@@ -54,6 +54,7 @@ struct UpdateArgs {
     const int* stop;
     int* iter;             // iteration counter (incremented once per launch)
     int tiles_x;           // tiles per row of the grid
+    int early;             // the next launch may start before this one ends
 };
 
 __device__ __forceinline__ float ld_img(const float* __restrict__ p, int N, int gx, int gy) {
@@ -231,6 +232,8 @@ __device__ __forceinline__ void update_tile(const UpdateArgs& a, const int bx, c
     }
     __syncthreads();
 
+    if (a.early) dependents_may_start();
+
     // ---- stage 3: dual step of the next iteration on the tile, and the writes --------
     const int lx = threadIdx.x + 1, ly = threadIdx.y + 1;
     const int gx = x0 + threadIdx.x, gy = y0 + threadIdx.y;
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(upd_tx(TILE) * upd_ty(TILE)) k_update_b(const 
     // 6.08 -> 5.58 us per launch at 256^2 against reading them from global memory)
     __shared__ UpdateArgs sa;
     const UpdateArgs& a = stage_args(args, pm.x, sa);
+    await_predecessor();
     if (a.stop && *(volatile const int*)a.stop) return;
     update_tile<REG, upd_tx(TILE), upd_ty(TILE)>(a, pm.y % a.tiles_x, pm.y / a.tiles_x, pm.y == 0);
 }
@@ -786,29 +790,34 @@ static UpdateArgs make_update_args(const Prob& pr, int par, bool gap_iter) {
     a.stop = &ws.info->stop;
     a.iter = &ws.info->iter;
     a.tiles_x = ceil_div(N, upd_tx(pr.g->shapes.update_tile));
+    // (before a K that runs as clusters the next launch starts only when this one has left the
+    // SMs: clusters placed among its CTAs needed a second wave, 56 against 50 us per iteration)
+    a.early = pr.g->view.n_slabs == 1;
     return a;
 }
 
 template <int TILE>
-static void launch_update_tile(int reg, const UpdateArgs* args, const int2* map, int n, cudaStream_t st) {
-    const dim3 blk(upd_tx(TILE), upd_ty(TILE));
-    if (reg == PAT_TV)
-        k_update_b<PAT_TV, TILE><<<n, blk, 0, st>>>(args, map);
-    else if (reg == PAT_TGV)
-        k_update_b<PAT_TGV, TILE><<<n, blk, 0, st>>>(args, map);
-    else
-        k_update_b<PAT_DTV, TILE><<<n, blk, 0, st>>>(args, map);
+static cudaError_t launch_update_tile(int reg, const UpdateArgs* args, const int2* map, int n, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)n);
+    cfg.blockDim = dim3(upd_tx(TILE), upd_ty(TILE));
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    set_dependent_launch(attr[0]);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (reg == PAT_TV) return cudaLaunchKernelEx(&cfg, k_update_b<PAT_TV, TILE>, args, map);
+    if (reg == PAT_TGV) return cudaLaunchKernelEx(&cfg, k_update_b<PAT_TGV, TILE>, args, map);
+    return cudaLaunchKernelEx(&cfg, k_update_b<PAT_DTV, TILE>, args, map);
 }
 
 static int launch_update_b(int reg, int tile, const UpdateArgs* args, const int2* map, int n, cudaStream_t st) {
     if (n <= 0) return PAT_OK;
     prof_mark(PAT_PHASE_UPDATE, st, true);
-    if (tile == PAT_UPD_64X4)
-        launch_update_tile<PAT_UPD_64X4>(reg, args, map, n, st);
-    else if (tile == PAT_UPD_32X8)
-        launch_update_tile<PAT_UPD_32X8>(reg, args, map, n, st);
-    else
-        launch_update_tile<PAT_UPD_32X4>(reg, args, map, n, st);
+    const cudaError_t e = tile == PAT_UPD_64X4   ? launch_update_tile<PAT_UPD_64X4>(reg, args, map, n, st)
+                          : tile == PAT_UPD_32X8 ? launch_update_tile<PAT_UPD_32X8>(reg, args, map, n, st)
+                                                 : launch_update_tile<PAT_UPD_32X4>(reg, args, map, n, st);
+    if (e != cudaSuccess) return cuda_fail(e, "k_update_b");
     PAT_LAUNCH_CHECK("k_update_b");
     prof_mark(PAT_PHASE_UPDATE, st, false);
     return PAT_OK;

@@ -287,9 +287,6 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdA
     __shared__ unsigned s_qmax;
     const int2 pm = map[blockIdx.x];
     const FwdArgs& a = stage_args(args, pm.x, sa);
-    // (every CTA of a cluster reads the same flag, so a stopped problem's clusters leave
-    // together, before any cluster barrier)
-    if (a.stop && *(volatile const int*)a.stop) return;
     const GeomView& g = a.g;
     const int N = g.n, T = g.n_t, S = g.n_slabs, M = g.quad_m, D = g.n_det;
     const unsigned rank = S > 1 ? cluster_rank() : 0u;
@@ -307,8 +304,14 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdA
         float2* s_det = reinterpret_cast<float2*>(smem + L.det);
         for (int i = threadIdx.x; i < 2 * M; i += NT) s_cs[i] = __ldg(&g.cs[i < M ? i : i - M]);
         for (int i = threadIdx.x; i < D; i += NT) s_det[i] = __ldg(&g.det[i]);
-        stage_slab<NT>(a.img, N, g.slab_stride, jlo, reff + 1, reinterpret_cast<float*>(smem + L.slab));
     }
+    await_predecessor();
+    gap = after_wait(gap);
+    // (every CTA of a cluster reads the same flag, so a stopped problem's clusters leave
+    // together, before any cluster barrier)
+    if (a.stop && *(volatile const int*)a.stop) return;
+    if (smem_img)
+        stage_slab<NT>(a.img, N, g.slab_stride, jlo, reff + 1, reinterpret_cast<float*>(smem + L.slab));
     if (threadIdx.x == 0) s_qmax = 0u;
     const int lane = threadIdx.x & 31;
     const float smul = (EPI == FWD_PROX && a.step_mul) ? __ldg(a.step_mul + 1) : 1.f;
@@ -375,6 +378,7 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdA
         // while another still reads its accumulators
         if (S > 1) cluster_sync(); else __syncthreads();
     }
+    dependents_may_start();
     if (EPI == FWD_PROX) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) qbits = max(qbits, __shfl_xor_sync(0xffffffffu, qbits, o));
@@ -532,14 +536,15 @@ static cudaLaunchConfig_t forward_config(int nblocks, int cluster, int smem, cud
     attr[0].val.clusterDim.x = (unsigned)cluster;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    set_dependent_launch(attr[1]);
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     return cfg;
 }
 
 int forward_clusters_per_gpu(int cluster, int smem) {
     int n = 0;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = forward_config(cluster, cluster, smem, nullptr, attr);
     const void* k = forward_threads(smem) == FWD_THREADS_WIDE ? (const void*)k_forward_b<FWD_PROX, FWD_THREADS_WIDE>
                                                               : (const void*)k_forward_b<FWD_PROX, FWD_THREADS>;
@@ -563,7 +568,7 @@ int launch_forward_b(int epi, const FwdArgs* args, const int2* map, int nblocks,
     if (nblocks <= 0) return PAT_OK;
     const int arc = forward_attributes();
     if (arc) return arc;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = forward_config(nblocks, cluster, smem, st, attr);
     if (epi == FWD_PROX) prof_mark(PAT_PHASE_FORWARD_PROX, st, true);
     const cudaError_t e = forward_threads(smem) == FWD_THREADS_WIDE ? launch_forward_nt<FWD_THREADS_WIDE>(epi, cfg, args, map, gap, fin)
