@@ -1,6 +1,7 @@
 // Exact transpose K^T of the circular-mean projector (Sec. 3.3.1, Sec. 4.2 eq. (K_def)) by
 // pixel tiles with fixed-point accumulation, and the K^T entry points.
 #include <algorithm>
+#include <initializer_list>
 
 #include "pat_internal.cuh"
 
@@ -123,8 +124,23 @@ __device__ __forceinline__ void adjoint_segment(const AdjConst& a, const float4 
     }
 }
 
+// Maximum of n <= ATHREADS words, in every thread of the CTA.
+__device__ __forceinline__ unsigned max_of_slots(const unsigned* slots, int n) {
+    __shared__ unsigned s_max[ATHREADS / 32];
+    const int tid = threadIdx.x;
+    const unsigned v = __reduce_max_sync(0xffffffffu, tid < n ? slots[tid] : 0u);
+    if ((tid & 31) == 0) s_max[tid >> 5] = v;
+    __syncthreads();
+    unsigned m = 0u;
+#pragma unroll
+    for (int w = 0; w < ATHREADS / 32; ++w) m = max(m, s_max[w]);
+    return m;
+}
+
+// max |y| comes from a.ymax_bits, or (n_slots > 0) is the maximum of that many block maxima.
 template <bool PREMUL>
-__device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index) {
+__device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index, const unsigned* slots = nullptr,
+                                             int n_slots = 0) {
     const int N = a.g.n;
     const int4 item = __ldg(reinterpret_cast<const int4*>(a.items + item_index));
     const int tile = item.x, nrec = item.z, split = item.w;
@@ -144,7 +160,7 @@ __device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index) {
     await_predecessor();
     if (a.stop && *(volatile const int*)a.stop) return;
     // the scale of the ATILE tile that holds this work tile
-    const float bound = __uint_as_float(*after_wait(a.ymax_bits)) * __ldg(&a.tile_kmax[(y0 / ATILE) * a.tiles_x + x0 / ATILE]);
+    const float bound = __uint_as_float(n_slots > 0 ? max_of_slots(after_wait(slots), n_slots) : *after_wait(a.ymax_bits)) * __ldg(&a.tile_kmax[(y0 / ATILE) * a.tiles_x + x0 / ATILE]);
     const float scale = 1073741824.0f / bound;  // 2^30 / bound
     const float* __restrict__ y = after_wait(a.y);
     const AdjConst ac{make_float2(a.g.dr_f, a.g.dr_f), make_float2(a.g.rh_f, a.g.rh_f), make_float2(scale, scale), a.g.wk, a.g.n_t};
@@ -198,8 +214,51 @@ __device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index) {
     }
 }
 
-__global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles(AdjArgs a) {
-    adjoint_item<false>(a, blockIdx.x);
+// K^T of one data set: slots hold the block maxima of |y| that k_adjoint_prep leaves; the
+// maximum goes to ymax_out for the conversion that follows.
+template <bool PREMUL>
+__global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles(const __grid_constant__ AdjArgs a,
+                                                                            const unsigned* __restrict__ slots, int n_slots,
+                                                                            unsigned* __restrict__ ymax_out) {
+    adjoint_item<PREMUL>(a, blockIdx.x, slots, n_slots);
+    if (blockIdx.x == 0) {
+        const unsigned m = max_of_slots(slots, n_slots);
+        if (threadIdx.x == 0) *ymax_out = m;
+    }
+    dependents_may_start();
+}
+
+// Before K^T of one data set: clears the fixed-point image, leaves each block's max |y| (as
+// float bits) in its slot and, when qw is not NULL, writes the data times the arc weights in
+// rows of row_stride(T).  One launch instead of a clear and a maximum, and the aligned copy
+// serves K^T's paired loads (pat_adjoint, 256^2 with 256 detectors: 36.9 -> 24.6 us per call).
+__global__ void __launch_bounds__(512) k_adjoint_prep(const float* __restrict__ y, const float* __restrict__ wk, int D, int T,
+                                                      float* __restrict__ qw, int* __restrict__ acc, long long nn,
+                                                      unsigned* __restrict__ slots) {
+    const long long first = blockIdx.x * (long long)blockDim.x + threadIdx.x, step = (long long)gridDim.x * blockDim.x;
+    for (long long i = first; i < nn; i += step) acc[i] = 0;
+    unsigned m = 0u;
+    const unsigned Tp = row_stride(T);
+    // rows padded to an even length: entry k == T of an odd row is zero
+    for (long long i = first; i < (long long)D * Tp; i += step) {
+        const unsigned d = (unsigned)i / Tp, k = (unsigned)i - d * Tp;   // D * Tp <= 2^32
+        float v = 0.f;
+        if (k < (unsigned)T) {
+            v = __ldg(y + (size_t)d * T + k);
+            m = max(m, __float_as_uint(fabsf(v)));
+            v *= __ldg(wk + k);
+        }
+        if (qw) qw[i] = v;
+    }
+    __shared__ unsigned s_max[16];
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = __reduce_max_sync(0xffffffffu, threadIdx.x < blockDim.x / 32 ? s_max[threadIdx.x] : 0u);
+        if (threadIdx.x == 0) slots[blockIdx.x] = m;
+    }
+    dependents_may_start();
 }
 
 template <bool PREMUL>
@@ -213,7 +272,10 @@ __global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles_b(co
 // out = the fixed-point K^T image in floating point
 __global__ void k_kt_to_float(KtView kt, int N, float* __restrict__ out) {
     const int gx = blockIdx.x * blockDim.x + threadIdx.x, gy = blockIdx.y * blockDim.y + threadIdx.y;
+    await_predecessor();
     if (gx >= N || gy >= N) return;
+    kt.acc = after_wait(kt.acc);
+    kt.ymax_bits = after_wait(kt.ymax_bits);
     out[(size_t)gy * N + gx] = kt.at(gx, gy, N);
 }
 
@@ -273,32 +335,47 @@ int launch_adjoint_b(const AdjArgs* args, const int2* map, int nblocks, bool pre
     return PAT_OK;
 }
 
-// K^T y through caller-provided scratch: the max word at ymax_bits and the fixed-point
-// image at acc (N*N int32), both already zero; no allocation and no profiling events.
-int launch_adjoint_into(const pat_geometry* g, const float* y, unsigned* ymax_bits, int* acc, float* out,
-                        cudaStream_t st) {
-    const int N = g->desc.n;
-    const long long S = (long long)g->desc.n_det * g->desc.n_t;
-    const int arc = launch_absmax(y, S, ymax_bits, st);
-    if (arc) return arc;
-    const AdjArgs a = make_adj_args(g, y, nullptr, ymax_bits, acc, nullptr);
-    k_adjoint_tiles<<<g->adj_items, ATHREADS, 0, st>>>(a);
-    PAT_LAUNCH_CHECK("k_adjoint_tiles");
-    dim3 blk(32, 8), grd(ceil_div(N, 32), ceil_div(N, 8));
-    k_kt_to_float<<<grd, blk, 0, st>>>(kt_view(g, acc, ymax_bits), N, out);
-    PAT_LAUNCH_CHECK("k_kt_to_float");
-    return PAT_OK;
+// K^T y through caller-provided scratch: head (a word for the maximum and n_slots for block
+// maxima), the fixed-point image acc (N*N int32) and, when not NULL, qw
+// (D * row_stride(T) floats, 8-byte aligned).  No allocation and no profiling events.
+int launch_adjoint_into(const pat_geometry* g, const float* y, unsigned* head, int n_slots, int* acc, float* qw,
+                        float* out, cudaStream_t st) {
+    const int N = g->desc.n, D = g->desc.n_det, T = g->desc.n_t;
+    const long long work = std::max((long long)N * N, (long long)D * T);
+    unsigned *ymax = head, *slots = head + 1;
+    n_slots = std::max(1, std::min({n_slots, ATHREADS, 2 * sm_count(), ceil_div(work, 512)}));
+    k_adjoint_prep<<<n_slots, 512, 0, st>>>(y, g->view.wk, D, T, qw, acc, (long long)N * N, slots);
+    PAT_LAUNCH_CHECK("k_adjoint_prep");
+    const AdjArgs a = make_adj_args(g, y, qw, ymax, acc, nullptr);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)g->adj_items);
+    cfg.blockDim = dim3(ATHREADS);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    set_dependent_launch(attr[0]);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const unsigned* cslots = slots;
+    cudaError_t e = qw ? cudaLaunchKernelEx(&cfg, k_adjoint_tiles<true>, a, cslots, n_slots, ymax)
+                       : cudaLaunchKernelEx(&cfg, k_adjoint_tiles<false>, a, cslots, n_slots, ymax);
+    count_launch();
+    if (e != cudaSuccess) return cuda_fail(e, "k_adjoint_tiles");
+    cfg.gridDim = dim3((unsigned)ceil_div(N, 32), (unsigned)ceil_div(N, 8));
+    cfg.blockDim = dim3(32, 8);
+    e = cudaLaunchKernelEx(&cfg, k_kt_to_float, kt_view(g, acc, ymax), N, out);
+    count_launch();
+    return e == cudaSuccess ? PAT_OK : cuda_fail(e, "k_kt_to_float");
 }
 
 int launch_adjoint(const pat_geometry* g, const float* y, float* out, cudaStream_t st) {
     int rc = ensure_precond(g, st);
     if (rc) return rc;
     char* scratch = nullptr;
-    const size_t bytes = 256 + (size_t)g->desc.n * g->desc.n * sizeof(int);
+    const size_t head = 4096, acc = ((size_t)g->desc.n * g->desc.n * sizeof(int) + 255) & ~(size_t)255;
+    const size_t bytes = head + acc + (size_t)g->desc.n_det * row_stride(g->desc.n_t) * sizeof(float);
     PAT_CUDA(cudaMallocAsync((void**)&scratch, bytes, st));
-    const cudaError_t e = cudaMemsetAsync(scratch, 0, bytes, st);
-    rc = e == cudaSuccess ? launch_adjoint_into(g, y, (unsigned*)scratch, (int*)(scratch + 256), out, st)
-                          : cuda_fail(e, "launch_adjoint: scratch");
+    rc = launch_adjoint_into(g, y, (unsigned*)scratch, (int)(head / 4) - 1, (int*)(scratch + head),
+                             (float*)(scratch + head + acc), out, st);
     cudaFreeAsync(scratch, st);
     return rc;
 }

@@ -1,5 +1,5 @@
 // pat_adjoint_noalloc: K^T y for callers that must not allocate device memory during
-// the call.  Its scratch (one max word and the fixed-point K^T image) lives in a
+// the call.  Its scratch (the maximum, block maxima and the fixed-point K^T image) lives in a
 // file-scope device array that every GPU loading this library holds until exit.
 #include <mutex>
 
@@ -8,7 +8,7 @@
 namespace pat {
 
 constexpr int kNoAllocMaxN = 1024;                       // largest image side served
-constexpr size_t kNoAllocHeadInts = 64;                  // 256 bytes: the max word
+constexpr size_t kNoAllocHeadInts = 64;                  // 256 bytes: the max word and block maxima
 constexpr size_t kNoAllocInts = kNoAllocHeadInts + (size_t)kNoAllocMaxN * kNoAllocMaxN;
 
 // 4 MiB + 256 B per device.  Host code must not use this name as an address: it is a
@@ -57,7 +57,6 @@ extern "C" int pat_adjoint_noalloc(const pat_geometry* g, const float* y_dev, fl
     int rc = noalloc_scratch(device, &scratch);
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    // the scratch keeps the previous call's contents: clear the part this call uses
-    PAT_CUDA(cudaMemsetAsync(scratch, 0, (kNoAllocHeadInts + (size_t)N * N) * sizeof(int), st));
-    return launch_adjoint_into(g, y_dev, (unsigned*)scratch, scratch + kNoAllocHeadInts, u_dev, st);
+    return launch_adjoint_into(g, y_dev, (unsigned*)scratch, (int)kNoAllocHeadInts - 1, scratch + kNoAllocHeadInts,
+                               nullptr, u_dev, st);
 }

@@ -449,9 +449,10 @@ int launch_forward(const pat_geometry* g, const float* u, float* y, cudaStream_t
 // K^T y into an N*N float image (allocates its scratch from the stream-ordered pool).
 int launch_adjoint(const pat_geometry* g, const float* y, float* out, cudaStream_t st);
 KtView kt_view(const pat_geometry* g, const int* acc, const unsigned* ymax_bits);
-// K^T y into an N*N float image using caller-provided, zeroed scratch (allocates nothing).
-int launch_adjoint_into(const pat_geometry* g, const float* y, unsigned* ymax_bits, int* acc, float* out,
-                        cudaStream_t st);
+// K^T y into an N*N float image using caller-provided scratch (allocates nothing): head holds
+// 1 + n_slots words, acc N*N, qw (or NULL) D * row_stride(T) floats on an 8-byte boundary.
+int launch_adjoint_into(const pat_geometry* g, const float* y, unsigned* head, int n_slots, int* acc, float* qw,
+                        float* out, cudaStream_t st);
 
 
 // max |y| as float bits into *out (which must hold 0 or a smaller value beforehand)

@@ -276,17 +276,13 @@ __device__ __forceinline__ void gap_pixel_share(const GapArgs& g, int first, int
 // K (Sec. 3.3.1, eq. (K_def)) for the row groups of one cluster, then the epilogue on
 // their rows.  The S partial sums of a row (one per slab) are added in rank (slab) order,
 // so the result does not depend on scheduling.
+// pm: problem (of gap and fin) and CTA of its plan.
 template <int EPI, int NT>
-__global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdArgs* __restrict__ args,
-                                                           const int2* __restrict__ map,
-                                                           const GapArgs* __restrict__ gap,
-                                                           const FinalArgs* __restrict__ fin) {
+__device__ __forceinline__ void forward_cta(const FwdArgs& a, const int2 pm, const GapArgs* __restrict__ gap,
+                                            const FinalArgs* __restrict__ fin) {
     extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ FwdArgs sa;
     __shared__ int s_next;
     __shared__ unsigned s_qmax;
-    const int2 pm = map[blockIdx.x];
-    const FwdArgs& a = stage_args(args, pm.x, sa);
     const GeomView& g = a.g;
     const int N = g.n, T = g.n_t, S = g.n_slabs, M = g.quad_m, D = g.n_det;
     const unsigned rank = S > 1 ? cluster_rank() : 0u;
@@ -412,6 +408,24 @@ __global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdA
     }
 }
 
+template <int EPI, int NT>
+__global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_b(const FwdArgs* __restrict__ args,
+                                                           const int2* __restrict__ map,
+                                                           const GapArgs* __restrict__ gap,
+                                                           const FinalArgs* __restrict__ fin) {
+    __shared__ FwdArgs sa;
+    const int2 pm = map[blockIdx.x];
+    forward_cta<EPI, NT>(stage_args(args, pm.x, sa), pm, gap, fin);
+}
+
+// y = K u of one image: the arguments are kernel parameters, so a call is one launch with
+// nothing to allocate or copy before it (64^2 with 64 detectors: 14.3 -> 8.2 us per call among
+// others, 205 -> 30 us alone, where the pool had to be refilled).
+template <int NT>
+__global__ void __launch_bounds__(NT, NT >= 1024 ? 1 : 2) k_forward_one(const __grid_constant__ FwdArgs a) {
+    forward_cta<FWD_Y, NT>(a, make_int2(0, (int)blockIdx.x), nullptr, nullptr);
+}
+
 // max |y| over n values as float bits (atomicMax; *out must start at 0)
 __global__ void k_absmax(const float* __restrict__ y, long long n, unsigned* __restrict__ out) {
     unsigned m = 0;
@@ -497,7 +511,7 @@ int forward_smem_bytes(int rows, int stride, int M, int D, bool staged) {
 // set once per kernel and device.
 template <int NT>
 static cudaError_t forward_attributes_nt() {
-    const void* ks[3] = {(const void*)k_forward_b<FWD_Y, NT>, (const void*)k_forward_b<FWD_PROX, NT>,
+    const void* ks[3] = {(const void*)k_forward_one<NT>, (const void*)k_forward_b<FWD_PROX, NT>,
                          (const void*)k_forward_b<FWD_GAP, NT>};
     for (const void* k : ks) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, FWD_SMEM_ONE);
@@ -558,7 +572,6 @@ int forward_clusters_per_gpu(int cluster, int smem) {
 template <int NT>
 static cudaError_t launch_forward_nt(int epi, const cudaLaunchConfig_t& cfg, const FwdArgs* args, const int2* map,
                                      const GapArgs* gap, const FinalArgs* fin) {
-    if (epi == FWD_Y) return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_Y, NT>, args, map, gap, fin);
     if (epi == FWD_PROX) return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_PROX, NT>, args, map, gap, fin);
     return cudaLaunchKernelEx(&cfg, k_forward_b<FWD_GAP, NT>, args, map, gap, fin);
 }
@@ -580,26 +593,18 @@ int launch_forward_b(int epi, const FwdArgs* args, const int2* map, int nblocks,
 }
 
 int launch_forward(const pat_geometry* g, const float* u, float* y, cudaStream_t st) {
-    const int nc = g->fwd_n_ctas;
-    const size_t map_off = (sizeof(FwdArgs) + 255) & ~(size_t)255;
-    const size_t bytes = map_off + (size_t)nc * sizeof(int2);
-    char* buf = nullptr;
-    PAT_CUDA(cudaMallocAsync((void**)&buf, bytes, st));
+    const int arc = forward_attributes();
+    if (arc) return arc;
     FwdArgs a = make_fwd_args(g, u);
     a.y = y;
-    std::vector<int2> map(nc);
-    for (int i = 0; i < nc; ++i) map[i] = make_int2(0, i);
-    int rc = PAT_OK;
-    cudaError_t e = cudaMemcpyAsync(buf, &a, sizeof a, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(buf + map_off, map.data(), (size_t)nc * sizeof(int2), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) rc = cuda_fail(e, "launch_forward: arguments");
-    // (copies from pageable host memory are staged before cudaMemcpyAsync returns, so the
-    // host arguments may go out of scope)
-    if (!rc)
-        rc = launch_forward_b(FWD_Y, (const FwdArgs*)buf, (const int2*)(buf + map_off), nc, g->view.n_slabs,
-                              g->fwd_smem, st);
-    cudaFreeAsync(buf, st);
-    return rc;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = forward_config(g->fwd_n_ctas, g->view.n_slabs, g->fwd_smem, st, attr);
+    cfg.numAttrs = 1;   // (the launch before it may be the caller's, which need not wait for its own predecessors)
+    const cudaError_t e = forward_threads(g->fwd_smem) == FWD_THREADS_WIDE
+                              ? cudaLaunchKernelEx(&cfg, k_forward_one<FWD_THREADS_WIDE>, a)
+                              : cudaLaunchKernelEx(&cfg, k_forward_one<FWD_THREADS>, a);
+    count_launch();
+    return e == cudaSuccess ? PAT_OK : cuda_fail(e, "k_forward_one");
 }
 
 int launch_absmax(const float* y, long long n, unsigned* out, cudaStream_t st) {
