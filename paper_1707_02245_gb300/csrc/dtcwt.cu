@@ -27,9 +27,12 @@ namespace {
 
 constexpr float kHalfInvSqrt2 = 0.35355339059327373f;   // 1 / (2 sqrt 2)
 
+// a mod m for a within a few m of [0, m) (an index plus or minus at most a filter's taps; a
+// division here took most of the transforms' instructions)
 __device__ __forceinline__ int imod(int a, int m) {
-    const int r = a % m;
-    return r < 0 ? r + m : r;
+    while (a < 0) a += m;
+    while (a >= m) a -= m;
+    return a;
 }
 
 // filters of tree `tree` (0 = a, 1 = b) at a level: low-pass h, high-pass g, length, offset
@@ -47,55 +50,122 @@ __device__ __forceinline__ AxisF axis_filters(const CwtBank& b, int tree, bool l
 // problem) can share one grid: blockIdx.z = 4 b + t for the per-tree kernels (tree t of
 // problem b), blockIdx.z = b or blockIdx.y = b for the others.
 
-// One analysis level of the four trees: out plane t (stride so, plane stride ps) block
-// M x M from in (plane t at in + t * in_ps, stride si; in_ps = 0 reads one image for all).
-__global__ void k_cwt_analysis(const float* __restrict__ in, long long in_ps, int si, float* __restrict__ out,
-                               long long ps, int so, int M, int level1, const CwtBank bank, const int* stop,
-                               long long pb, float* __restrict__ ll, long long ll_ps) {
-    const long long po = pb * (blockIdx.z >> 2);
-    in = at_bytes(in, po);
-    out = at_bytes(out, po);
-    ll = ll ? at_bytes(ll, po) : ll;
-    stop = stop ? at_bytes(stop, po) : stop;
-    if (stop && *(volatile const int*)stop) return;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, t = blockIdx.z & 3;
-    if (x >= M || y >= M) return;
-    const AxisF fx = axis_filters(bank, t >> 1, level1), fy = axis_filters(bank, t & 1, level1);
+// One analysis step of tree t at (x, y) of its M x M output, from src (stride si).  L > 0:
+// filters of L taps, all their loads in flight at once; 0: any length.
+//
+// The transforms are bound by latency at 256^2 (ten launches of an iteration): the loads'
+// addresses without divisions, all loads of a value at once and launches on one another's
+// tails took a DT-CWT iteration with 128 detectors from 110 to 66 us.  One launch for all
+// coarse levels (a cluster per tree, a cluster barrier per level) was slower: 75 us.
+template <int L>
+__device__ __forceinline__ float cwt_analysis_at(const float* src, int si, int M, int x, int y, const AxisF& fx,
+                                                 const AxisF& fy) {
     const int h2 = M >> 1;
     const bool hx = x >= h2, hy = y >= h2;
     const int kx = hx ? x - h2 : x, ky = hy ? y - h2 : y;
     const float* fxv = hx ? fx.g : fx.h;
     const float* fyv = hy ? fy.g : fy.h;
-    const float* src = in + in_ps * t;
     float acc = 0.f;
+    if (L > 0) {
+        float v[L > 0 ? L : 1][L > 0 ? L : 1];
+#pragma unroll
+        for (int a = 0; a < L; ++a) {
+            const float* row = src + (size_t)imod(2 * ky + a + fy.off, M) * si;
+#pragma unroll
+            for (int b = 0; b < L; ++b) v[a][b] = row[imod(2 * kx + b + fx.off, M)];
+        }
+#pragma unroll
+        for (int a = 0; a < L; ++a) {
+            float r = 0.f;
+#pragma unroll
+            for (int b = 0; b < L; ++b) r = fmaf(fxv[b], v[a][b], r);
+            acc = fmaf(fyv[a], r, acc);
+        }
+        return acc;
+    }
     for (int a = 0; a < fy.len; ++a) {
         const float* row = src + (size_t)imod(2 * ky + a + fy.off, M) * si;
         float r = 0.f;
-        for (int b = 0; b < fx.len; ++b) r = fmaf(fxv[b], __ldg(row + imod(2 * kx + b + fx.off, M)), r);
+        for (int b = 0; b < fx.len; ++b) r = fmaf(fxv[b], row[imod(2 * kx + b + fx.off, M)], r);
         acc = fmaf(fyv[a], r, acc);
     }
-    out[ps * t + (size_t)y * so + x] = acc;
-    if (ll && !hx && !hy) ll[ll_ps * t + (size_t)y * h2 + x] = acc;   // the next level's input (stride M / 2)
+    return acc;
+}
+
+// One analysis level of the four trees: out plane t (stride so, plane stride ps) block
+// M x M from in (plane t at in + t * in_ps, stride si; in_ps = 0 reads one image for all).
+template <int L>
+__global__ void k_cwt_analysis(const float* in, long long in_ps, int si, float* out,
+                               long long ps, int so, int M, int level1, const CwtBank bank, const int* stop,
+                               long long pb, float* ll, long long ll_ps) {
+    const long long po = pb * (blockIdx.z >> 2);
+    in = at_bytes(in, po);
+    out = at_bytes(out, po);
+    ll = ll ? at_bytes(ll, po) : ll;
+    stop = stop ? at_bytes(stop, po) : stop;
+    await_predecessor();
+    if (stop && *(volatile const int*)stop) return;
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, t = blockIdx.z & 3;
+    if (x < M && y < M) {
+        const int h2 = M >> 1;
+        const float acc = cwt_analysis_at<L>(in + in_ps * t, si, M, x, y, axis_filters(bank, t >> 1, level1),
+                                          axis_filters(bank, t & 1, level1));
+        out[ps * t + (size_t)y * so + x] = acc;
+        if (ll && x < h2 && y < h2) ll[ll_ps * t + (size_t)y * h2 + x] = acc;   // the next level's input (stride M / 2)
+    }
+    dependents_may_start();
 }
 
 // Transpose of one analysis level of tree t applied to the coefficient block (in plane t,
 // stride si, quadrants of size M/2): value at (y, x) of the M x M output.
 // The LL quadrant comes from ll (stride sl) and the three detail quadrants from c (stride
 // si); both are c itself for the coarsest level.
-__device__ __forceinline__ float cwt_synth_at(const float* __restrict__ ll, int sl, const float* __restrict__ c,
-                                              int si, int M, int x, int y, const AxisF& fx, const AxisF& fy) {
+template <int L>
+__device__ __forceinline__ float cwt_synth_at(const float* ll, int sl, const float* c, int si, int M, int x, int y,
+                                              const AxisF& fx, const AxisF& fy) {
     const int h2 = M >> 1;
     float acc = 0.f;
     // taps a with y = 2 ky + a + off (mod M): a has the parity of y - off
-    for (int a = imod(y - fy.off, 2); a < fy.len; a += 2) {
+    const int a0 = (y - fy.off) & 1, b0 = (x - fx.off) & 1;
+    if (L > 0) {
+        constexpr int H = L > 0 ? L / 2 : 1;
+        float v[H][H][4];
+#pragma unroll
+        for (int p = 0; p < H; ++p) {
+            const int ky = imod(y - (a0 + 2 * p) - fy.off, M) >> 1;
+            const float *r0 = c + (size_t)ky * si, *r1 = c + (size_t)(ky + h2) * si, *rl = ll + (size_t)ky * sl;
+#pragma unroll
+            for (int q = 0; q < H; ++q) {
+                const int kx = imod(x - (b0 + 2 * q) - fx.off, M) >> 1;
+                v[p][q][0] = rl[kx];
+                v[p][q][1] = r0[kx + h2];
+                v[p][q][2] = r1[kx];
+                v[p][q][3] = r1[kx + h2];
+            }
+        }
+#pragma unroll
+        for (int p = 0; p < H; ++p) {
+            const int a = a0 + 2 * p;
+            float lo = 0.f, hi = 0.f;
+#pragma unroll
+            for (int q = 0; q < H; ++q) {
+                const int b = b0 + 2 * q;
+                lo = fmaf(fx.h[b], v[p][q][0], fmaf(fx.g[b], v[p][q][1], lo));
+                hi = fmaf(fx.h[b], v[p][q][2], fmaf(fx.g[b], v[p][q][3], hi));
+            }
+            acc = fmaf(fy.h[a], lo, fmaf(fy.g[a], hi, acc));
+        }
+        return acc;
+    }
+    for (int a = a0; a < fy.len; a += 2) {
         const int ky = imod(y - a - fy.off, M) >> 1;
         float lo = 0.f, hi = 0.f;
-        for (int b = imod(x - fx.off, 2); b < fx.len; b += 2) {
+        for (int b = b0; b < fx.len; b += 2) {
             const int kx = imod(x - b - fx.off, M) >> 1;
             const float* r0 = c + (size_t)ky * si;
             const float* r1 = c + (size_t)(ky + h2) * si;
-            lo = fmaf(fx.h[b], __ldg(ll + (size_t)ky * sl + kx), fmaf(fx.g[b], __ldg(r0 + kx + h2), lo));
-            hi = fmaf(fx.h[b], __ldg(r1 + kx), fmaf(fx.g[b], __ldg(r1 + kx + h2), hi));
+            lo = fmaf(fx.h[b], ll[(size_t)ky * sl + kx], fmaf(fx.g[b], r0[kx + h2], lo));
+            hi = fmaf(fx.h[b], r1[kx], fmaf(fx.g[b], r1[kx + h2], hi));
         }
         acc = fmaf(fy.h[a], lo, fmaf(fy.g[a], hi, acc));
     }
@@ -105,40 +175,48 @@ __device__ __forceinline__ float cwt_synth_at(const float* __restrict__ ll, int 
 // Levels >= 2: out plane t (M x M, stride so, plane stride ops) from the detail quadrants
 // of in plane t (stride si, plane stride ips) and the LL quadrant in ll (stride sl, plane
 // stride lps: the level above's output, or in itself at the coarsest level).
-__global__ void k_cwt_synthesis(const float* __restrict__ ll, long long lps, int sl, const float* __restrict__ in,
-                                long long ips, int si, float* __restrict__ out, long long ops, int so, int M,
+template <int L>
+__global__ void k_cwt_synthesis(const float* ll, long long lps, int sl, const float* in,
+                                long long ips, int si, float* out, long long ops, int so, int M,
                                 const CwtBank bank, const int* stop, long long pb) {
     const long long po = pb * (blockIdx.z >> 2);
     ll = at_bytes(ll, po);
     in = at_bytes(in, po);
     out = at_bytes(out, po);
     stop = stop ? at_bytes(stop, po) : stop;
+    await_predecessor();
     if (stop && *(volatile const int*)stop) return;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y, t = blockIdx.z & 3;
-    if (x >= M || y >= M) return;
-    const AxisF fx = axis_filters(bank, t >> 1, false), fy = axis_filters(bank, t & 1, false);
-    out[ops * t + (size_t)y * so + x] = cwt_synth_at(ll + lps * t, sl, in + ips * t, si, M, x, y, fx, fy);
+    if (x < M && y < M) {
+        const AxisF fx = axis_filters(bank, t >> 1, false), fy = axis_filters(bank, t & 1, false);
+        out[ops * t + (size_t)y * so + x] = cwt_synth_at<L>(ll + lps * t, sl, in + ips * t, si, M, x, y, fx, fy);
+    }
+    dependents_may_start();
 }
 
 // Level 1 and the sum of the four trees: out (N x N) = sum_t T_t^T level 1 of plane t (LL
 // quadrants from ll, stride sl, plane stride lps).
-__global__ void k_cwt_synthesis_sum(const float* __restrict__ ll, long long lps, int sl, const float* __restrict__ in,
-                                    long long ips, int si, float* __restrict__ out, int N, const CwtBank bank,
+template <int L>
+__global__ void k_cwt_synthesis_sum(const float* ll, long long lps, int sl, const float* in,
+                                    long long ips, int si, float* out, int N, const CwtBank bank,
                                     const int* stop, long long pb) {
     const long long po = pb * blockIdx.z;
     ll = at_bytes(ll, po);
     in = at_bytes(in, po);
     out = at_bytes(out, po);
     stop = stop ? at_bytes(stop, po) : stop;
+    await_predecessor();
     if (stop && *(volatile const int*)stop) return;
     const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-    if (x >= N || y >= N) return;
-    float acc = 0.f;
+    if (x < N && y < N) {
+        float acc = 0.f;
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
-        acc += cwt_synth_at(ll + lps * t, sl, in + ips * t, si, N, x, y, axis_filters(bank, t >> 1, true),
-                            axis_filters(bank, t & 1, true));
-    out[(size_t)y * N + x] = acc;
+        for (int t = 0; t < 4; ++t)
+            acc += cwt_synth_at<L>(ll + lps * t, sl, in + ips * t, si, N, x, y, axis_filters(bank, t >> 1, true),
+                                axis_filters(bank, t & 1, true));
+        out[(size_t)y * N + x] = acc;
+    }
+    dependents_may_start();
 }
 
 
@@ -158,27 +236,45 @@ __device__ __forceinline__ void combine_at(const float* __restrict__ T, long lon
     }
 }
 
+// The coefficients c of one position in tree form, each times 1/2, into the T planes (the
+// change back from the complex pairs is the transpose of combine_at's change).
+__device__ __forceinline__ void uncombine_at(const float (&c)[4], float* __restrict__ T, long long NN, long long i, bool ll) {
+    if (ll) {
+        T[i] = 0.5f * c[0];
+        T[NN + i] = 0.5f * c[1];
+        T[2 * NN + i] = 0.5f * c[2];
+        T[3 * NN + i] = 0.5f * c[3];
+    } else {
+        T[i] = (c[0] + c[2]) * kHalfInvSqrt2;
+        T[NN + i] = (c[1] - c[3]) * kHalfInvSqrt2;
+        T[2 * NN + i] = (c[1] + c[3]) * kHalfInvSqrt2;
+        T[3 * NN + i] = (c[2] - c[0]) * kHalfInvSqrt2;
+    }
+}
+
 // r <- prox_{sigma F2*}(r + sigma W ubar) (Sec. 3.2) from the T planes of ubar: every complex
 // detail coefficient onto the disc of radius alpha (its two rows share one step), every LL
-// coefficient clipped to [-alpha, alpha].
+// coefficient clipped to [-alpha, alpha].  T_r receives the new r in tree form, for W^T.
 __global__ void k_cwt_dual(float* __restrict__ r, const float* __restrict__ T, const float* __restrict__ sig_r,
                            const float* step_mul, const float* scal, int N, int ll_side, const int* stop,
-                           long long pb) {
+                           long long pb, float* __restrict__ T_r) {
     const long long po = pb * blockIdx.y;
     r = at_bytes(r, po);
     T = at_bytes(T, po);
+    T_r = at_bytes(T_r, po);
     sig_r = at_bytes(sig_r, po);
     step_mul = at_bytes(step_mul, po);
     stop = stop ? at_bytes(stop, po) : stop;
+    await_predecessor();
     if (stop && *(volatile const int*)stop) return;
     const long long NN = (long long)N * N;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= NN) return;
     const float alpha = *at_bytes(scal, po);
-    const int x = (int)(i % N), y = (int)(i / N);
+    const int y = (int)i / N, x = (int)i - y * N;   // N <= 16384
     const bool ll = x < ll_side && y < ll_side;
     float c[4];
-    combine_at(T, NN, i, ll, c);
+    combine_at(after_wait(T), NN, i, ll, c);
     const float sm = __ldg(step_mul + 1);
     float v[4];
 #pragma unroll
@@ -199,32 +295,43 @@ __global__ void k_cwt_dual(float* __restrict__ r, const float* __restrict__ T, c
     }
 #pragma unroll
     for (int k = 0; k < 4; ++k) r[k * NN + i] = v[k];
+    uncombine_at(v, T_r, NN, i, ll);
+    dependents_may_start();
 }
 
-// T planes of W^T: the coefficients r in tree form, each times 1/2 (the change back from the
-// complex pairs is the transpose of the change above)
-__global__ void k_cwt_uncombine(const float* __restrict__ r, float* __restrict__ T, int N, int ll_side, const int* stop,
-                                long long pb) {
-    const long long po = pb * blockIdx.y;
-    r = at_bytes(r, po);
-    T = at_bytes(T, po);
-    stop = stop ? at_bytes(stop, po) : stop;
-    if (stop && *(volatile const int*)stop) return;
+// T planes of W^T: the coefficients r in tree form (for the API)
+__global__ void k_cwt_uncombine(const float* __restrict__ r, float* __restrict__ T, int N, int ll_side) {
     const long long NN = (long long)N * N;
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= NN) return;
-    const int x = (int)(i % N), y = (int)(i / N);
-    const float c0 = r[i], c1 = r[NN + i], c2 = r[2 * NN + i], c3 = r[3 * NN + i];
-    if (x < ll_side && y < ll_side) {
-        T[i] = 0.5f * c0;
-        T[NN + i] = 0.5f * c1;
-        T[2 * NN + i] = 0.5f * c2;
-        T[3 * NN + i] = 0.5f * c3;
-    } else {
-        T[i] = (c0 + c2) * kHalfInvSqrt2;
-        T[NN + i] = (c1 - c3) * kHalfInvSqrt2;
-        T[2 * NN + i] = (c1 + c3) * kHalfInvSqrt2;
-        T[3 * NN + i] = (c2 - c0) * kHalfInvSqrt2;
+    const float c[4] = {r[i], r[NN + i], r[2 * NN + i], r[3 * NN + i]};
+    uncombine_at(c, T, NN, i, (int)(i % N) < ll_side && (int)(i / N) < ll_side);
+}
+
+// sigma_r (4 N^2) and tau_u (N^2) of the alpha = 1 rule from the |W| tables of cwt_abs_tables:
+// a row's step is that of its level, orientation and plane; a pixel's column sum of |W| is the
+// sum over the levels of its residue's entry.
+__global__ void k_cwt_steps(const float* __restrict__ sig_tab, const double* __restrict__ fold,
+                            const float* __restrict__ kcol, int N, int levels, float* __restrict__ sig_r,
+                            float* __restrict__ tau) {
+    const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
+    if (x >= N || y >= N) return;
+    const size_t NN = (size_t)N * N, i = (size_t)y * N + x;
+    int l = 1;
+    while (l < levels && x < (N >> l) && y < (N >> l)) ++l;
+    const bool xh = x >= (N >> l), yh = y >= (N >> l);
+    const int band = 3 * (l - 1) + (xh && yh ? 2 : xh ? 0 : yh ? 1 : 3);   // HL, LH, HH; LL after the last level's
+    if (sig_r)
+        for (int c = 0; c < 4; ++c) sig_r[c * NN + i] = __ldg(sig_tab + 4 * band + c);
+    if (tau) {
+        double s = (double)kcol[i], w = 0.0;
+        for (int k = 1; k <= levels; ++k) {
+            const int P = 1 << k;
+            w += __ldg(fold + (size_t)(y & (P - 1)) * P + (x & (P - 1)));
+            fold += (size_t)P * P;
+        }
+        s += w;
+        tau[i] = s > 0 ? (float)(1.0 / s) : 1.f;
     }
 }
 
@@ -342,110 +449,116 @@ int cwt_bank(const double* h1, int l1, const double* hq, int lq, CwtBank& bank, 
     return PAT_OK;
 }
 
-// Row sums (4 N^2, the W layout) and column sums (N^2) of |W| in FP64.  Every row of W is a
-// circular shift of the row at coefficient index (0, 0) of its level, orientation and
-// plane, by 2^l per index, so all rows of one (level, orientation, plane) have the same sum,
-// and a column's sum over them is that row's |entries| summed over the pixels congruent to
-// the column modulo 2^l.  A row is built from the 1-D level functions of the two trees: the
-// level-l functions of a tree are sum_t f[t] (level l - 1 low-pass row (2k + t + o) mod M).
-void cwt_abs_sums(int n, int levels, const std::vector<double>& h1, const std::vector<double>& hq,
-                  std::vector<double>& rows, std::vector<double>& cols) {
-    const size_t NN = (size_t)n * n;
-    rows.assign(4 * NN, 0.0);
-    cols.assign(NN, 0.0);
+// Row and column sums of |W| in FP64, as tables.  Every row of W is a circular shift of the row
+// at coefficient index (0, 0) of its level, orientation and plane, by 2^l per index, so all
+// rows of one (level, orientation, plane) have the same sum: rows[4 band + plane], bands HL,
+// LH, HH of level 1, 2, ..., then LL of the last.  A column's sum over them is that row's
+// |entries| summed over the pixels congruent to the column modulo 2^l: fold holds, level by
+// level, the 2^l x 2^l sums over the level's orientations and planes.  The (0, 0) row is the
+// product of the two trees' 1-D level functions, f_l = sum_t f[t] shift(low_{l-1}, (t + o)
+// 2^(l-1)), of which only the entries that are not zero are visited (13 ms of host time per
+// call at 256^2 when the whole N x N rows were, 0.1 ms now).
+void cwt_abs_tables(int n, int levels, const std::vector<double>& h1, const std::vector<double>& hq,
+                    std::vector<double>& rows, std::vector<double>& fold) {
+    rows.assign(4 * (3 * (size_t)levels + 1), 0.0);
+    fold.clear();
     auto hp = [](const std::vector<double>& h) {
         std::vector<double> g(h.size());
         for (size_t k = 0; k < h.size(); ++k) g[k] = ((k & 1) ? -1.0 : 1.0) * h[h.size() - 1 - k];
         return g;
     };
-    std::vector<double> qb(hq.rbegin(), hq.rend());
-    // low-pass rows of the previous level per tree (M rows of length n)
-    std::vector<double> low[2];
+    const std::vector<double> qb(hq.rbegin(), hq.rend());
+    std::vector<double> low[2];   // index-0 low-pass function of the previous level, per tree
     for (int tr = 0; tr < 2; ++tr) {
-        low[tr].assign(NN, 0.0);
-        for (int i = 0; i < n; ++i) low[tr][(size_t)i * n + i] = 1.0;
+        low[tr].assign(n, 0.0);
+        low[tr][0] = 1.0;
     }
-    int M = n;
     const double c2 = 1.0 / (2.0 * std::sqrt(2.0));
-    std::vector<double> R(NN);
     for (int l = 1; l <= levels; ++l) {
-        const int h2 = M / 2;
-        std::vector<double> lo[2], hi[2];   // index-0 function and all rows of the new level
+        std::vector<double> lo[2], hi[2];
         for (int tr = 0; tr < 2; ++tr) {
             const std::vector<double>& h = l == 1 ? h1 : (tr ? qb : hq);
             const std::vector<double> g = hp(h);
             const int off = l == 1 ? tr : 0;
-            lo[tr].assign((size_t)h2 * n, 0.0);
-            hi[tr].assign((size_t)h2 * n, 0.0);
-            for (int k = 0; k < h2; ++k)
-                for (size_t t = 0; t < h.size(); ++t) {
-                    const double* src = &low[tr][(size_t)((2 * k + (int)t + off) % M) * n];
-                    for (int x = 0; x < n; ++x) {
-                        lo[tr][(size_t)k * n + x] += h[t] * src[x];
-                        hi[tr][(size_t)k * n + x] += g[t] * src[x];
-                    }
+            lo[tr].assign(n, 0.0);
+            hi[tr].assign(n, 0.0);
+            for (size_t t = 0; t < h.size(); ++t) {
+                const long long shift = ((long long)(t + off) << (l - 1)) % n;
+                for (int x = 0; x < n; ++x) {
+                    const double src = low[tr][(size_t)((x - shift + n) % n)];
+                    lo[tr][x] += h[t] * src;
+                    hi[tr][x] += g[t] * src;
                 }
+            }
         }
-        const int P = 1 << l;   // period of the column sums of this level
+        const int P = 1 << l;
+        const size_t f0 = fold.size();
+        fold.resize(f0 + (size_t)P * P, 0.0);
         const bool last = l == levels;
         // orientations: (x high, y high) in {(1,0) HL, (0,1) LH, (1,1) HH}, and LL at the last level
         for (int o = 0; o < (last ? 4 : 3); ++o) {
             const bool xh = o == 0 || o == 2, yh = o == 1 || o == 2, isll = o == 3;
-            const double* fx[2] = {(xh ? hi[0] : lo[0]).data(), (xh ? hi[1] : lo[1]).data()};   // index 0 rows
-            const double* fy[2] = {(yh ? hi[0] : lo[0]).data(), (yh ? hi[1] : lo[1]).data()};
-            const int bx = isll ? 0 : (xh ? h2 : 0), by = isll ? 0 : (yh ? h2 : 0);
+            const std::vector<double>*fx = xh ? hi : lo, *fy = yh ? hi : lo;
+            std::vector<int> sx, sy;   // where either tree's function is not zero
+            for (int k = 0; k < n; ++k) {
+                if (fx[0][k] != 0 || fx[1][k] != 0) sx.push_back(k);
+                if (fy[0][k] != 0 || fy[1][k] != 0) sy.push_back(k);
+            }
             for (int c = 0; c < 4; ++c) {
-                // R[y][x] = the (0, 0) row of plane c
-                for (int y = 0; y < n; ++y)
-                    for (int x = 0; x < n; ++x) {
+                double s = 0.0;
+                for (int y : sy)
+                    for (int x : sx) {
                         const double aa = fy[0][y] * fx[0][x], ab = fy[1][y] * fx[0][x];
                         const double ba = fy[0][y] * fx[1][x], bb = fy[1][y] * fx[1][x];
                         double v;
                         if (isll) v = 0.5 * (c == 0 ? aa : c == 1 ? ab : c == 2 ? ba : bb);
                         else v = c2 * (c == 0 ? aa - bb : c == 1 ? ab + ba : c == 2 ? aa + bb : ba - ab);
-                        R[(size_t)y * n + x] = std::fabs(v);
+                        v = std::fabs(v);
+                        s += v;
+                        fold[f0 + (size_t)(y % P) * P + (x % P)] += v;
                     }
-                double s = 0.0;
-                std::vector<double> fold((size_t)P * P, 0.0);
-                for (int y = 0; y < n; ++y)
-                    for (int x = 0; x < n; ++x) {
-                        s += R[(size_t)y * n + x];
-                        fold[(size_t)(y % P) * P + (x % P)] += R[(size_t)y * n + x];
-                    }
-                for (int ky = 0; ky < h2; ++ky)
-                    for (int kx = 0; kx < h2; ++kx) rows[c * NN + (size_t)(by + ky) * n + bx + kx] = s;
-                for (int y = 0; y < n; ++y)
-                    for (int x = 0; x < n; ++x) cols[(size_t)y * n + x] += fold[(size_t)(y % P) * P + (x % P)];
+                rows[4 * (3 * (size_t)(l - 1) + o) + c] = s;
             }
         }
-        low[0].swap(lo[0]);
-        low[1].swap(lo[1]);
-        M = h2;
+        for (int tr = 0; tr < 2; ++tr) low[tr].swap(lo[tr]);
     }
+}
+
+int launch_cwt_steps(const float* sig_tab, const double* fold, const float* kcol, int N, int levels, float* sig_r,
+                     float* tau, cudaStream_t st) {
+    k_cwt_steps<<<grid_of(N, 1), dim3(32, 8), 0, st>>>(sig_tab, fold, kcol, N, levels, sig_r, tau);
+    PAT_LAUNCH_CHECK("k_cwt_steps");
+    return PAT_OK;
 }
 
 // The LL block a level passes to the next lives in scratch, so no level overwrites its own
 // input: level l >= 2 reads buffer X_l and writes X_{l+1}, X_l = scratch (4 (N/2)^2 floats)
 // for even l and scratch + N^2 (4 (N/4)^2 floats) for odd l.  scratch: 5 N^2 / 4 floats.
-static float* cwt_ll_buffer(float* scratch, int N, int l) { return (l & 1) ? scratch + (size_t)N * N : scratch; }
+static float* cwt_ll_buffer(float* scratch, int N, int l) {
+    return (l & 1) ? scratch + (size_t)N * N : scratch;
+}
 
-// out (4 T planes of N x N) = T in.
+#define CWT_LAUNCH(call, what)                                  \
+    do {                                                        \
+        const cudaError_t e_ = (call);                          \
+        count_launch();                                         \
+        if (e_ != cudaSuccess) return cuda_fail(e_, what);      \
+    } while (0)
+
+// out (4 T planes of N x N) = T in.  dep: launched behind the library's own kernels, so the
+// first one may start on its predecessor's tail.
 int launch_cwt_analysis(const float* in, int N, int levels, const CwtBank& bank, float* out, float* scratch,
-                        const int* stop, cudaStream_t st, int B, long long pb) {
+                        const int* stop, cudaStream_t st, int B, long long pb, bool dep) {
     const dim3 blk(32, 8);
-    const long long NN = (long long)N * N;
-    k_cwt_analysis<<<grid_of(N, 4 * B), blk, 0, st>>>(in, 0, N, out, NN, N, N, 1, bank, stop, pb,
-                                                      levels >= 2 ? cwt_ll_buffer(scratch, N, 2) : nullptr,
-                                                      (long long)(N / 2) * (N / 2));
-    PAT_LAUNCH_CHECK("k_cwt_analysis");
-    for (int l = 2, M = N / 2; l <= levels; ++l, M /= 2) {
-        const long long mm = (long long)M * M;
-        k_cwt_analysis<<<grid_of(M, 4 * B), blk, 0, st>>>(cwt_ll_buffer(scratch, N, l), mm, M, out, NN, N, M, 0, bank,
-                                                          stop, pb,
-                                                          l < levels ? cwt_ll_buffer(scratch, N, l + 1) : nullptr,
-                                                          (long long)(M / 2) * (M / 2));
-        PAT_LAUNCH_CHECK("k_cwt_analysis");
-    }
+    const long long NN = (long long)N * N, zero = 0;
+    CWT_LAUNCH(launch_ex(bank.l1 == 4 ? k_cwt_analysis<4> : k_cwt_analysis<0>, grid_of(N, 4 * B), blk, st, dep, in, zero, N, out, NN, N, N, 1, bank, stop, pb,
+                         levels >= 2 ? cwt_ll_buffer(scratch, N, 2) : nullptr, (long long)(N / 2) * (N / 2)),
+               "k_cwt_analysis");
+    for (int l = 2, M = N / 2; l <= levels; ++l, M /= 2)
+        CWT_LAUNCH(launch_ex(bank.lq == 4 ? k_cwt_analysis<4> : k_cwt_analysis<0>, grid_of(M, 4 * B), blk, st, true, cwt_ll_buffer(scratch, N, l),
+                             (long long)M * M, M, out, NN, N, M, 0, bank, stop, pb,
+                             l < levels ? cwt_ll_buffer(scratch, N, l + 1) : nullptr, (long long)(M / 2) * (M / 2)),
+                   "k_cwt_analysis");
     return PAT_OK;
 }
 
@@ -462,31 +575,24 @@ int launch_cwt_synthesis(float* in, int N, int levels, const CwtBank& bank, floa
         const int M = N >> (l - 1);
         const long long mm = (long long)M * M;
         float* dst = cwt_ll_buffer(scratch, N, l);
-        k_cwt_synthesis<<<grid_of(M, 4 * B), blk, 0, st>>>(ll, lps, sl, in, NN, N, dst, mm, M, M, bank, stop, pb);
-        PAT_LAUNCH_CHECK("k_cwt_synthesis");
+        CWT_LAUNCH(launch_ex(bank.lq == 4 ? k_cwt_synthesis<4> : k_cwt_synthesis<0>, grid_of(M, 4 * B), blk, st, true, ll, lps, sl, in, NN, N, dst, mm, M, M,
+                             bank, stop, pb),
+                   "k_cwt_synthesis");
         ll = dst;
         lps = mm;
         sl = M;
     }
-    k_cwt_synthesis_sum<<<grid_of(N, B), blk, 0, st>>>(ll, lps, sl, in, NN, N, out, N, bank, stop, pb);
-    PAT_LAUNCH_CHECK("k_cwt_synthesis_sum");
+    CWT_LAUNCH(launch_ex(bank.l1 == 4 ? k_cwt_synthesis_sum<4> : k_cwt_synthesis_sum<0>, grid_of(N, B), blk, st, true, ll, lps, sl, in, NN, N, out, N, bank, stop, pb),
+               "k_cwt_synthesis_sum");
     return PAT_OK;
 }
 
 int launch_cwt_dual(float* r, const float* T, const float* sig_r, const float* step_mul, const float* scal, int N,
-                    int levels, const int* stop, cudaStream_t st, int B, long long pb) {
+                    int levels, const int* stop, cudaStream_t st, int B, long long pb, float* T_r) {
     const long long NN = (long long)N * N;
-    k_cwt_dual<<<dim3((unsigned)ceil_div(NN, 256), B), 256, 0, st>>>(r, T, sig_r, step_mul, scal, N, N >> levels,
-                                                                     stop, pb);
-    PAT_LAUNCH_CHECK("k_cwt_dual");
-    return PAT_OK;
-}
-
-int launch_cwt_uncombine(const float* r, float* T, int N, int levels, const int* stop, cudaStream_t st, int B,
-                         long long pb) {
-    const long long NN = (long long)N * N;
-    k_cwt_uncombine<<<dim3((unsigned)ceil_div(NN, 256), B), 256, 0, st>>>(r, T, N, N >> levels, stop, pb);
-    PAT_LAUNCH_CHECK("k_cwt_uncombine");
+    CWT_LAUNCH(launch_ex(k_cwt_dual, dim3((unsigned)ceil_div(NN, 256), B), dim3(256), st, true, r, T, sig_r, step_mul, scal,
+                         N, N >> levels, stop, pb, T_r),
+               "k_cwt_dual");
     return PAT_OK;
 }
 
@@ -525,10 +631,12 @@ extern "C" int pat_dtcwt_transform(int n, int levels, const double* h1_host, int
     float* T = buf;
     float* scratch = buf + 4 * NN;
     if (inverse) {
-        rc = launch_cwt_uncombine(in_dev, T, n, levels, nullptr, st, 1, 0);
+        k_cwt_uncombine<<<(unsigned)ceil_div(NN, 256), 256, 0, st>>>(in_dev, T, n, n >> levels);
+        count_launch();
+        if (cudaGetLastError() != cudaSuccess) rc = fail(PAT_ERR_CUDA, "k_cwt_uncombine");
         if (!rc) rc = launch_cwt_synthesis(T, n, levels, bank, out_dev, scratch, nullptr, st, 1, 0);
     } else {
-        rc = launch_cwt_analysis(in_dev, n, levels, bank, T, scratch, nullptr, st, 1, 0);
+        rc = launch_cwt_analysis(in_dev, n, levels, bank, T, scratch, nullptr, st, 1, 0, false);
         if (!rc) {
             k_cwt_combine<<<(unsigned)ceil_div(NN, 256), 256, 0, st>>>(T, out_dev, n, n >> levels);
             count_launch();

@@ -277,6 +277,20 @@ inline void set_dependent_launch(cudaLaunchAttribute& attr) {
     attr.val.programmaticStreamSerializationAllowed = 1;
 }
 inline int ceil_div(long long a, long long b) { return (int)((a + b - 1) / b); }
+// kernel<<<grid, block, 0, st>>>(args...); dep: it calls await_predecessor and may start on its
+// predecessor's tail
+template <class... P, class... A>
+inline cudaError_t launch_ex(void (*kernel)(P...), dim3 grid, dim3 block, cudaStream_t st, bool dep, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    set_dependent_launch(attr[0]);
+    cfg.attrs = attr;
+    cfg.numAttrs = dep ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 // p moved on by b bytes: problem k of a batch whose per-problem buffers lie a fixed byte
 // stride apart reads its buffers at the first problem's pointers plus k times that stride
@@ -416,17 +430,17 @@ struct CwtGapArgs {
 };
 int cwt_bank(const double* h1, int l1, const double* hq, int lq, CwtBank& bank, std::vector<double>* h1_out,
              std::vector<double>* hq_out);
-void cwt_abs_sums(int n, int levels, const std::vector<double>& h1, const std::vector<double>& hq,
-                  std::vector<double>& rows, std::vector<double>& cols);
+void cwt_abs_tables(int n, int levels, const std::vector<double>& h1, const std::vector<double>& hq,
+                    std::vector<double>& rows, std::vector<double>& fold);
+int launch_cwt_steps(const float* sig_tab, const double* fold, const float* kcol, int N, int levels, float* sig_r,
+                     float* tau, cudaStream_t st);
 // the DT-CWT's T planes (analysis) and its transpose; scratch: 5 N^2 / 4 floats per problem
 int launch_cwt_analysis(const float* in, int N, int levels, const CwtBank& bank, float* out, float* scratch,
-                        const int* stop, cudaStream_t st, int B, long long ps);
+                        const int* stop, cudaStream_t st, int B, long long ps, bool dep);
 int launch_cwt_synthesis(float* in, int N, int levels, const CwtBank& bank, float* out, float* scratch,
                          const int* stop, cudaStream_t st, int B, long long ps);
 int launch_cwt_dual(float* r, const float* T, const float* sig_r, const float* step_mul, const float* scal, int N,
-                    int levels, const int* stop, cudaStream_t st, int B, long long ps);
-int launch_cwt_uncombine(const float* r, float* T, int N, int levels, const int* stop, cudaStream_t st, int B,
-                         long long ps);
+                    int levels, const int* stop, cudaStream_t st, int B, long long ps, float* T_r);
 int launch_cwt_gap_pixels(const CwtGapArgs& a, int nblocks, cudaStream_t st, int B, long long ps);
 // the orthonormal Daubechies-4 transform (wavelet.cu)
 bool wav_levels_ok(int n, int levels);

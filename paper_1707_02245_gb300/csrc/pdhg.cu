@@ -1134,8 +1134,8 @@ struct WavModel {
     long long nr = 0;
     CwtBank bank{};
     std::vector<double> h1, hq;
-    // the |W| row sums (with the DT-CWT, paired per complex coefficient) and column sums,
-    // filled by the first wav_steps call and shared by the problems of a batch
+    // the |W| row sums and column sums (with the DT-CWT the tables of cwt_abs_tables, rows
+    // paired per complex coefficient), filled by the first wav_steps call and shared by the problems of a batch
     std::vector<double> rows, cols;
 };
 
@@ -1172,16 +1172,11 @@ static int wav_steps(const pat_geometry* g, WavModel& m, float* sig_q, float* ta
     if (rc) return rc;
     std::vector<double>& rows = m.rows;
     std::vector<double>& cols = m.cols;
-    if (rows.empty() && m.kind == PAT_WAVELET_DTCWT) {
-        cwt_abs_sums(N, m.J, m.h1, m.hq, rows, cols);
-        const int side = N >> m.J;
-        for (long long i = 0; i < NN; ++i) {
-            if ((int)(i % N) < side && (int)(i / N) < side) continue;   // LL: one row each
-            for (int a = 0; a < 4; a += 2) {
-                const double mx = std::max(rows[a * NN + i], rows[(a + 1) * NN + i]);
-                rows[a * NN + i] = rows[(a + 1) * NN + i] = mx;
-            }
-        }
+    const bool cwt = m.kind == PAT_WAVELET_DTCWT;
+    if (rows.empty() && cwt) {
+        cwt_abs_tables(N, m.J, m.h1, m.hq, rows, cols);
+        for (size_t b = 0; b + 4 < rows.size(); b += 4)   // (not LL, the last: one row each)
+            for (int a = 0; a < 4; a += 2) rows[b + a] = rows[b + a + 1] = std::max(rows[b + a], rows[b + a + 1]);
     } else if (rows.empty()) {
         wav_abs_sums(N, m.J, rows, cols);
     }
@@ -1193,7 +1188,19 @@ static int wav_steps(const pat_geometry* g, WavModel& m, float* sig_q, float* ta
             PAT_LAUNCH_CHECK("k_scale_f32");
         }
     }
-    if (tau_u) {
+    if (cwt && (tau_u || sig_r)) {
+        std::vector<float> sig(rows.size());
+        for (size_t k = 0; k < rows.size(); ++k) sig[k] = rows[k] > 0 ? (float)(1.0 / rows[k] / s_ratio) : 1.f;
+        char* tab = nullptr;   // the column table, then the steps (copies from pageable memory are staged before they return)
+        const size_t fb = cols.size() * sizeof(double), sb = sig.size() * sizeof(float);
+        PAT_CUDA(cudaMallocAsync((void**)&tab, fb + sb, st));
+        cudaError_t e = cudaMemcpyAsync(tab, cols.data(), fb, cudaMemcpyHostToDevice, st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(tab + fb, sig.data(), sb, cudaMemcpyHostToDevice, st);
+        rc = e == cudaSuccess ? launch_cwt_steps((const float*)(tab + fb), (const double*)tab, g->pc.kcol, N, m.J, sig_r, tau_u, st)
+                              : cuda_fail(e, "wav_steps: copy");
+        cudaFreeAsync(tab, st);
+        if (rc) return rc;
+    } else if (tau_u) {
         double* wcol = nullptr;
         PAT_CUDA(cudaMallocAsync(&wcol, NN * sizeof(double), st));
         rc = cudaMemcpyAsync(wcol, cols.data(), NN * sizeof(double), cudaMemcpyHostToDevice, st) == cudaSuccess
@@ -1202,12 +1209,12 @@ static int wav_steps(const pat_geometry* g, WavModel& m, float* sig_q, float* ta
         if (!rc) PAT_CUDA(cudaStreamSynchronize(st));   // the host vector dies with this call
         cudaFreeAsync(wcol, st);
         if (rc) return rc;
-        if (s_ratio != 1.0) {
-            k_scale_f32<<<ceil_div(NN, 256), 256, 0, st>>>(tau_u, NN, (float)s_ratio);
-            PAT_LAUNCH_CHECK("k_scale_f32");
-        }
     }
-    if (sig_r) {
+    if (tau_u && s_ratio != 1.0) {
+        k_scale_f32<<<ceil_div(NN, 256), 256, 0, st>>>(tau_u, NN, (float)s_ratio);
+        PAT_LAUNCH_CHECK("k_scale_f32");
+    }
+    if (sig_r && !cwt) {
         std::vector<float> h((size_t)m.nr);
         for (long long i = 0; i < m.nr; ++i) h[i] = rows[i] > 0 ? (float)(1.0 / rows[i] / s_ratio) : 1.f;
         PAT_CUDA(cudaMemcpyAsync(sig_r, h.data(), m.nr * sizeof(float), cudaMemcpyHostToDevice, st));
@@ -1362,8 +1369,8 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
         const int par = it & 1;
         int e = launch_forward_groups(FWD_PROX, (const FwdArgs*)(base + fw_off[par]), gp, base, s);
         if (cwt) {
-            if (!e) e = launch_cwt_analysis(ubar, N, J, wm.bank, wb, scr, &in->stop, s, B, ps);
-            if (!e) e = launch_cwt_dual(r, wb, sigr, in->step_mul, scal, N, J, &in->stop, s, B, ps);
+            if (!e) e = launch_cwt_analysis(ubar, N, J, wm.bank, wb, scr, &in->stop, s, B, ps, true);
+            if (!e) e = launch_cwt_dual(r, wb, sigr, in->step_mul, scal, N, J, &in->stop, s, B, ps, scrt);
         } else {
             if (!e) e = launch_wav_analysis(ubar, N, J, wb, scr, &in->stop, s, B, ps);
             if (!e) e = launch_wav_dual(r, wb, sigr, in->step_mul, scal, NN, &in->stop, s, B, ps);
@@ -1371,7 +1378,6 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
         if (!e)
             e = launch_adjoint_b((const AdjArgs*)(base + ad_off[par]), (const int2*)(base + amap_off), n_adj, true, s);
         if (cwt) {
-            if (!e) e = launch_cwt_uncombine(r, scrt, N, J, &in->stop, s, B, ps);
             if (!e) e = launch_cwt_synthesis(scrt, N, J, wm.bank, wtr, scr, &in->stop, s, B, ps);
         } else {
             if (!e) e = launch_wav_synthesis(r, N, J, wtr, scr, &in->stop, s, B, ps);
@@ -1392,7 +1398,7 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
         pa.iter = &in->iter;
         if (!e) e = launch_wav_primal(pa, s, B, ps);
         if (gap && !e) {
-            e = cwt ? launch_cwt_analysis(u, N, J, wm.bank, wu, scr2, &in->stop, s, B, ps)
+            e = cwt ? launch_cwt_analysis(u, N, J, wm.bank, wu, scr2, &in->stop, s, B, ps, true)
                     : launch_wav_analysis(u, N, J, wu, scr2, &in->stop, s, B, ps);
             if (!e) e = launch_forward_groups(FWD_GAP, (const FwdArgs*)(base + fg_off), gp, base, s);
             if (cwt) {

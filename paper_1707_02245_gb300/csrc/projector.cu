@@ -196,9 +196,8 @@ __host__ __device__ __forceinline__ FwdSmem fwd_smem_layout(int rows, int stride
     return l;
 }
 
-// cluster helpers: rank in the cluster, barrier over the cluster's CTAs (orders shared
-// memory writes before the barrier with reads after it), and a load from the shared
-// memory of CTA `rank` at the offset of the local address p
+// Rank in the cluster, and a barrier over the cluster's CTAs that orders memory writes before
+// it with reads after it.
 __device__ __forceinline__ unsigned cluster_rank() {
     unsigned r;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -207,6 +206,7 @@ __device__ __forceinline__ unsigned cluster_rank() {
 __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
+// A load from the shared memory of CTA `rank` at the offset of the local address p.
 __device__ __forceinline__ float ld_cluster(const float* p, unsigned rank) {
     unsigned a = smem_addr(p), ra;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(a), "r"(rank));

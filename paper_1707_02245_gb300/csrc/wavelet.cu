@@ -122,6 +122,9 @@ __global__ void k_wav_primal(WavPrimalArgs a, long long ps) {
     a.qmax_next = at_bytes(a.qmax_next, po);
     if (a.stop) a.stop = at_bytes(a.stop, po);
     if (a.iter) a.iter = at_bytes(a.iter, po);
+    await_predecessor();
+    a.kt.acc = after_wait(a.kt.acc);
+    a.wtr = after_wait(a.wtr);
     if (a.stop && *(volatile const int*)a.stop) return;
     const int N = a.n;
     const int gx = blockIdx.x * blockDim.x + threadIdx.x, gy = blockIdx.y * blockDim.y + threadIdx.y;
@@ -305,8 +308,9 @@ int launch_wav_dual(float* r, const float* wub, const float* sig_r, const float*
 }
 
 int launch_wav_primal(const WavPrimalArgs& a, cudaStream_t st, int B, long long ps) {
-    k_wav_primal<<<dim3(ceil_div(a.n, 32), ceil_div(a.n, 8), B), dim3(32, 8), 0, st>>>(a, ps);
-    PAT_LAUNCH_CHECK("k_wav_primal");
+    const cudaError_t e = launch_ex(k_wav_primal, dim3(ceil_div(a.n, 32), ceil_div(a.n, 8), B), dim3(32, 8), st, true, a, ps);
+    count_launch();
+    if (e != cudaSuccess) return cuda_fail(e, "k_wav_primal");
     return PAT_OK;
 }
 
