@@ -3,7 +3,10 @@
 // The forward pass (also the data gradient, with flipped weights) is an implicit GEMM with
 // M = pixels, N = output channels, K = 9 * input channels ordered (tap, channel), channels
 // innermost; a 16-byte vector of 8 channels never straddles a tap because the channel
-// counts are multiples of 8.  It has two kernels, chosen by shape:
+// counts are multiples of 8.  It has three kernels, chosen by shape; all
+// accumulate in the same order and give the same bits:
+//  - k_conv_halo (32, 64 or 96 input channels on wide images): tcgen05.mma on pixel tiles
+//    staged once with their halo, the weights resident (described at the kernel);
 //  - k_conv_fwd_tc (64 or more input channels, or 32 in and more than 32 out): TMA boxes
 //    into swizzled shared memory, tcgen05.mma with the accumulator in tensor memory,
 //    warp-specialised and persistent (described at the kernel);
@@ -251,6 +254,11 @@ constexpr long long T_WAIT_CYCLES = 2000000000LL;   // about 1 s at 2 GHz
 
 __device__ unsigned int g_tc_timeouts;
 
+// whether FP32 outputs can be stored 32 bytes at a time
+inline int wide_stores(const FwdArgs& f) {
+    return f.y32 && (reinterpret_cast<uintptr_t>(f.y32) & 31) == 0 && f.y_ps % 8 == 0 ? 1 : 0;
+}
+
 struct TcArgs {
     int B, H, W, cin, cout, relu;
     int bx_log2, by;        // tile: 2^bx_log2 x by pixels
@@ -259,7 +267,7 @@ struct TcArgs {
     const float* bias;
     bf16* y;
     float* y32;
-    int y_ps;
+    int y_ps, w32;
 };
 
 template <int BN>
@@ -283,19 +291,25 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
 }
 
-// waits for the completion of phase `parity` of the barrier; false after the time limit
+// whether phase `parity` of the barrier is complete (the instruction may wait a little)
+__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
+    uint32_t done;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+
+// waits for the completion of phase `parity` of the barrier; false after the time limit.  The
+// clock is read only once the phase was found incomplete.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    if (mbar_try(bar, parity)) return true;
     const long long t0 = clock64();
-    while (true) {
-        uint32_t done;
-        asm volatile(
-            "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(bar), "r"(parity)
-            : "memory");
-        if (done) return true;
+    while (!mbar_try(bar, parity))
         if (clock64() - t0 > T_WAIT_CYCLES) return false;
-    }
+    return true;
 }
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, int c0, int c1, int c2, int c3,
@@ -375,6 +389,39 @@ __device__ __forceinline__ TcTile tc_tile(const TcArgs& a, int t, int BN) {
     q.n = r / a.tiles_y;
     q.n0 = nt * BN;
     return q;
+}
+
+// eight output channels of a pixel: bias (8 values or NULL), ReLU and a 16- or 32-byte store at
+// element i (w32: y32 and its pixels lie on 32-byte boundaries, so that a lane's store is a whole
+// sector)
+template <bool F32>
+__device__ __forceinline__ void store8(const float* v, const float* bias, int relu, bf16* y, float* y32, long long i, int w32) {
+    float w[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        w[e] = v[e] + (bias ? bias[e] : 0.f);
+        if (relu) w[e] = fmaxf(w[e], 0.f);
+    }
+    if (F32) {
+        if (w32) {
+            asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n" ::"l"(y32 + i), "f"(w[0]), "f"(w[1]),
+                         "f"(w[2]), "f"(w[3]), "f"(w[4]), "f"(w[5]), "f"(w[6]), "f"(w[7])
+                         : "memory");
+            return;
+        }
+        float4* dst = reinterpret_cast<float4*>(y32 + i);
+        dst[0] = make_float4(w[0], w[1], w[2], w[3]);
+        dst[1] = make_float4(w[4], w[5], w[6], w[7]);
+    } else {
+        uint4 u;
+        __nv_bfloat162 t0 = __floats2bfloat162_rn(w[0], w[1]), t1 = __floats2bfloat162_rn(w[2], w[3]);
+        __nv_bfloat162 t2 = __floats2bfloat162_rn(w[4], w[5]), t3 = __floats2bfloat162_rn(w[6], w[7]);
+        u.x = *reinterpret_cast<uint32_t*>(&t0);
+        u.y = *reinterpret_cast<uint32_t*>(&t1);
+        u.z = *reinterpret_cast<uint32_t*>(&t2);
+        u.w = *reinterpret_cast<uint32_t*>(&t3);
+        *reinterpret_cast<uint4*>(y + i) = u;
+    }
 }
 
 template <int BN, bool F32>
@@ -545,26 +592,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 for (int h = 0; h < 2; ++h) {
                     const int o = q.n0 + cb16 * 16 + 8 * h;
                     if (o >= a.cout) continue;   // cout is a multiple of 8
-                    float w[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        w[e] = v[8 * h + e] + (a.bias ? __ldg(a.bias + o + e) : 0.f);
-                        if (a.relu) w[e] = fmaxf(w[e], 0.f);
-                    }
-                    if (F32) {
-                        float4* dst = reinterpret_cast<float4*>(a.y32 + pp * a.y_ps + o);
-                        dst[0] = make_float4(w[0], w[1], w[2], w[3]);
-                        dst[1] = make_float4(w[4], w[5], w[6], w[7]);
-                    } else {
-                        uint4 u;
-                        __nv_bfloat162 t0 = __floats2bfloat162_rn(w[0], w[1]), t1 = __floats2bfloat162_rn(w[2], w[3]);
-                        __nv_bfloat162 t2 = __floats2bfloat162_rn(w[4], w[5]), t3 = __floats2bfloat162_rn(w[6], w[7]);
-                        u.x = *reinterpret_cast<uint32_t*>(&t0);
-                        u.y = *reinterpret_cast<uint32_t*>(&t1);
-                        u.z = *reinterpret_cast<uint32_t*>(&t2);
-                        u.w = *reinterpret_cast<uint32_t*>(&t3);
-                        *reinterpret_cast<uint4*>(a.y + pp * a.y_ps + o) = u;
-                    }
+                    store8<F32>(v + 8 * h, a.bias ? a.bias + o : nullptr, a.relu, a.y, a.y32, pp * a.y_ps + o, a.w32);
                 }
             }
             tc_fence_before();
@@ -577,6 +605,212 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     if (warp == 1) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(C::NCOLS) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// forward on tcgen05 with the taps taken from one halo tile: what bounds k_conv_fwd_tc on wide
+// images is the L2 -> SM traffic of reading every pixel nine times and the weights once per
+// tile (6-9 TB/s measured).  Here a CTA keeps the weights of its N tile in shared memory for
+// all its pixel tiles, and a pixel tile of 8 x 16 is staged once with its one-pixel halo, as
+// TMA boxes {CB channels, 10, 18, 1} swizzled by the row size.  A tile row of 8 pixels is one
+// 8-row group of the MMA's A operand (SBO = a halo row of 10 pixels), and a tap is the same
+// descriptor moved by 10 dy + dx pixel rows: the swizzle is a function of the address, so the
+// moved rows are read as TMA wrote them.  MMAs run in the order (tap, channel) of the other
+// kernels, so the sums have the same bits.  (Rows of 16 bytes without swizzle need no such
+// argument, but their MMAs took 240 clocks each instead of 46-64.)
+//   Warp 0 is the TMA producer, warp 1 issues the MMAs, warps 2-9 drain the accumulators;
+// waits are bounded as in k_conv_fwd_tc.
+//   Measured, batch 8, FP32 output, us per call (before): 256^2 32 -> 32 35 (82), 96 -> 32 70
+// (190), 32 -> 96 58 (142); 128^2 64 -> 64 18.5 (31), 64 -> 192 35 (103), 824 TFLOP/s.  The
+// narrow layers are now bound by one thread's issue of N = 32 MMAs (46 clocks each) and the
+// waits between tiles, the wide ones by the FP32 stores.
+// ---------------------------------------------------------------------------------------
+constexpr int HTX = 8, HTY = 16;                       // pixel tile
+constexpr int HPX = HTX + 2, HPY = HTY + 2;            // with its halo
+constexpr int H_THREADS = 320;
+constexpr int H_MAX_STAGES = 4, H_NACC = 4;
+constexpr int H_SMEM = 224 * 1024;                     // shared memory a CTA may take
+static_assert(HTX * HTY == TBM && HTX == 8, "a tile row is an 8-row group");
+
+struct HaloArgs {
+    int B, H, W, cin, cout, relu;
+    const float* bias;
+    bf16* y;
+    float* y32;
+    int y_ps, w32;
+    int bn, tiles_n, tiles_x, tiles_y, tiles, stages;
+};
+
+constexpr int halo_region(int cb) { return (HPX * HPY * cb * 2 + 1023) / 1024 * 1024; }   // a box of the halo, 1024-byte aligned
+constexpr int halo_smem(int cin, int cb, int bn, int stages) {
+    return 9 * cin * bn * 2 + stages * (cin / cb) * halo_region(cb) + 8 * (2 * H_MAX_STAGES + 2 * H_NACC + 2) + 16 + bn * 4 + 1024;
+}
+
+// CB: channels per box, NQ: boxes per halo tile (cin = CB NQ)
+template <bool F32, int CB, int NQ>
+__global__ void __launch_bounds__(H_THREADS, 1)
+    k_conv_halo(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const HaloArgs a) {
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    constexpr uint32_t a_reg = (uint32_t)halo_region(CB), stage_bytes = NQ * a_reg;
+    const uint32_t b_reg = (uint32_t)(a.bn * CB * 2);
+    const uint32_t sB = smem_u32(smem), sA = sB + 9u * NQ * b_reg;
+    const uint32_t bars = sA + (uint32_t)a.stages * stage_bytes;
+    auto full = [&](int s) { return bars + 8u * s; };
+    auto empty = [&](int s) { return bars + 8u * (H_MAX_STAGES + s); };
+    auto accf = [&](int b) { return bars + 8u * (2 * H_MAX_STAGES + b); };
+    auto acce = [&](int b) { return bars + 8u * (2 * H_MAX_STAGES + H_NACC + b); };
+    const uint32_t fin = bars + 8u * (2 * H_MAX_STAGES + 2 * H_NACC), wfull = fin + 8u;
+    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + (wfull + 8u - sB));
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(slot + 1);
+    float* s_bias = reinterpret_cast<float*>(slot + 4);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int n0 = ((int)blockIdx.x % a.tiles_n) * a.bn;
+    const int t_first = (int)blockIdx.x / a.tiles_n, t_step = (int)gridDim.x / a.tiles_n;
+
+    if (tid == 0) {
+        for (int s = 0; s < a.stages; ++s) {
+            mbar_init(full(s), 1);
+            mbar_init(empty(s), 1);
+        }
+        for (int b = 0; b < H_NACC; ++b) {
+            mbar_init(accf(b), 1);
+            mbar_init(acce(b), 8);   // one arrival per epilogue warp
+        }
+        mbar_init(fin, 1);
+        mbar_init(wfull, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    for (int o = tid; o < a.bn; o += H_THREADS) s_bias[o] = a.bias && n0 + o < a.cout ? __ldg(a.bias + n0 + o) : 0.f;
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(slot)), "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *slot;
+    auto give_up = [&]() {
+        *abort_flag = 1;
+        atomicAdd(&g_tc_timeouts, 1u);
+    };
+    auto tile_of = [&](int t, int& n, int& x0, int& y0) {
+        const int tx = t % a.tiles_x, r = t / a.tiles_x;
+        x0 = tx * HTX;
+        y0 = (r % a.tiles_y) * HTY;
+        n = r / a.tiles_y;
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---- TMA producer: the weights once, then one halo tile per stage ----
+            mbar_expect_tx(wfull, 9u * NQ * b_reg);
+            for (int q = 0; q < 9 * NQ; ++q) tma_load_2d(sB + q * b_reg, &tmB, q * CB, n0, wfull);   // o >= cout: zero fill
+            int it = 0;
+            for (int t = t_first; t < a.tiles && !*abort_flag; t += t_step, ++it) {
+                const int s = it % a.stages;
+                if (!mbar_wait(empty(s), ((it / a.stages) & 1) ^ 1)) {
+                    give_up();
+                    break;
+                }
+                mbar_expect_tx(full(s), (uint32_t)(HPX * HPY * CB * NQ * 2));
+                int n, x0, y0;
+                tile_of(t, n, x0, y0);
+                for (int q = 0; q < NQ; ++q)   // outside the image: zero fill
+                    tma_load_4d(sA + s * stage_bytes + q * a_reg, &tmA, q * CB, x0 - 1, y0 - 1, n, full(s));
+            }
+            // every copy issued has landed before the CTA may end (bounded)
+            if (!mbar_wait(wfull, 0)) give_up();
+            for (int j = it - 1; j >= 0 && j >= it - a.stages; --j)
+                if (!mbar_wait(full(j % a.stages), (j / a.stages) & 1)) {
+                    give_up();
+                    break;
+                }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            // ---- MMA issuer ----
+            const uint32_t idesc = tc_idesc(TBM, a.bn);
+            constexpr uint32_t layout = CB == 16 ? 6u : CB == 32 ? 4u : 2u;
+            constexpr uint32_t row = CB * 2;   // bytes of a pixel (and of an output channel) in a box
+            const uint64_t da = tc_desc(0, 16, HPX * row, layout), db = tc_desc(0, 16, 8 * row, layout) + (sB >> 4);
+            const uint32_t b16 = b_reg >> 4;
+            int it = 0;
+            const bool ok = mbar_wait(wfull, 0);
+            if (!ok) give_up();
+            for (int t = t_first; t < a.tiles && ok && !*abort_flag; t += t_step, ++it) {
+                const int b = it % H_NACC, s = it % a.stages;
+                if (!mbar_wait(acce(b), ((it / H_NACC) & 1) ^ 1) || !mbar_wait(full(s), (it / a.stages) & 1)) {
+                    give_up();
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t d = tmem + (uint32_t)(b * TBM);   // accumulators 128 columns apart
+                const uint64_t dt = da + ((sA + s * stage_bytes) >> 4);
+                // unrolled: one thread issues, and with loop arithmetic between them its MMAs
+                // came 200 clocks apart
+#pragma unroll
+                for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q)
+#pragma unroll
+                        for (int e = 0; e < CB / 16; ++e)   // 16 channels
+                            tc_mma(d, dt + (((tap / 3) * HPX + tap % 3) * row + q * a_reg + e * 32) / 16,
+                                   db + (uint64_t)((tap * NQ + q) * b16 + e * 2), idesc, (tap | q | e) != 0);
+                tc_commit(empty(s));
+                tc_commit(accf(b));
+            }
+            // every MMA issued has finished before the tensor memory is freed (bounded)
+            tc_commit(fin);
+            if (!mbar_wait(fin, 0)) give_up();
+        }
+    } else {
+        // ---- epilogue: warps 2..9; TMEM lane = pixel 8 ly + lx of the tile; the two warps of a
+        // quarter take alternate 16 columns ----
+        const int quarter = warp & 3, half = (warp - 2) >> 2, row = quarter * 32 + lane;
+        const int ly = row / HTX, lx = row % HTX;
+        const uint32_t tl_lane = tmem + ((uint32_t)(quarter * 32) << 16);
+        int it = 0;
+        for (int t = t_first; t < a.tiles; t += t_step, ++it) {
+            const int b = it % H_NACC;
+            int ok = 0;
+            if (lane == 0) ok = mbar_wait(accf(b), (it / H_NACC) & 1) ? 1 : 0;
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            if (!ok) {
+                if (lane == 0) give_up();
+                break;
+            }
+            tc_fence_after();
+            int n, x0, y0;
+            tile_of(t, n, x0, y0);
+            const int y = y0 + ly, x = x0 + lx;
+            const bool valid = y < a.H && x < a.W;
+            const long long pp = ((long long)n * a.H + y) * a.W + x;
+            for (int c16 = 16 * half; c16 < a.bn; c16 += 32) {
+                float v[16];
+                __syncwarp();
+                tc_ld16(tl_lane + (uint32_t)(b * TBM + c16), v);
+                if (!valid) continue;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int o = n0 + c16 + 8 * h;
+                    if (o >= a.cout) continue;   // cout is a multiple of 8
+                    store8<F32>(v + 8 * h, s_bias + c16 + 8 * h, a.relu, a.y, a.y32, pp * a.y_ps + o, a.w32);
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acce(b));
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u) : "memory");
     }
 }
 
@@ -1110,6 +1344,7 @@ int launch_fwd_tc(const FwdArgs& f, cudaStream_t st) {
     a.y = f.y;
     a.y32 = f.y32;
     a.y_ps = f.y_ps;
+    a.w32 = wide_stores(f);
     const CUtensorMapSwizzle sw = a.cb == 64   ? CU_TENSOR_MAP_SWIZZLE_128B
                                   : a.cb == 32 ? CU_TENSOR_MAP_SWIZZLE_64B
                                   : a.cb == 16 ? CU_TENSOR_MAP_SWIZZLE_32B
@@ -1140,6 +1375,86 @@ int launch_fwd_tc(const FwdArgs& f, cudaStream_t st) {
     k_conv_fwd_tc<BN, F32><<<grid, TC_THREADS, C::SMEM, st>>>(ma, mb, a);
     PAT_LAUNCH_CHECK("k_conv_fwd_tc");
     return PAT_OK;
+}
+
+constexpr int HALO_MIN_TILES = 2;   // work tiles per SM (64 -> 64 channels, batch 8: 18.5 against 30.9 us at 128^2, 10.9 against 11.3 at 32^2)
+// channels per box
+constexpr int halo_cb(int cin) { return cin == 64 ? 64 : 32; }
+
+// The halo kernel's plan for a layer; false where another kernel is the better one.
+//  - cin of 32, 64 or 96, whose halo fits two stages beside the weights of an N tile: the
+//    widest N of 128, 96, 64, 32 that pads cout least.
+//  - enough pixel tiles that the weights' load is paid for.
+bool plan_halo(const FwdArgs& f, HaloArgs& a) {
+    if (f.cin != 32 && f.cin != 64 && f.cin != 96) return false;
+    const int cb = halo_cb(f.cin);
+    a.tiles_x = (f.W + HTX - 1) / HTX;
+    a.tiles_y = (f.H + HTY - 1) / HTY;
+    const long long tiles = (long long)f.B * a.tiles_x * a.tiles_y;
+    int best = 0;
+    for (int bn : {128, 96, 64, 32}) {
+        if (halo_smem(f.cin, cb, bn, 2) > H_SMEM) continue;
+        auto padded = [&](int n) { return (f.cout + n - 1) / n * n; };
+        if (!best || padded(bn) < padded(best)) best = bn;
+    }
+    if (!best) return false;
+    a.bn = best;
+    a.tiles_n = (f.cout + best - 1) / best;
+    if (a.tiles_n > sm_count() || tiles * a.tiles_n < HALO_MIN_TILES * sm_count() || tiles > (1LL << 30)) return false;
+    a.tiles = (int)tiles;
+    a.stages = 2;
+    while (a.stages < H_MAX_STAGES && halo_smem(f.cin, cb, best, a.stages + 1) <= H_SMEM) ++a.stages;
+    a.B = f.B;
+    a.H = f.H;
+    a.W = f.W;
+    a.cin = f.cin;
+    a.cout = f.cout;
+    a.relu = f.relu;
+    a.bias = f.bias;
+    a.y = f.y;
+    a.y32 = f.y32;
+    a.y_ps = f.y_ps;
+    a.w32 = wide_stores(f);
+    return true;
+}
+
+template <bool F32, int CB, int NQ>
+int launch_halo_cin(const FwdArgs& f, const HaloArgs& a, cudaStream_t st) {
+    const EncodeTiledFn enc = encode_tiled();
+    if (!enc) return fail(PAT_ERR_CUDA, "conv3x3: cuTensorMapEncodeTiled is not available");
+    const CUtensorMapSwizzle sw = CB == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
+    CUtensorMap ma, mb;
+    const cuuint64_t ps = (cuuint64_t)f.x_ps * 2;
+    const cuuint64_t dA[4] = {(cuuint64_t)f.cin, (cuuint64_t)f.W, (cuuint64_t)f.H, (cuuint64_t)f.B};
+    const cuuint64_t sA[3] = {ps, ps * f.W, ps * f.W * f.H};
+    const cuuint32_t bA[4] = {(cuuint32_t)CB, HPX, HPY, 1};
+    const cuuint32_t es[4] = {1, 1, 1, 1};
+    CUresult r = enc(&ma, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)f.x, dA, sA, bA, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                     sw, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3: activation tensor map");
+    const int K = 9 * f.cin;
+    const cuuint64_t dB[2] = {(cuuint64_t)K, (cuuint64_t)f.cout};
+    const cuuint64_t sB[1] = {(cuuint64_t)K * 2};
+    const cuuint32_t bB[2] = {(cuuint32_t)CB, (cuuint32_t)a.bn};
+    r = enc(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)f.w, dB, sB, bB, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
+            CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    if (r != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3: weight tensor map");
+    // a host-side attribute of the function (allowed under graph capture), set once
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_conv_halo<F32, CB, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, H_SMEM);
+    PAT_CUDA(attr);
+    const int per = std::min(std::max(1, sm_count() / a.tiles_n), a.tiles);   // CTAs of one N tile
+    k_conv_halo<F32, CB, NQ><<<per * a.tiles_n, H_THREADS, halo_smem(CB * NQ, CB, a.bn, a.stages), st>>>(ma, mb, a);
+    PAT_LAUNCH_CHECK("k_conv_halo");
+    return PAT_OK;
+}
+
+template <bool F32>
+int launch_halo(const FwdArgs& f, const HaloArgs& a, cudaStream_t st) {
+    static_assert(halo_cb(32) == 32 && halo_cb(64) == 64 && halo_cb(96) == 32, "boxes of the plan");
+    if (f.cin == 32) return launch_halo_cin<F32, 32, 1>(f, a, st);
+    if (f.cin == 64) return launch_halo_cin<F32, 64, 1>(f, a, st);
+    return launch_halo_cin<F32, 32, 3>(f, a, st);
 }
 
 template <int BM>
@@ -1258,10 +1573,12 @@ int conv3x3_fwd(const View& x, int B, int H, int W, int cin, const bf16* w, cons
     a.cin = cin;
     a.cout = cout;
     a.relu = relu ? 1 : 0;
-    // The tensor-memory kernel wins where a pixel's channels fill 64-byte or 128-byte TMA
+    // The halo kernel where it applies.  Else the tensor-memory kernel wins where a pixel's channels fill 64-byte or 128-byte TMA
     // rows and the GEMM is wide enough (measured at batch 8: 1.6-2.5x for 64 or more input
     // channels); with 8-24 input channels, or 32 in and at most 32 out, the warp-level
     // kernel is as fast or faster (its loads are not bound by TMA's row rate).
+    HaloArgs h;
+    if (plan_halo(a, h)) return y_f32 ? launch_halo<true>(a, h, st) : launch_halo<false>(a, h, st);
     const bool tc = cin % 32 == 0 && (cin >= 64 || cout >= 64);
     if (y_f32) {
         if (cout <= 32) return tc ? launch_fwd_tc<32, true>(a, st) : launch_fwd<32, true>(a, st);
