@@ -12,8 +12,9 @@
 //    warp-specialised and persistent (described at the kernel);
 //  - k_conv_fwd (the narrow layers): a three-stage cp.async ring feeding mma.sync
 //    m16n8k16 through ldmatrix; out-of-image taps are zero-filled by the copy itself.
-// Weight gradient: k_conv_wgrad_tc (tcgen05; every layer with at most 256 output
-// channels, described at the kernel), else k_conv_wgrad (mma.sync: M = output channels,
+// Weight gradient: k_conv_wgrad_halo (tcgen05; the wide layers with up to 64, or 128, output
+// channels), k_conv_wgrad_tc (tcgen05; the others with at most 256 output channels; both
+// described at the kernel), else k_conv_wgrad (mma.sync: M = output channels,
 // N = (tap, input channel), K = pixels, the pixel-major operands transposed by
 // ldmatrix.trans).  Both split the pixels; each split writes its own partial tile, and a
 // second kernel sums the splits in a fixed order, so the result is deterministic.
@@ -1204,6 +1205,178 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     }
 }
 
+// ---------------------------------------------------------------------------------------
+// weight gradient of the wide layers with the taps taken from one halo tile: k_conv_wgrad_tc
+// reads x once per tap and the output gradient once per M tile from L2 (7 TB/s measured).
+// Here a pixel tile of 16 x 8 is staged once, x with its halo as a box {CB channels, 18, 10, 1},
+// dz as boxes of 16 x 8 pixels, and all nine taps of the CB channels accumulate at once:
+//  - K of an MMA is 16 pixels of an image row; both operands are MN-major as in
+//    k_conv_wgrad_tc, and a tap (dy, dx) is x's descriptor moved by 18 dy + dx pixel rows;
+//  - the 128 rows of an MMA are 128 / CB neighbouring dx: LBO, the step to the next channel
+//    box, is one pixel row.  So CB = 32 takes dx = 0..3 in one MMA, CB = 64 dx = 0, 1 and
+//    2, 3 in two; dx = 3 is computed and dropped;
+//  - the 3 (CB = 32) or 6 (CB = 64) accumulators of BN columns stay in tensor memory for all
+//    of a CTA's pixel tiles and are written once, to part[split][o][k].
+// A CTA is one (channel box, split of the pixel tiles); k_sum_splits adds the splits.
+// Measured, batch 8, us per call with its sums (k_conv_wgrad_tc): 256^2 32 -> 32 53 (113), 96 -> 32
+// 102 (273); 128^2 64 -> 64 42 (54), 192 -> 64 62 (126).  One thread issues the MMAs (46 clocks
+// at N = 32 and 64); the sums of splits and columns are 25 us of each call.
+// ---------------------------------------------------------------------------------------
+constexpr int GTX = 16, GTY = 8;                       // pixel tile
+constexpr int GPX = GTX + 2, GPY = GTY + 2;            // with its halo
+constexpr int G_MAX_STAGES = 6;
+
+struct WgHaloArgs {
+    int cin, cout, nq;                                 // nq: channel boxes of x
+    int tiles_x, tiles_y, tiles, per;                  // pixel tiles, and how many a CTA takes
+    float* part;
+};
+
+template <int CB, int BN>
+struct WgHaloCfg {
+    static constexpr int CBO = BN % 64 == 0 ? 64 : 32;                                  // channels per box of dz
+    static constexpr int MT = CB == 64 ? 2 : 1;                                         // MMAs per dy
+    static constexpr int A_BYTES = (GPX * GPY * CB * 2 + 1023) / 1024 * 1024;           // (dx = 3 reads at most one row past the box)
+    static constexpr int B_BYTES = GTX * GTY * BN * 2;
+    static constexpr int STAGE = A_BYTES + B_BYTES;
+    static constexpr int FIT = 220 * 1024 / STAGE;
+    static constexpr int STAGES = FIT < G_MAX_STAGES ? FIT : G_MAX_STAGES;
+    static constexpr int BAR_OFF = STAGES * STAGE;
+    static constexpr int SMEM = BAR_OFF + 8 * (2 * STAGES + 1) + 16 + 1024;
+    static constexpr int ACC = 3 * MT;
+    static_assert(ACC * BN <= 512 && STAGES >= 2 && GPX * GPY * CB * 2 + CB * 2 <= A_BYTES, "fits");
+};
+
+template <int CB, int BN>
+__global__ void __launch_bounds__(TC_THREADS, 1)
+    k_conv_wgrad_halo(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmD, const WgHaloArgs a) {
+    using C = WgHaloCfg<CB, BN>;
+    constexpr int S = C::STAGES, MT = C::MT;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const uint32_t sbase = smem_u32(smem);
+    const uint32_t bars = sbase + C::BAR_OFF;
+    auto full = [&](int s) { return bars + 8u * s; };
+    auto empty = [&](int s) { return bars + 8u * (S + s); };
+    const uint32_t fin = bars + 8u * (2 * S);
+    uint32_t* slot = reinterpret_cast<uint32_t*>(smem + C::BAR_OFF + 8 * (2 * S + 1));
+    volatile int* abort_flag = reinterpret_cast<volatile int*>(slot + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int q = (int)blockIdx.x % a.nq, z = (int)blockIdx.x / a.nq;
+    const int t0 = z * a.per, t1 = min(a.tiles, t0 + a.per);
+
+    if (tid == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(full(s), 1);
+            mbar_init(empty(s), 1);
+        }
+        mbar_init(fin, 1);
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(slot)), "r"(512u)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *slot;
+    auto give_up = [&]() {
+        *abort_flag = 1;
+        atomicAdd(&g_tc_timeouts, 1u);
+    };
+
+    if (warp == 0) {
+        if (lane == 0) {
+            // ---- TMA producer ----
+            int it = 0;
+            for (int t = t0; t < t1 && !*abort_flag; ++t, ++it) {
+                const int s = it % S;
+                if (!mbar_wait(empty(s), ((it / S) & 1) ^ 1)) {
+                    give_up();
+                    break;
+                }
+                mbar_expect_tx(full(s), (uint32_t)(GPX * GPY * CB * 2 + C::B_BYTES));
+                const int tx = t % a.tiles_x, rr = t / a.tiles_x;
+                const int x0 = tx * GTX, y0 = (rr % a.tiles_y) * GTY, n = rr / a.tiles_y;
+                const uint32_t As = sbase + s * C::STAGE, Bs = As + C::A_BYTES;
+                tma_load_4d(As, &tmX, q * CB, x0 - 1, y0 - 1, n, full(s));   // outside the image: zero fill
+#pragma unroll
+                for (int j = 0; j < BN / C::CBO; ++j)
+                    tma_load_4d(Bs + j * (GTX * GTY * C::CBO * 2), &tmD, j * C::CBO, x0, y0, n, full(s));
+            }
+            // every copy issued has landed before the CTA may end (bounded)
+            for (int j = it - 1; j >= 0 && j >= it - S; --j)
+                if (!mbar_wait(full(j % S), (j / S) & 1)) {
+                    give_up();
+                    break;
+                }
+        }
+    } else if (warp == 1) {
+        if (lane == 0) {
+            // ---- MMA issuer ----
+            constexpr uint32_t IDESC = tc_idesc_mn(TBM, BN);
+            constexpr uint32_t rowx = CB * 2, rowd = C::CBO * 2;
+            const uint64_t da = tc_desc(0, rowx, 8 * rowx, CB == 64 ? 2u : 4u);
+            const uint64_t db = tc_desc(0, GTX * GTY * rowd, 8 * rowd, C::CBO == 64 ? 2u : 4u);
+            int it = 0;
+            for (int t = t0; t < t1 && !*abort_flag; ++t, ++it) {
+                const int s = it % S;
+                if (!mbar_wait(full(s), (it / S) & 1)) {
+                    give_up();
+                    break;
+                }
+                tc_fence_after();
+                const uint64_t dx = da + ((sbase + s * C::STAGE) >> 4), dd = db + ((sbase + s * C::STAGE + C::A_BYTES) >> 4);
+                const uint32_t more = it != 0;
+#pragma unroll
+                for (int r = 0; r < GTY; ++r)
+#pragma unroll
+                    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+                        for (int m = 0; m < MT; ++m)
+                            tc_mma(tmem + (uint32_t)((dy * MT + m) * BN), dx + ((r + dy) * GPX + 2 * m) * rowx / 16,
+                                   dd + r * GTX * rowd / 16, IDESC, r == 0 ? more : 1u);
+                tc_commit(empty(s));
+            }
+            // every MMA issued has finished (bounded): the accumulators are complete
+            tc_commit(fin);
+            if (!mbar_wait(fin, 0)) give_up();
+        }
+    }
+    __syncthreads();
+    tc_fence_after();
+    // ---- epilogue: warps 2..5; TMEM lane = row: channel and dx ----
+    if (warp >= 2 && !*abort_flag) {
+        const int quarter = warp & 3, row = quarter * 32 + lane;
+        const uint32_t tl_lane = tmem + ((uint32_t)(quarter * 32) << 16);
+        const int K = 9 * a.cin;
+        float* out = a.part + (size_t)z * a.cout * K;
+#pragma unroll
+        for (int i = 0; i < C::ACC; ++i) {
+            const int dy = i / MT, dx = 2 * (i % MT) + row / CB;
+            const int k = (dy * 3 + dx) * a.cin + q * CB + row % CB;
+#pragma unroll
+            for (int c16 = 0; c16 < BN; c16 += 16) {
+                float v[16];
+                __syncwarp();
+                tc_ld16(tl_lane + (uint32_t)(i * BN + c16), v);
+                if (dx > 2) continue;
+#pragma unroll
+                for (int e = 0; e < 16; ++e) out[(size_t)(c16 + e) * K + k] = v[e];   // BN = cout
+            }
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(512u) : "memory");
+    }
+}
+
 // part[g][o] = sum of dz[p][o] over the pixel range g of G equal ranges (a fixed order:
 // 8-channel vectors by thread, rows strided by the block's row phases, then the phases in
 // order)
@@ -1469,6 +1642,23 @@ int launch_wgrad(const WgradArgs& a, int splits, cudaStream_t st) {
 
 constexpr int COLSUM_BLOCKS = 512;   // pixel ranges of the bias-gradient column sums
 
+// dw = the sum of the splits' partial tiles (part: [splits][cout][K]), db = the column sums of dz
+int finish_wgrad(const View& dz, long long P, int cout, int K, int splits, float* dw, float* db, float* part,
+                 cudaStream_t st) {
+    const long long nw = (long long)cout * K;
+    k_sum_splits<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(part, splits, nw, dw);
+    PAT_LAUNCH_CHECK("k_sum_splits");
+    if (db) {
+        const int G = (int)std::max<long long>(1, std::min<long long>(COLSUM_BLOCKS, (P + 63) / 64));
+        float* pb = part + (size_t)splits * nw;
+        k_colsum_part<<<G, 256, 0, st>>>(dz.p, dz.ps, P, cout, pb);
+        PAT_LAUNCH_CHECK("k_colsum_part");
+        k_sum_cols<<<(unsigned)((cout + 7) / 8), 256, 0, st>>>(pb, G, cout, db);
+        PAT_LAUNCH_CHECK("k_sum_cols");
+    }
+    return PAT_OK;
+}
+
 template <int BN>
 int launch_wgrad_tc(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, float* db,
                     float* part, int max_splits, cudaStream_t st) {
@@ -1522,19 +1712,64 @@ int launch_wgrad_tc(const View& x, const View& dz, int B, int H, int W, int cin,
     PAT_CUDA(attr);
     k_conv_wgrad_tc<BN><<<std::min(a.total, sm_count()), TC_THREADS, C::SMEM, st>>>(mx, md, a);
     PAT_LAUNCH_CHECK("k_conv_wgrad_tc");
-    const long long nw = (long long)cout * K;
-    k_sum_splits<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(part, a.splits, nw, dw);
-    PAT_LAUNCH_CHECK("k_sum_splits");
-    if (db) {
-        const long long P = (long long)B * H * W;
-        const int G = (int)std::max<long long>(1, std::min<long long>(COLSUM_BLOCKS, (P + 63) / 64));
-        float* pb = part + (size_t)a.splits * nw;
-        k_colsum_part<<<G, 256, 0, st>>>(dz.p, dz.ps, P, cout, pb);
-        PAT_LAUNCH_CHECK("k_colsum_part");
-        k_sum_cols<<<(unsigned)((cout + 7) / 8), 256, 0, st>>>(pb, G, cout, db);
-        PAT_LAUNCH_CHECK("k_sum_cols");
-    }
-    return PAT_OK;
+    return finish_wgrad(dz, (long long)B * H * W, cout, K, a.splits, dw, db, part, st);
+}
+
+template <int CB, int BN>
+int launch_wgrad_halo(const View& x, const View& dz, int B, int H, int W, int cin, float* dw, float* db, float* part,
+                      int max_splits, cudaStream_t st) {
+    using C = WgHaloCfg<CB, BN>;
+    const EncodeTiledFn enc = encode_tiled();
+    if (!enc) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: cuTensorMapEncodeTiled is not available");
+    WgHaloArgs a;
+    a.cin = cin;
+    a.cout = BN;
+    a.nq = cin / CB;
+    a.tiles_x = (W + GTX - 1) / GTX;
+    a.tiles_y = (H + GTY - 1) / GTY;
+    a.tiles = B * a.tiles_x * a.tiles_y;
+    const int want = std::max(1, std::min(max_splits, sm_count() / a.nq));
+    a.per = (a.tiles + want - 1) / want;
+    const int splits = (a.tiles + a.per - 1) / a.per;
+    a.part = part;
+    CUtensorMap mx, md;
+    const cuuint32_t es[4] = {1, 1, 1, 1};
+    auto map4 = [&](CUtensorMap* m, const View& v, int ch, int cb, int bx, int by) {
+        const cuuint64_t ps = (cuuint64_t)v.ps * 2;
+        const cuuint64_t dims[4] = {(cuuint64_t)ch, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)B};
+        const cuuint64_t strides[3] = {ps, ps * W, ps * W * H};
+        const cuuint32_t box[4] = {(cuuint32_t)cb, (cuuint32_t)bx, (cuuint32_t)by, 1};
+        return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)v.p, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   cb == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    };
+    if (map4(&mx, x, cin, CB, GPX, GPY) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: activation tensor map");
+    if (map4(&md, dz, BN, C::CBO, GTX, GTY) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: gradient tensor map");
+    static const cudaError_t attr =
+        cudaFuncSetAttribute(k_conv_wgrad_halo<CB, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
+    PAT_CUDA(attr);
+    k_conv_wgrad_halo<CB, BN><<<splits * a.nq, TC_THREADS, C::SMEM, st>>>(mx, md, a);
+    PAT_LAUNCH_CHECK("k_conv_wgrad_halo");
+    return finish_wgrad(dz, (long long)B * H * W, BN, 9 * cin, splits, dw, db, part, st);
+}
+
+// Whether the halo weight gradient takes a layer: channels in whole boxes, accumulators for
+// all output channels in tensor memory, and at least two pixel tiles per CTA.
+bool wgrad_halo_applies(int B, int H, int W, int cin, int cout) {
+    const bool fits = cin % 64 == 0 ? cout == 32 || cout == 64 : cin % 32 == 0 && (cout == 32 || cout == 64 || cout == 128);
+    const long long tiles = (long long)B * ((W + GTX - 1) / GTX) * ((H + GTY - 1) / GTY);
+    const int nq = cin / (cin % 64 == 0 ? 64 : 32);
+    return fits && nq <= 8 && tiles * nq >= 2LL * sm_count() && tiles < (1LL << 30);
+}
+
+int launch_wgrad_halo_any(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, float* db,
+                          float* part, int splits, cudaStream_t st) {
+    if (cin % 64 == 0)
+        return cout == 32 ? launch_wgrad_halo<64, 32>(x, dz, B, H, W, cin, dw, db, part, splits, st)
+                          : launch_wgrad_halo<64, 64>(x, dz, B, H, W, cin, dw, db, part, splits, st);
+    if (cout == 32) return launch_wgrad_halo<32, 32>(x, dz, B, H, W, cin, dw, db, part, splits, st);
+    if (cout == 64) return launch_wgrad_halo<32, 64>(x, dz, B, H, W, cin, dw, db, part, splits, st);
+    return launch_wgrad_halo<32, 128>(x, dz, B, H, W, cin, dw, db, part, splits, st);
 }
 
 struct SplitPlan {
@@ -1590,14 +1825,21 @@ int conv3x3_fwd(const View& x, int B, int H, int W, int cin, const bf16* w, cons
     return tc ? launch_fwd_tc<128, false>(a, st) : launch_fwd<128, false>(a, st);
 }
 
+// most splits a weight gradient may use (its partial tiles are allocated for them)
+static int wgrad_max_splits(int B, int H, int W, int cin, int cout) {
+    const int n = plan_splits(B, H, W, cin, cout).splits;
+    return wgrad_halo_applies(B, H, W, cin, cout) ? std::max(n, sm_count() / (cin / (cin % 64 == 0 ? 64 : 32))) : n;
+}
+
 size_t wgrad_partial_floats(int B, int H, int W, int cin, int cout) {
-    const SplitPlan sp = plan_splits(B, H, W, cin, cout);
-    return (size_t)sp.splits * cout * (9 * (size_t)cin + 1) + (size_t)COLSUM_BLOCKS * cout;
+    return (size_t)wgrad_max_splits(B, H, W, cin, cout) * cout * (9 * (size_t)cin + 1) + (size_t)COLSUM_BLOCKS * cout;
 }
 
 int conv3x3_wgrad(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, float* db,
                   float* part, cudaStream_t st) {
     const SplitPlan sp = plan_splits(B, H, W, cin, cout);
+    if (B > 0 && H > 0 && W > 0 && wgrad_halo_applies(B, H, W, cin, cout))
+        return launch_wgrad_halo_any(x, dz, B, H, W, cin, cout, dw, db, part, wgrad_max_splits(B, H, W, cin, cout), st);
     // the tensor-memory kernel (every layer with at most 256 output channels)
     if (cout <= 256 && B > 0 && H > 0 && W > 0) {
         if (cout <= 32) return launch_wgrad_tc<32>(x, dz, B, H, W, cin, cout, dw, db, part, sp.splits, st);

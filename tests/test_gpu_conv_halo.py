@@ -48,3 +48,28 @@ def test_halo_convolution_edges(b, h, w, cin, cout, relu, shift):
     err = (y.double().permute(0, 3, 1, 2) - ref).abs()
     assert bool((err <= 2e-5 * mag).all()), float((err / mag).max())
     assert P.pat_nn_wait_timeouts() == 0
+
+
+@pytest.mark.parametrize("b,h,w,cin,cout", [
+    (90, 15, 15, 32, 32), (40, 17, 33, 32, 64), (20, 33, 31, 32, 128), (24, 25, 47, 64, 32), (10, 63, 65, 64, 64),
+    (40, 9, 16, 96, 64), (13, 40, 49, 192, 64), (20, 24, 32, 128, 32),
+])
+def test_halo_weight_gradient_edges(b, h, w, cin, cout):
+    """The weight gradient of the wide layers: ragged pixel tiles of 16 x 8, one to three channel
+    boxes of 32 or 64, every width of the accumulators, and a last CTA with fewer tiles."""
+    g = torch.Generator(device=DEV).manual_seed(h + w + cin + cout)
+    x = torch.randn(b, h, w, cin, generator=g, device=DEV).bfloat16()
+    dy = torch.randn(b, h, w, cout, generator=g, device=DEV).bfloat16()
+    dw = torch.full((cout, 3, 3, cin), float("nan"), device=DEV)
+    db = torch.full((cout,), float("nan"), device=DEV)
+    P.pat_conv3x3_backward_weight(x, dy, b, h, w, cin, cout, dw, db)
+
+    def reference(a, d):
+        p = torch.nn.functional.pad(a.double(), (0, 0, 1, 1, 1, 1))
+        d = d.double().reshape(-1, cout)
+        return torch.stack([torch.stack([d.T @ p[:, i:i + h, j:j + w].reshape(-1, cin) for j in range(3)], 1)
+                            for i in range(3)], 1)
+
+    assert bool(((dw.double() - reference(x, dy)).abs() <= 2e-5 * reference(x.abs(), dy.abs())).all())
+    assert bool(((db.double() - dy.double().sum((0, 1, 2))).abs() <= 2e-5 * dy.double().abs().sum((0, 1, 2))).all())
+    assert P.pat_nn_wait_timeouts() == 0
