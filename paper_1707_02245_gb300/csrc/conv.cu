@@ -1218,9 +1218,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 //  - the 3 (CB = 32) or 6 (CB = 64) accumulators of BN columns stay in tensor memory for all
 //    of a CTA's pixel tiles and are written once, to part[split][o][k].
 // A CTA is one (channel box, split of the pixel tiles); k_sum_splits adds the splits.
-// Measured, batch 8, us per call with its sums (k_conv_wgrad_tc): 256^2 32 -> 32 53 (113), 96 -> 32
-// 102 (273); 128^2 64 -> 64 42 (54), 192 -> 64 62 (126).  One thread issues the MMAs (46 clocks
-// at N = 32 and 64); the sums of splits and columns are 25 us of each call.
+// Measured, batch 8, us per call with its sums (k_conv_wgrad_tc): 256^2 32 -> 32 46 (113), 96 -> 32
+// 96 (273); 128^2 64 -> 64 31 (55), 192 -> 64 60 (127).  One thread issues the MMAs (46 clocks at
+// N = 32 and 64); the sums of splits and columns are 10 to 15 us of each call.
 // ---------------------------------------------------------------------------------------
 constexpr int GTX = 16, GTY = 8;                       // pixel tile
 constexpr int GPX = GTX + 2, GPY = GTY + 2;            // with its halo
@@ -1389,6 +1389,7 @@ __global__ void __launch_bounds__(256) k_colsum_part(const bf16* __restrict__ dz
     const int phases = 256 / nv, v = tid % nv, ph = tid / nv;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (ph < phases) {
+#pragma unroll 4
         for (long long p = p0 + ph; p < p1; p += phases) {
             const uint4 q = __ldg(reinterpret_cast<const uint4*>(dz + p * ps) + v);
             const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&q);
@@ -1415,33 +1416,53 @@ __global__ void __launch_bounds__(256) k_colsum_part(const bf16* __restrict__ dz
 
 // out[c] = sum_g part[g][c], one warp per column: lane l adds rows l, l + 32, ... in order,
 // then a fixed butterfly over the lanes
-__global__ void __launch_bounds__(256) k_sum_cols(const float* __restrict__ part, int rows, int cols,
-                                                  float* __restrict__ out) {
-    const int c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+__device__ __forceinline__ void sum_col(const float* __restrict__ part, int rows, int cols, int c, float* __restrict__ out) {
+    const int lane = threadIdx.x & 31;
     if (c >= cols) return;
     float s = 0.f;
+#pragma unroll 4
     for (int g = lane; g < rows; g += 32) s += __ldg(part + (size_t)g * cols + c);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) out[c] = s;
 }
 
-// out[i] = sum_z part[z][i]
-__global__ void k_sum_splits(const float* __restrict__ part, int splits, long long n, float* __restrict__ out) {
-    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    // eight running sums (split z into sum z mod 8), added in order at the end: a fixed
-    // order with eight loads in flight
-    float s[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    int z = 0;
-    for (; z + 8 <= splits; z += 8)
+// out[i] = sum_z part[z][i] over the splits, and (blocks past the first `blocks`) the column sums
+// of colpart.  Eight running sums (split z into sum z mod 8), added in order at the end: a fixed
+// order.  A warp takes one of the eight for 32 outputs: with a thread taking all eight, a layer
+// of 9216 weights and 152 splits was 36 blocks of 19 dependent rounds each.  Weight gradient
+// calls, batch 8: 32 -> 32 at 256^2 53 -> 46 us, 32 -> 64 at 128^2 35 -> 26, 64 -> 64 42 -> 31.
+__global__ void __launch_bounds__(256) k_sum_splits(const float* __restrict__ part, int splits, long long n,
+                                                    float* __restrict__ out, int blocks, const float* __restrict__ colpart,
+                                                    int rows, int cols, float* __restrict__ colout) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((int)blockIdx.x >= blocks) {
+        sum_col(colpart, rows, cols, ((int)blockIdx.x - blocks) * 8 + warp, colout);
+        return;
+    }
+    __shared__ float sh[8][32];
+    const long long i = (long long)blockIdx.x * 32 + lane;
+    float s = 0.f;
+    if (i < n) {
+#pragma unroll 4
+        for (int z = warp; z < splits; z += 8) s += __ldg(part + (size_t)z * n + i);
+    }
+    sh[warp][lane] = s;
+    __syncthreads();
+    if (warp == 0 && i < n) {
+        float t = 0.f;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) s[j] += __ldg(part + (size_t)(z + j) * n + i);
-    for (int j = 0; z < splits; ++z, ++j) s[j] += __ldg(part + (size_t)z * n + i);
-    float t = 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) t += s[j];
-    out[i] = t;
+        for (int j = 0; j < 8; ++j) t += sh[j][lane];
+        out[i] = t;
+    }
+}
+
+int launch_sum_splits(const float* part, int splits, long long n, float* out, const float* colpart, int rows, int cols,
+                      float* colout, cudaStream_t st) {
+    const int blocks = (int)((n + 31) / 32), more = colout ? (cols + 7) / 8 : 0;
+    k_sum_splits<<<blocks + more, 256, 0, st>>>(part, splits, n, out, blocks, colpart, rows, cols, colout);
+    PAT_LAUNCH_CHECK("k_sum_splits");
+    return PAT_OK;
 }
 
 __global__ void k_flip_weights(const bf16* __restrict__ w, int cout, int cin, bf16* __restrict__ wf) {
@@ -1646,17 +1667,15 @@ constexpr int COLSUM_BLOCKS = 512;   // pixel ranges of the bias-gradient column
 int finish_wgrad(const View& dz, long long P, int cout, int K, int splits, float* dw, float* db, float* part,
                  cudaStream_t st) {
     const long long nw = (long long)cout * K;
-    k_sum_splits<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(part, splits, nw, dw);
-    PAT_LAUNCH_CHECK("k_sum_splits");
+    float* pb = nullptr;
+    int G = 0;
     if (db) {
-        const int G = (int)std::max<long long>(1, std::min<long long>(COLSUM_BLOCKS, (P + 63) / 64));
-        float* pb = part + (size_t)splits * nw;
+        G = (int)std::max<long long>(1, std::min<long long>(COLSUM_BLOCKS, (P + 63) / 64));
+        pb = part + (size_t)splits * nw;
         k_colsum_part<<<G, 256, 0, st>>>(dz.p, dz.ps, P, cout, pb);
         PAT_LAUNCH_CHECK("k_colsum_part");
-        k_sum_cols<<<(unsigned)((cout + 7) / 8), 256, 0, st>>>(pb, G, cout, db);
-        PAT_LAUNCH_CHECK("k_sum_cols");
     }
-    return PAT_OK;
+    return launch_sum_splits(part, splits, nw, dw, pb, G, cout, db, st);
 }
 
 template <int BN>
@@ -1863,13 +1882,9 @@ int conv3x3_wgrad(const View& x, const View& dz, int B, int H, int W, int cin, i
     a.chunks_per_split = (int)sp.per;
     int rc = cout <= 32 ? launch_wgrad<32>(a, sp.splits, st) : launch_wgrad<64>(a, sp.splits, st);
     if (rc) return rc;
-    k_sum_splits<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(part, sp.splits, nw, dw);
-    PAT_LAUNCH_CHECK("k_sum_splits");
-    if (db) {
-        k_sum_splits<<<(unsigned)((cout + 255) / 256), 256, 0, st>>>(a.part_b, sp.splits, cout, db);
-        PAT_LAUNCH_CHECK("k_sum_splits");
-    }
-    return PAT_OK;
+    rc = launch_sum_splits(part, sp.splits, nw, dw, nullptr, 0, 0, nullptr, st);
+    if (!rc && db) rc = launch_sum_splits(a.part_b, sp.splits, cout, db, nullptr, 0, 0, nullptr, st);
+    return rc;
 }
 
 unsigned wait_timeouts() {
