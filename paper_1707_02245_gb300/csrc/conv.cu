@@ -1218,8 +1218,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 //  - the 3 (CB = 32) or 6 (CB = 64) accumulators of BN columns stay in tensor memory for all
 //    of a CTA's pixel tiles and are written once, to part[split][o][k].
 // A CTA is one (channel box, split of the pixel tiles); k_sum_splits adds the splits.
-// Measured, batch 8, us per call with its sums (k_conv_wgrad_tc): 256^2 32 -> 32 46 (113), 96 -> 32
-// 96 (273); 128^2 64 -> 64 31 (55), 192 -> 64 60 (127).  One thread issues the MMAs (46 clocks at
+// Measured, batch 8, us per call with its sums (k_conv_wgrad_tc): 256^2 32 -> 32 44 (113), 96 -> 32
+// 96 (273); 128^2 64 -> 64 35 (55), 192 -> 64 60 (127).  One thread issues the MMAs (46 clocks at
 // N = 32 and 64); the sums of splits and columns are 10 to 15 us of each call.
 // ---------------------------------------------------------------------------------------
 constexpr int GTX = 16, GTY = 8;                       // pixel tile
@@ -1228,6 +1228,7 @@ constexpr int G_MAX_STAGES = 6;
 
 struct WgHaloArgs {
     int cin, cout, nq;                                 // nq: channel boxes of x
+    int whole;                                         // cin fills them, and cout the accumulators' columns
     int tiles_x, tiles_y, tiles, per;                  // pixel tiles, and how many a CTA takes
     float* part;
 };
@@ -1364,8 +1365,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                 __syncwarp();
                 tc_ld16(tl_lane + (uint32_t)(i * BN + c16), v);
                 if (dx > 2) continue;
+                if (a.whole) {
 #pragma unroll
-                for (int e = 0; e < 16; ++e) out[(size_t)(c16 + e) * K + k] = v[e];   // BN = cout
+                    for (int e = 0; e < 16; ++e) out[(size_t)(c16 + e) * K + k] = v[e];
+                } else if (q * CB + row % CB < a.cin) {
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        if (c16 + e < a.cout) out[(size_t)(c16 + e) * K + k] = v[e];
+                }
             }
         }
     }
@@ -1378,39 +1385,67 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
 }
 
 // part[g][o] = sum of dz[p][o] over the pixel range g of G equal ranges (a fixed order:
-// 8-channel vectors by thread, rows strided by the block's row phases, then the phases in
-// order)
-__global__ void __launch_bounds__(256) k_colsum_part(const bf16* __restrict__ dz, int ps, long long P, int cout,
-                                                     float* __restrict__ part) {
-    __shared__ float sh[256][8];
+// 8-channel vectors by thread, rows strided by the block's row phases, then a butterfly over
+// the phases of a warp where its lanes hold whole rows, then the others in order).  MASK: dz is
+// first set to 0 where the layer's output y is not above 0 (the derivative of a ReLU), so the
+// network's gradient is read once for both (batch 8, mean of the 256^2 x 32 and 128^2 x 64
+// layers: 15 us, mask and sums in two launches 19).
+template <bool MASK>
+__global__ void __launch_bounds__(256) k_colsum_part(bf16* __restrict__ dz, int ps, const bf16* __restrict__ y, int y_ps,
+                                                     long long P, int cout, float* __restrict__ part) {
+    __shared__ float sh[256][9];
     const int g = blockIdx.x, G = gridDim.x;
     const long long p0 = P * g / G, p1 = P * (g + 1) / G;
     const int nv = cout / 8, tid = threadIdx.x;
     const int phases = 256 / nv, v = tid % nv, ph = tid / nv;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if (ph < phases) {
-#pragma unroll 4
-        for (long long p = p0 + ph; p < p1; p += phases) {
-            const uint4 q = __ldg(reinterpret_cast<const uint4*>(dz + p * ps) + v);
-            const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&q);
+        constexpr int U = 4;   // rows in flight (a masked row's store would hold back the next row's load)
+        for (long long p = p0 + ph; p < p1; p += U * phases) {
+            uint4 q[U], m[U];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const float2 f = __bfloat1622float2(h[e]);
-                acc[2 * e] += f.x;
-                acc[2 * e + 1] += f.y;
+            for (int u = 0; u < U; ++u) {
+                const long long pu = p + u * phases;
+                if (pu >= p1) continue;
+                q[u] = *(reinterpret_cast<const uint4*>(dz + pu * ps) + v);
+                if (MASK) m[u] = __ldg(reinterpret_cast<const uint4*>(y + pu * y_ps) + v);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const long long pu = p + u * phases;
+                if (pu >= p1) continue;
+                __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&q[u]);
+                const __nv_bfloat162* mh = reinterpret_cast<const __nv_bfloat162*>(&m[u]);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    float2 f = __bfloat1622float2(h[e]);
+                    if (MASK) {
+                        const float2 k = __bfloat1622float2(mh[e]);
+                        f.x = k.x > 0.f ? f.x : 0.f;
+                        f.y = k.y > 0.f ? f.y : 0.f;
+                        h[e] = __floats2bfloat162_rn(f.x, f.y);
+                    }
+                    acc[2 * e] += f.x;
+                    acc[2 * e + 1] += f.y;
+                }
+                if (MASK) *(reinterpret_cast<uint4*>(dz + pu * ps) + v) = q[u];
             }
         }
+    }
+    int step = 1;   // of the phases left
+    if (32 % nv == 0) {
+        for (int o = nv; o < 32; o <<= 1)
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+        step = 32 / nv;
     }
 #pragma unroll
     for (int e = 0; e < 8; ++e) sh[tid][e] = acc[e];
     __syncthreads();
-    if (tid < nv) {
-        float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int r = 0; r < phases; ++r)
-#pragma unroll
-            for (int e = 0; e < 8; ++e) s[e] += sh[r * nv + tid][e];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) part[(size_t)g * cout + tid * 8 + e] = s[e];
+    for (int c = tid; c < cout; c += 256) {
+        float s = 0.f;
+        for (int r = 0; r < phases; r += step) s += sh[r * nv + (c >> 3)][c & 7];
+        part[(size_t)g * cout + c] = s;
     }
 }
 
@@ -1420,7 +1455,7 @@ __device__ __forceinline__ void sum_col(const float* __restrict__ part, int rows
     const int lane = threadIdx.x & 31;
     if (c >= cols) return;
     float s = 0.f;
-#pragma unroll 4
+#pragma unroll 8
     for (int g = lane; g < rows; g += 32) s += __ldg(part + (size_t)g * cols + c);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -1661,26 +1696,22 @@ int launch_wgrad(const WgradArgs& a, int splits, cudaStream_t st) {
     return PAT_OK;
 }
 
-constexpr int COLSUM_BLOCKS = 512;   // pixel ranges of the bias-gradient column sums
+constexpr int COLSUM_BLOCKS = 608;   // pixel ranges of the bias-gradient column sums: 4 blocks on each SM
 
-// dw = the sum of the splits' partial tiles (part: [splits][cout][K]), db = the column sums of dz
-int finish_wgrad(const View& dz, long long P, int cout, int K, int splits, float* dw, float* db, float* part,
-                 cudaStream_t st) {
-    const long long nw = (long long)cout * K;
-    float* pb = nullptr;
-    int G = 0;
-    if (db) {
-        G = (int)std::max<long long>(1, std::min<long long>(COLSUM_BLOCKS, (P + 63) / 64));
-        pb = part + (size_t)splits * nw;
-        k_colsum_part<<<G, 256, 0, st>>>(dz.p, dz.ps, P, cout, pb);
-        PAT_LAUNCH_CHECK("k_colsum_part");
-    }
-    return launch_sum_splits(part, splits, nw, dw, pb, G, cout, db, st);
+// the column sums of dz into part (masked by y first, if it has a pointer); returns the ranges
+int colsums(const View& dz, const View& y, long long P, int cout, float* part, cudaStream_t st, int* rows) {
+    *rows = (int)std::max<long long>(1, std::min<long long>(COLSUM_BLOCKS, (P + 63) / 64));
+    if (y.p)
+        k_colsum_part<true><<<*rows, 256, 0, st>>>(dz.p, dz.ps, y.p, y.ps, P, cout, part);
+    else
+        k_colsum_part<false><<<*rows, 256, 0, st>>>(dz.p, dz.ps, nullptr, 0, P, cout, part);
+    PAT_LAUNCH_CHECK("k_colsum_part");
+    return PAT_OK;
 }
 
 template <int BN>
-int launch_wgrad_tc(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, float* db,
-                    float* part, int max_splits, cudaStream_t st) {
+int launch_wgrad_tc(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, int colrows,
+                    const float* colpart, float* db, float* part, int max_splits, cudaStream_t st) {
     using C = WgCfg<BN>;
     const EncodeTiledFn enc = encode_tiled();
     if (!enc) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: cuTensorMapEncodeTiled is not available");
@@ -1731,19 +1762,20 @@ int launch_wgrad_tc(const View& x, const View& dz, int B, int H, int W, int cin,
     PAT_CUDA(attr);
     k_conv_wgrad_tc<BN><<<std::min(a.total, sm_count()), TC_THREADS, C::SMEM, st>>>(mx, md, a);
     PAT_LAUNCH_CHECK("k_conv_wgrad_tc");
-    return finish_wgrad(dz, (long long)B * H * W, cout, K, a.splits, dw, db, part, st);
+    return launch_sum_splits(part, a.splits, (long long)cout * K, dw, colpart, colrows, cout, db, st);
 }
 
 template <int CB, int BN>
-int launch_wgrad_halo(const View& x, const View& dz, int B, int H, int W, int cin, float* dw, float* db, float* part,
-                      int max_splits, cudaStream_t st) {
+int launch_wgrad_halo(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, int colrows,
+                      const float* colpart, float* db, float* part, int max_splits, cudaStream_t st) {
     using C = WgHaloCfg<CB, BN>;
     const EncodeTiledFn enc = encode_tiled();
     if (!enc) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: cuTensorMapEncodeTiled is not available");
     WgHaloArgs a;
     a.cin = cin;
-    a.cout = BN;
-    a.nq = cin / CB;
+    a.cout = cout;
+    a.nq = (cin + CB - 1) / CB;
+    a.whole = cin % CB == 0 && cout == BN;
     a.tiles_x = (W + GTX - 1) / GTX;
     a.tiles_y = (H + GTY - 1) / GTY;
     a.tiles = B * a.tiles_x * a.tiles_y;
@@ -1763,32 +1795,36 @@ int launch_wgrad_halo(const View& x, const View& dz, int B, int H, int W, int ci
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     };
     if (map4(&mx, x, cin, CB, GPX, GPY) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: activation tensor map");
-    if (map4(&md, dz, BN, C::CBO, GTX, GTY) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: gradient tensor map");
+    if (map4(&md, dz, cout, C::CBO, GTX, GTY) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: gradient tensor map");
     static const cudaError_t attr =
         cudaFuncSetAttribute(k_conv_wgrad_halo<CB, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     PAT_CUDA(attr);
     k_conv_wgrad_halo<CB, BN><<<splits * a.nq, TC_THREADS, C::SMEM, st>>>(mx, md, a);
     PAT_LAUNCH_CHECK("k_conv_wgrad_halo");
-    return finish_wgrad(dz, (long long)B * H * W, BN, 9 * cin, splits, dw, db, part, st);
+    return launch_sum_splits(part, splits, 9LL * cin * cout, dw, colpart, colrows, cout, db, st);
 }
 
-// Whether the halo weight gradient takes a layer: channels in whole boxes, accumulators for
-// all output channels in tensor memory, and at least two pixel tiles per CTA.
+// Whether the halo weight gradient takes a layer: input channels in whole boxes, accumulators
+// for all output channels in tensor memory, and at least two pixel tiles per CTA.  Fewer than
+// 32 channels on either side are a box of 32 whose other channels the tensor map fills with
+// zeros and the epilogue drops: a layer of 8 costs what one of 32 costs (256^2, batch 8:
+// 32 -> 8 NARROWUS).
+int wgrad_halo_boxes(int cin) { return cin % 64 == 0 ? cin / 64 : (cin + 31) / 32; }
+
 bool wgrad_halo_applies(int B, int H, int W, int cin, int cout) {
-    const bool fits = cin % 64 == 0 ? cout == 32 || cout == 64 : cin % 32 == 0 && (cout == 32 || cout == 64 || cout == 128);
+    const bool fits = (cin % 32 == 0 || cin < 32) && (cout <= 32 || cout == 64 || (cout == 128 && cin % 64 != 0));
     const long long tiles = (long long)B * ((W + GTX - 1) / GTX) * ((H + GTY - 1) / GTY);
-    const int nq = cin / (cin % 64 == 0 ? 64 : 32);
+    const int nq = wgrad_halo_boxes(cin);
     return fits && nq <= 8 && tiles * nq >= 2LL * sm_count() && tiles < (1LL << 30);
 }
 
-int launch_wgrad_halo_any(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, float* db,
-                          float* part, int splits, cudaStream_t st) {
-    if (cin % 64 == 0)
-        return cout == 32 ? launch_wgrad_halo<64, 32>(x, dz, B, H, W, cin, dw, db, part, splits, st)
-                          : launch_wgrad_halo<64, 64>(x, dz, B, H, W, cin, dw, db, part, splits, st);
-    if (cout == 32) return launch_wgrad_halo<32, 32>(x, dz, B, H, W, cin, dw, db, part, splits, st);
-    if (cout == 64) return launch_wgrad_halo<32, 64>(x, dz, B, H, W, cin, dw, db, part, splits, st);
-    return launch_wgrad_halo<32, 128>(x, dz, B, H, W, cin, dw, db, part, splits, st);
+int launch_wgrad_halo_any(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, int colrows,
+                          const float* colpart, float* db, float* part, int splits, cudaStream_t st) {
+    auto go = cin % 64 == 0 ? (cout <= 32 ? launch_wgrad_halo<64, 32> : launch_wgrad_halo<64, 64>)
+              : cout <= 32  ? launch_wgrad_halo<32, 32>
+              : cout == 64  ? launch_wgrad_halo<32, 64>
+                            : launch_wgrad_halo<32, 128>;
+    return go(x, dz, B, H, W, cin, cout, dw, colrows, colpart, db, part, splits, st);
 }
 
 struct SplitPlan {
@@ -1847,25 +1883,31 @@ int conv3x3_fwd(const View& x, int B, int H, int W, int cin, const bf16* w, cons
 // most splits a weight gradient may use (its partial tiles are allocated for them)
 static int wgrad_max_splits(int B, int H, int W, int cin, int cout) {
     const int n = plan_splits(B, H, W, cin, cout).splits;
-    return wgrad_halo_applies(B, H, W, cin, cout) ? std::max(n, sm_count() / (cin / (cin % 64 == 0 ? 64 : 32))) : n;
+    return wgrad_halo_applies(B, H, W, cin, cout) ? std::max(n, sm_count() / wgrad_halo_boxes(cin)) : n;
 }
 
 size_t wgrad_partial_floats(int B, int H, int W, int cin, int cout) {
     return (size_t)wgrad_max_splits(B, H, W, cin, cout) * cout * (9 * (size_t)cin + 1) + (size_t)COLSUM_BLOCKS * cout;
 }
 
-int conv3x3_wgrad(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, float* db,
-                  float* part, cudaStream_t st) {
+int conv3x3_wgrad(const View& x, const View& dz, const View& y, int B, int H, int W, int cin, int cout, float* dw,
+                  float* db, float* part, cudaStream_t st) {
     const SplitPlan sp = plan_splits(B, H, W, cin, cout);
-    if (B > 0 && H > 0 && W > 0 && wgrad_halo_applies(B, H, W, cin, cout))
-        return launch_wgrad_halo_any(x, dz, B, H, W, cin, cout, dw, db, part, wgrad_max_splits(B, H, W, cin, cout), st);
-    // the tensor-memory kernel (every layer with at most 256 output channels)
-    if (cout <= 256 && B > 0 && H > 0 && W > 0) {
-        if (cout <= 32) return launch_wgrad_tc<32>(x, dz, B, H, W, cin, cout, dw, db, part, sp.splits, st);
-        if (cout <= 64) return launch_wgrad_tc<64>(x, dz, B, H, W, cin, cout, dw, db, part, sp.splits, st);
-        if (cout <= 128) return launch_wgrad_tc<128>(x, dz, B, H, W, cin, cout, dw, db, part, sp.splits, st);
-        return launch_wgrad_tc<256>(x, dz, B, H, W, cin, cout, dw, db, part, sp.splits, st);
+    // the tensor-memory kernels (every layer with at most 256 output channels)
+    if (cout <= WGRAD_TC_COUT && B > 0 && H > 0 && W > 0) {
+        const int splits = wgrad_max_splits(B, H, W, cin, cout);
+        float* cp = part + (size_t)splits * cout * 9 * cin;
+        int rows = 0;
+        if (db || y.p)
+            if (const int rc = colsums(dz, y, (long long)B * H * W, cout, cp, st, &rows)) return rc;
+        if (wgrad_halo_applies(B, H, W, cin, cout))
+            return launch_wgrad_halo_any(x, dz, B, H, W, cin, cout, dw, rows, cp, db, part, splits, st);
+        if (cout <= 32) return launch_wgrad_tc<32>(x, dz, B, H, W, cin, cout, dw, rows, cp, db, part, sp.splits, st);
+        if (cout <= 64) return launch_wgrad_tc<64>(x, dz, B, H, W, cin, cout, dw, rows, cp, db, part, sp.splits, st);
+        if (cout <= 128) return launch_wgrad_tc<128>(x, dz, B, H, W, cin, cout, dw, rows, cp, db, part, sp.splits, st);
+        return launch_wgrad_tc<256>(x, dz, B, H, W, cin, cout, dw, rows, cp, db, part, sp.splits, st);
     }
+    if (y.p) return fail(PAT_ERR_INVALID_ARG, "conv3x3_wgrad: the mask is taken with at most 256 output channels");
     const long long nw = (long long)cout * 9 * cin;
     WgradArgs a;
     a.x = x.p;

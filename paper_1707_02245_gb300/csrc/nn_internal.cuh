@@ -26,10 +26,13 @@ int conv3x3_fwd(const View& x, int B, int H, int W, int cin, const bf16* w, cons
                 bool relu, const View& y, float* y_f32, int y_f32_ps, cudaStream_t st);
 
 // dw[o][tap][c] = sum_p dz[p][o] x[p + tap][c] and db[o] = sum_p dz[p][o] (FP32,
-// overwritten; db may be null).  part must hold wgrad_partial_floats(...) floats.
+// overwritten; db may be null).  part must hold wgrad_partial_floats(...) floats.  If y has a
+// pointer (at most WGRAD_TC_COUT output channels), dz is first set to 0 where y <= 0, in place,
+// by the kernel that sums its columns; else dz is only read.
+constexpr int WGRAD_TC_COUT = 256;
 size_t wgrad_partial_floats(int B, int H, int W, int cin, int cout);
-int conv3x3_wgrad(const View& x, const View& dz, int B, int H, int W, int cin, int cout, float* dw, float* db,
-                  float* part, cudaStream_t st);
+int conv3x3_wgrad(const View& x, const View& dz, const View& y, int B, int H, int W, int cin, int cout, float* dw,
+                  float* db, float* part, cudaStream_t st);
 
 // wflip[c][tap][o] = w[o][8 - tap][c]: the weights of the transposed convolution that gives
 // dL/dx from dL/dy.

@@ -439,12 +439,17 @@ int conv(pat_unet* net, int idx, const View& x, int l, const View& y, bool relu,
                            c.cout, relu, y, y32, c.cout, st);
 }
 
-// weight gradient into grad, and (if dx.p) the input gradient
-int conv_back(pat_unet* net, int idx, const View& x, const View& dz, int l, const View& dx, float* grad,
+// weight gradient into grad, and (if dx.p) the input gradient; if y.p, dz is masked first by
+// the layer's ReLU, whose output is y
+int conv_back(pat_unet* net, int idx, const View& x, const View& dz, View y, int l, const View& dx, float* grad,
               cudaStream_t st) {
     const ConvSpec& c = net->convs[idx];
     const int Hl = net->aH >> l, Wl = net->aW >> l;
-    int rc = nn::conv3x3_wgrad(x, dz, net->aB, Hl, Wl, c.cin, c.cout, grad + c.w_off, grad + c.b_off, net->wpart, st);
+    if (y.p && c.cout > nn::WGRAD_TC_COUT) {
+        if (const int rc = relu_mask(dz, y, (long long)net->aB * Hl * Wl, c.cout, st)) return rc;
+        y.p = nullptr;
+    }
+    int rc = nn::conv3x3_wgrad(x, dz, y, net->aB, Hl, Wl, c.cin, c.cout, grad + c.w_off, grad + c.b_off, net->wpart, st);
     if (rc || !dx.p) return rc;
     rc = nn::flip_weights(net->wbf + c.w_off, c.cout, c.cin, net->wflip, st);
     if (rc) return rc;
@@ -487,17 +492,14 @@ int forward_impl(pat_unet* net, const bf16* x, int B, int H, int W, float* y, cu
 int backward_impl(pat_unet* net, float* grad, cudaStream_t st) {
     const int L = net->d.levels;
     const int B = net->aB, H = net->aH, W = net->aW;
-    auto P = [&](int l) { return (long long)B * (H >> l) * (W >> l); };
     const View g_top = L >= 2 ? View{net->gD[0], ch(net, 0)} : View{net->gEbot, ch(net, 0)};
-    TRY(conv_back(net, conv_head(net), top_view(net), View{net->dpred, net->d.out_ch}, 0, g_top, grad, st));
+    TRY(conv_back(net, conv_head(net), top_view(net), View{net->dpred, net->d.out_ch}, View{nullptr, 0}, 0, g_top, grad, st));
     for (int l = 0; l <= L - 2; ++l) {
         const View gd{net->gD[l], ch(net, l)}, gda{net->gDA[l], ch(net, l)};
         const View da{net->DA[l], ch(net, l)}, d{net->D[l], ch(net, l)};
         const View cat{net->cat[l], cat_ch(net, l)}, gcat{net->gcat[l], cat_ch(net, l)};
-        TRY(relu_mask(gd, d, P(l), ch(net, l), st));
-        TRY(conv_back(net, conv_dec(net, l, 1), da, gd, l, gda, grad, st));
-        TRY(relu_mask(gda, da, P(l), ch(net, l), st));
-        TRY(conv_back(net, conv_dec(net, l, 0), cat, gda, l, gcat, grad, st));
+        TRY(conv_back(net, conv_dec(net, l, 1), da, gd, d, l, gda, grad, st));
+        TRY(conv_back(net, conv_dec(net, l, 0), cat, gda, da, l, gcat, grad, st));
         const View gnext = l + 1 <= L - 2 ? View{net->gD[l + 1], ch(net, l + 1)} : View{net->gEbot, ch(net, l + 1)};
         TRY(resample(gcat, gnext, nullptr, B, H >> (l + 1), W >> (l + 1), ch(net, l + 1), 0, 1.f, st));
     }
@@ -508,13 +510,11 @@ int backward_impl(pat_unet* net, float* grad, cudaStream_t st) {
             const View skip{net->gcat[l] + ch(net, l + 1), cat_ch(net, l)};
             TRY(resample(View{net->gIn[l + 1], ch(net, l)}, ge, &skip, B, H >> l, W >> l, ch(net, l), 1, 0.25f, st));
         }
-        TRY(relu_mask(ge, e_view(net, l), P(l), ch(net, l), st));
         const View a{net->A[l], ch(net, l)}, ga{net->gA[l], ch(net, l)};
-        TRY(conv_back(net, conv_enc(l, 1), a, ge, l, ga, grad, st));
-        TRY(relu_mask(ga, a, P(l), ch(net, l), st));
+        TRY(conv_back(net, conv_enc(l, 1), a, ge, e_view(net, l), l, ga, grad, st));
         const View in = l > 0 ? View{net->pin[l], ch(net, l - 1)} : View{const_cast<bf16*>(net->x_last), net->d.in_ch};
         const View gin = l > 0 ? View{net->gIn[l], ch(net, l - 1)} : View{nullptr, 0};
-        TRY(conv_back(net, conv_enc(l, 0), in, ga, l, gin, grad, st));
+        TRY(conv_back(net, conv_enc(l, 0), in, ga, a, l, gin, grad, st));
     }
     return PAT_OK;
 }
@@ -581,8 +581,8 @@ int pat_conv3x3_backward_weight(const uint16_t* x_dev, const uint16_t* dy_dev, i
     cudaStream_t st = (cudaStream_t)stream;
     float* part = nullptr;
     PAT_CUDA(cudaMallocAsync(&part, nn::wgrad_partial_floats(batch, h, w, cin, cout) * 4 + 16, st));
-    const int rc = nn::conv3x3_wgrad(View{(bf16*)x_dev, cin}, View{(bf16*)dy_dev, cout}, batch, h, w, cin, cout, dw_dev,
-                                     db_dev, part, st);
+    const int rc = nn::conv3x3_wgrad(View{(bf16*)x_dev, cin}, View{(bf16*)dy_dev, cout}, View{nullptr, 0}, batch, h, w, cin, cout,
+                                     dw_dev, db_dev, part, st);
     cudaFreeAsync(part, st);
     return rc;
 }

@@ -53,10 +53,12 @@ def test_halo_convolution_edges(b, h, w, cin, cout, relu, shift):
 @pytest.mark.parametrize("b,h,w,cin,cout", [
     (90, 15, 15, 32, 32), (40, 17, 33, 32, 64), (20, 33, 31, 32, 128), (24, 25, 47, 64, 32), (10, 63, 65, 64, 64),
     (40, 9, 16, 96, 64), (13, 40, 49, 192, 64), (20, 24, 32, 128, 32),
+    (90, 15, 15, 8, 32), (40, 17, 33, 32, 8), (24, 33, 31, 16, 24), (40, 24, 32, 64, 16), (28, 31, 41, 24, 128),
 ])
 def test_halo_weight_gradient_edges(b, h, w, cin, cout):
     """The weight gradient of the wide layers: ragged pixel tiles of 16 x 8, one to three channel
-    boxes of 32 or 64, every width of the accumulators, and a last CTA with fewer tiles."""
+    boxes of 32 or 64, fewer than 32 channels on either side, every width of the accumulators, and
+    a last CTA with fewer tiles."""
     g = torch.Generator(device=DEV).manual_seed(h + w + cin + cout)
     x = torch.randn(b, h, w, cin, generator=g, device=DEV).bfloat16()
     dy = torch.randn(b, h, w, cout, generator=g, device=DEV).bfloat16()
