@@ -1808,7 +1808,7 @@ int launch_wgrad_halo(const View& x, const View& dz, int B, int H, int W, int ci
 // for all output channels in tensor memory, and at least two pixel tiles per CTA.  Fewer than
 // 32 channels on either side are a box of 32 whose other channels the tensor map fills with
 // zeros and the epilogue drops: a layer of 8 costs what one of 32 costs (256^2, batch 8:
-// 32 -> 8 NARROWUS).
+// 32 -> 8: 43 us per call with its sums, with k_conv_wgrad_tc 113).
 int wgrad_halo_boxes(int cin) { return cin % 64 == 0 ? cin / 64 : (cin + 31) / 32; }
 
 bool wgrad_halo_applies(int B, int H, int W, int cin, int cout) {
