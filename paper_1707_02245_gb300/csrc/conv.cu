@@ -1464,38 +1464,57 @@ __device__ __forceinline__ void sum_col(const float* __restrict__ part, int rows
 
 // out[i] = sum_z part[z][i] over the splits, and (blocks past the first `blocks`) the column sums
 // of colpart.  Eight running sums (split z into sum z mod 8), added in order at the end: a fixed
-// order.  A warp takes one of the eight for 32 outputs: with a thread taking all eight, a layer
-// of 9216 weights and 152 splits was 36 blocks of 19 dependent rounds each.  Weight gradient
-// calls, batch 8: 32 -> 32 at 256^2 53 -> 46 us, 32 -> 64 at 128^2 35 -> 26, 64 -> 64 42 -> 31.
+// order.  G warps share 32 outputs, each with 8 / G of the sums: with G = 1 a layer of 9216
+// weights and 152 splits was 36 blocks of 19 dependent rounds each.  Weight gradient calls,
+// batch 8, G = 8 against 1: 32 -> 32 at 256^2 46 against 53 us, 32 -> 64 at 128^2 26 against 35,
+// 64 -> 64 31 against 42; but the network's pass, with layers of 590 k weights, 1.89 ms with G = 8
+// throughout and 1.87 with the rule of launch_sum_splits.
+template <int G>
 __global__ void __launch_bounds__(256) k_sum_splits(const float* __restrict__ part, int splits, long long n,
                                                     float* __restrict__ out, int blocks, const float* __restrict__ colpart,
                                                     int rows, int cols, float* __restrict__ colout) {
+    constexpr int V = 8 / G, OUT = 256 / G;   // sums per thread, outputs per block
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if ((int)blockIdx.x >= blocks) {
         sum_col(colpart, rows, cols, ((int)blockIdx.x - blocks) * 8 + warp, colout);
         return;
     }
-    __shared__ float sh[8][32];
-    const long long i = (long long)blockIdx.x * 32 + lane;
-    float s = 0.f;
+    __shared__ float sh[8][OUT];
+    const int o = warp / G * 32 + lane, first = warp % G * V;
+    const long long i = (long long)blockIdx.x * OUT + o;
+    float s[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) s[j] = 0.f;
     if (i < n) {
-#pragma unroll 4
-        for (int z = warp; z < splits; z += 8) s += __ldg(part + (size_t)z * n + i);
+        int z = first;
+#pragma unroll (G >= 4 ? 4 : 1)
+        for (; z + V <= splits; z += 8)
+#pragma unroll
+            for (int j = 0; j < V; ++j) s[j] += __ldg(part + (size_t)(z + j) * n + i);
+#pragma unroll
+        for (int j = 0; j < V; ++j)
+            if (z + j < splits) s[j] += __ldg(part + (size_t)(z + j) * n + i);
     }
-    sh[warp][lane] = s;
+#pragma unroll
+    for (int j = 0; j < V; ++j) sh[first + j][o] = s[j];
     __syncthreads();
-    if (warp == 0 && i < n) {
+    if (first == 0 && i < n) {
         float t = 0.f;
 #pragma unroll
-        for (int j = 0; j < 8; ++j) t += sh[j][lane];
+        for (int j = 0; j < 8; ++j) t += sh[j][o];
         out[i] = t;
     }
 }
 
 int launch_sum_splits(const float* part, int splits, long long n, float* out, const float* colpart, int rows, int cols,
                       float* colout, cudaStream_t st) {
-    const int blocks = (int)((n + 31) / 32), more = colout ? (cols + 7) / 8 : 0;
-    k_sum_splits<<<blocks + more, 256, 0, st>>>(part, splits, n, out, blocks, colpart, rows, cols, colout);
+    // the fewest warps per output that give every SM its 2048 threads (more only add rounds of
+    // blocks whose warps have no split left)
+    const long long want = 2048LL * sm_count();
+    const int G = n >= want ? 1 : 2 * n >= want ? 2 : 4 * n >= want ? 4 : 8;
+    const int blocks = (int)((n * G + 255) / 256), more = colout ? (cols + 7) / 8 : 0;
+    auto kernel = G == 1 ? k_sum_splits<1> : G == 2 ? k_sum_splits<2> : G == 4 ? k_sum_splits<4> : k_sum_splits<8>;
+    kernel<<<blocks + more, 256, 0, st>>>(part, splits, n, out, blocks, colpart, rows, cols, colout);
     PAT_LAUNCH_CHECK("k_sum_splits");
     return PAT_OK;
 }

@@ -53,6 +53,7 @@ def test_halo_convolution_edges(b, h, w, cin, cout, relu, shift):
 @pytest.mark.parametrize("b,h,w,cin,cout", [
     (90, 15, 15, 32, 32), (40, 17, 33, 32, 64), (20, 33, 31, 32, 128), (24, 25, 47, 64, 32), (10, 63, 65, 64, 64),
     (40, 9, 16, 96, 64), (13, 40, 49, 192, 64), (20, 24, 32, 128, 32),
+    (2, 16, 16, 128, 128), (1, 9, 8, 160, 128), (3, 8, 9, 192, 192),   # other kernels, 4, 2 and 1 warps per sum of splits
     (90, 15, 15, 8, 32), (40, 17, 33, 32, 8), (24, 33, 31, 16, 24), (40, 24, 32, 64, 16), (28, 31, 41, 24, 128),
 ])
 def test_halo_weight_gradient_edges(b, h, w, cin, cout):
