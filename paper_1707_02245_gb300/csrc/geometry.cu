@@ -935,6 +935,7 @@ extern "C" int pat_create_geometry(const pat_geometry_desc* desc, pat_geometry**
         delete g;
         return rc;
     }
+    solve_pool_users(g->device, 1);
     *out = g;
     return PAT_OK;
 }
@@ -1067,6 +1068,7 @@ extern "C" void pat_destroy_geometry(pat_geometry* g) {
     cudaSetDevice(g->device);
     cudaDeviceSynchronize();
     free_tables(g);
+    solve_pool_users(g->device, -1);
     cudaSetDevice(cur);
     delete g;
 }

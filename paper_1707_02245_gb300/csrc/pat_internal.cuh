@@ -251,6 +251,9 @@ __device__ __forceinline__ void point_coords(const G& g, float2 det, float r, fl
     t.j0 = (int)fly;
 }
 
+// Counts the geometries of a device; with the last, the solves' memory pool gives back what it keeps.
+void solve_pool_users(int dev, int change);
+
 // Programmatic dependent launch of the iteration's kernels.  Near its end every CTA lets the
 // next launch start (dependents_may_start; once all CTAs have, it starts on the SMs that are
 // free), and reads only what no kernel writes (arguments, maps, geometry tables) before
