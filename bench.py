@@ -728,10 +728,10 @@ def time_unet_step(P, WS, torch, net, x8, t8, cw, n, stream, steps=10):
     return {"step_ms": step_ms,
             "roofline": {"bound": "tensor", "achieved": tf, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
                          "frac": tf / peaks["bf16_tflops"], "flop_per_step": step_fl,
-                         "kernels": "k_conv_wgrad_tc (tcgen05, TMEM accumulators, TMA) for every weight gradient; "
-                                    "k_conv_fwd_tc for the forward and data-gradient layers with 32-channel multiples "
-                                    "and >= 64 channels on one side; k_conv_fwd (mma.sync) for the 8-channel input "
-                                    "and output layers and the 32 -> 32 forward",
+                         "kernels": "k_conv_halo and k_conv_wgrad_halo (tcgen05, TMEM accumulators, TMA; one staged "
+                                    "tile for all taps) for the layers of 32 to 96 input and up to 128 output channels; "
+                                    "k_conv_fwd_tc and k_conv_wgrad_tc (the same units, a tile per tap) for the wider "
+                                    "ones; k_conv_fwd (mma.sync) for the forward layers of 8 input channels",
                          "peak_source": "measured bf16 burst (MEASURED_PEAKS.json)"}}
 
 
