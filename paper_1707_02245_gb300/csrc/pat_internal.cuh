@@ -338,8 +338,9 @@ struct FwdArgs {
     const float* step_mul; // {tau multiplier s, sigma multiplier 1/s} (device) or NULL
     float* qw;             // rows of row_stride(T)
     unsigned* qmax_bits;
-    double* partials;      // FWD_GAP: term c of K CTA i at [c * n_part + i]
-    int n_part;            // K CTAs of the problem
+    double* partials;      // FWD_GAP: term c of CTA i at [c * n_part + i]
+    int n_part;            // FWD_GAP: CTAs of the problem; those from n_ctas on only take pixels
+    int n_ctas;            // CTAs of the plan
     const int* stop;
 };
 
