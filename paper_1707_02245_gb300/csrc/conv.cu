@@ -23,6 +23,7 @@
 #include <algorithm>
 #include <mutex>
 
+#include "device_once.h"
 #include "nn_internal.cuh"
 #include "pat_internal.cuh"
 
@@ -1530,14 +1531,20 @@ __global__ void k_flip_weights(const bf16* __restrict__ w, int cout, int cin, bf
     wf[i] = w[((size_t)o * 9 + (8 - t)) * cin + c];
 }
 
+// Raises the kernel's limit of dynamic shared memory on the current device: a host-side attribute
+// of the function (no stream work; allowed under graph capture) that each device keeps by itself.
+int raise_smem(DeviceOnce& once, const void* kernel, int bytes) {
+    int dev = 0;
+    PAT_CUDA(cudaGetDevice(&dev));
+    const int e = once.run(dev, [&] { return (int)cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes); });
+    return e == 0 ? PAT_OK : cuda_fail((cudaError_t)e, "shared-memory limit of a convolution kernel");
+}
+
 template <int BN, bool F32>
 int launch_fwd(const FwdArgs& a, cudaStream_t st) {
     const size_t smem = (size_t)STAGES * (FBM + BN) * FROW * sizeof(bf16);
-    // a host-side attribute of the function (no stream work; allowed under graph capture),
-    // set once
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_conv_fwd<BN, F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    PAT_CUDA(attr);
+    static DeviceOnce once;
+    if (const int rc = raise_smem(once, (const void*)k_conv_fwd<BN, F32>, (int)smem)) return rc;
     const long long P = (long long)a.B * a.H * a.W;
     dim3 grid((unsigned)((P + FBM - 1) / FBM), (unsigned)((a.cout + BN - 1) / BN));
     k_conv_fwd<BN, F32><<<grid, THREADS, smem, st>>>(a);
@@ -1615,10 +1622,8 @@ int launch_fwd_tc(const FwdArgs& f, cudaStream_t st) {
     r = enc(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)f.w, dB, sB, bB, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3: weight tensor map");
-    // a host-side attribute of the function (allowed under graph capture), set once
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_conv_fwd_tc<BN, F32>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    PAT_CUDA(attr);
+    static DeviceOnce once;
+    if (const int rc = raise_smem(once, (const void*)k_conv_fwd_tc<BN, F32>, C::SMEM)) return rc;
     const int grid = (int)std::min<long long>(total, sm_count());
     k_conv_fwd_tc<BN, F32><<<grid, TC_THREADS, C::SMEM, st>>>(ma, mb, a);
     PAT_LAUNCH_CHECK("k_conv_fwd_tc");
@@ -1687,10 +1692,8 @@ int launch_halo_cin(const FwdArgs& f, const HaloArgs& a, cudaStream_t st) {
     r = enc(&mb, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, (void*)f.w, dB, sB, bB, es, CU_TENSOR_MAP_INTERLEAVE_NONE, sw,
             CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3: weight tensor map");
-    // a host-side attribute of the function (allowed under graph capture), set once
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_conv_halo<F32, CB, NQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, H_SMEM);
-    PAT_CUDA(attr);
+    static DeviceOnce once;
+    if (const int rc = raise_smem(once, (const void*)k_conv_halo<F32, CB, NQ>, H_SMEM)) return rc;
     const int per = std::min(std::max(1, sm_count() / a.tiles_n), a.tiles);   // CTAs of one N tile
     k_conv_halo<F32, CB, NQ><<<per * a.tiles_n, H_THREADS, halo_smem(CB * NQ, CB, a.bn, a.stages), st>>>(ma, mb, a);
     PAT_LAUNCH_CHECK("k_conv_halo");
@@ -1776,9 +1779,8 @@ int launch_wgrad_tc(const View& x, const View& dz, int B, int H, int W, int cin,
     };
     if (map4(&mx, x, cin, a.cbx) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: activation tensor map");
     if (map4(&md, dz, cout, a.cbo) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: gradient tensor map");
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_conv_wgrad_tc<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    PAT_CUDA(attr);
+    static DeviceOnce once;
+    if (const int rc = raise_smem(once, (const void*)k_conv_wgrad_tc<BN>, C::SMEM)) return rc;
     k_conv_wgrad_tc<BN><<<std::min(a.total, sm_count()), TC_THREADS, C::SMEM, st>>>(mx, md, a);
     PAT_LAUNCH_CHECK("k_conv_wgrad_tc");
     return launch_sum_splits(part, a.splits, (long long)cout * K, dw, colpart, colrows, cout, db, st);
@@ -1815,9 +1817,8 @@ int launch_wgrad_halo(const View& x, const View& dz, int B, int H, int W, int ci
     };
     if (map4(&mx, x, cin, CB, GPX, GPY) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: activation tensor map");
     if (map4(&md, dz, cout, C::CBO, GTX, GTY) != CUDA_SUCCESS) return fail(PAT_ERR_CUDA, "conv3x3_wgrad: gradient tensor map");
-    static const cudaError_t attr =
-        cudaFuncSetAttribute(k_conv_wgrad_halo<CB, BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
-    PAT_CUDA(attr);
+    static DeviceOnce once;
+    if (const int rc = raise_smem(once, (const void*)k_conv_wgrad_halo<CB, BN>, C::SMEM)) return rc;
     k_conv_wgrad_halo<CB, BN><<<splits * a.nq, TC_THREADS, C::SMEM, st>>>(mx, md, a);
     PAT_LAUNCH_CHECK("k_conv_wgrad_halo");
     return launch_sum_splits(part, splits, 9LL * cin * cout, dw, colpart, colrows, cout, db, st);
