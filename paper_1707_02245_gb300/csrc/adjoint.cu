@@ -137,13 +137,16 @@ __device__ __forceinline__ unsigned max_of_slots(const unsigned* slots, int n) {
     return m;
 }
 
-// max |y| comes from a.ymax_bits, or (n_slots > 0) is the maximum of that many block maxima.
+// n_items work items of one tile, from item_index on, whose records follow one another.  max |y|
+// comes from a.ymax_bits, or (n_slots > 0) is the maximum of that many block maxima.
 template <bool PREMUL>
-__device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index, const unsigned* slots = nullptr,
-                                             int n_slots = 0) {
+__device__ __forceinline__ void adjoint_items(const AdjArgs& a, int item_index, int n_items, const unsigned* slots = nullptr,
+                                              int n_slots = 0) {
     const int N = a.g.n;
-    const int4 item = __ldg(reinterpret_cast<const int4*>(a.items + item_index));
-    const int tile = item.x, nrec = item.z, split = item.w;
+    const int4* __restrict__ items = reinterpret_cast<const int4*>(a.items + item_index);
+    int4 item = __ldg(items);
+    const int tile = item.x;
+    int nrec = item.z, split = item.w;
     const int x0 = (tile % a.wtiles_x) * WTILE, y0 = (tile / a.wtiles_x) * WTILE;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ __align__(16) int acc[ACELL * ASTRIDE];
@@ -182,14 +185,26 @@ __device__ __forceinline__ void adjoint_item(const AdjArgs& a, int item_index, c
             }
         };
         float4 geo, seg;
-        while (first < split) {
-            advance(geo, seg);
-            adjoint_segment<PREMUL, false>(ac, geo, seg, y, sub2, bx, by, cells);
-        }
-        cells += AKIND;
-        while (first < nrec) {
-            advance(geo, seg);
-            adjoint_segment<PREMUL, true>(ac, geo, seg, y, sub2, by, bx, cells);
+        while (true) {
+            while (first < split) {
+                advance(geo, seg);
+                adjoint_segment<PREMUL, false>(ac, geo, seg, y, sub2, bx, by, cells);
+            }
+            while (first < nrec) {
+                advance(geo, seg);
+                adjoint_segment<PREMUL, true>(ac, geo, seg, y, sub2, by, bx, cells + AKIND);
+            }
+            if (--n_items == 0) break;
+            recs += 2 * nrec;
+            item = __ldg(++items);
+            nrec = item.z;
+            split = item.w;
+            first = warp * AROWS;
+            j = first + lane / ALANES;
+            if (j < nrec) {
+                q = __ldg(recs + 2 * j);
+                s = __ldg(recs + 2 * j + 1);
+            }
         }
     }
     __syncthreads();
@@ -220,7 +235,7 @@ template <bool PREMUL>
 __global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles(const __grid_constant__ AdjArgs a,
                                                                             const unsigned* __restrict__ slots, int n_slots,
                                                                             unsigned* __restrict__ ymax_out) {
-    adjoint_item<PREMUL>(a, blockIdx.x, slots, n_slots);
+    adjoint_items<PREMUL>(a, blockIdx.x, 1, slots, n_slots);
     if (blockIdx.x == 0) {
         const unsigned m = max_of_slots(slots, n_slots);
         if (threadIdx.x == 0) *ymax_out = m;
@@ -265,8 +280,8 @@ template <bool PREMUL>
 __global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles_b(const AdjArgs* __restrict__ args,
                                                             const int2* __restrict__ map) {
     const int2 pm = map[blockIdx.x];
-    const AdjArgs& a = args[pm.x];   // (a shared copy would be reloaded after every shared atomic)
-    adjoint_item<PREMUL>(a, pm.y);
+    const AdjArgs& a = args[adj_map_problem(pm)];   // (a shared copy would be reloaded after every shared atomic)
+    adjoint_items<PREMUL>(a, pm.y, adj_map_count(pm));
 }
 
 // out = the fixed-point K^T image in floating point
@@ -314,6 +329,40 @@ int adjoint_blocks_per_sm() {
         n = 4;
     }
     return n;
+}
+
+// Waves of CTAs a batch's K^T keeps.  A geometry's items fill one wave, so a batch of B has B waves
+// of them, and with few candidates an item is mostly its CTA's fixed cost: the chain of loads before
+// the first point, and clearing, merging and flushing the accumulators.  Beyond this many waves a
+// CTA takes several items of a tile.  us per launch with one item each, with 3 waves, (2, 8): 64
+// problems of 64^2 with 64 detectors 203, 87 (91, 90); 8 of them 26.7, 18.6 (15.1, 26.7); 16 of
+// 256^2 with 128 139, 120 (123, 127); 4 of 256^2 with 256 62.4, 62.4 (65.3, 62.4); 8 uneven ones
+// 61.4, 55.9 (53.0, 61.4).
+constexpr int ADJ_BATCH_WAVES = 3;
+
+std::vector<int2> adjoint_map(const pat_geometry* const* g, int B) {
+    long long total = 0;
+    for (int b = 0; b < B; ++b) total += g[b]->adj_items;
+    const long long slots = (long long)sm_count() * adjoint_blocks_per_sm();
+    const int most = (int)std::min<long long>(ADJ_MAP_ITEMS, std::max<long long>(1, total / (ADJ_BATCH_WAVES * slots)));
+    std::vector<std::pair<float, int2>> v;
+    for (int b = 0; b < B; ++b) {
+        const std::vector<int>& tile = g[b]->adj_item_tile;
+        for (int i = 0, n; i < g[b]->adj_items; i += n) {
+            for (n = 1; i + n < g[b]->adj_items && tile[i + n] == tile[i]; ++n) {}
+            const int parts = ceil_div(n, most);
+            for (int p = 0; p < parts; ++p) {
+                const int i0 = i + n * p / parts, i1 = i + n * (p + 1) / parts;
+                float cost = 0.f;
+                for (int k = i0; k < i1; ++k) cost += g[b]->adj_item_cost[k];
+                v.push_back({cost, adj_map_entry(b, i0, i1 - i0)});
+            }
+        }
+    }
+    std::stable_sort(v.begin(), v.end(), [](const std::pair<float, int2>& x, const std::pair<float, int2>& y) { return x.first > y.first; });
+    std::vector<int2> map;
+    for (const auto& e : v) map.push_back(e.second);
+    return map;
 }
 
 int launch_adjoint_b(const AdjArgs* args, const int2* map, int nblocks, bool premul, cudaStream_t st) {

@@ -848,6 +848,23 @@ static int install_adjoint_plan(pat_geometry* g, const PointTables& pt, int wave
     AdjWork aw;
     const int rc = adjoint_worklist(dd, pt, (double)sm_count() * adjoint_blocks_per_sm(), aw, 1 << 30, waves);
     if (rc) return rc;
+    // the items of a tile together, the tile with the heaviest item first
+    std::vector<int> rank(aw.wtiles, -1), order(aw.items.size());
+    int ranks = 0;
+    for (size_t i = 0; i < order.size(); ++i) {
+        order[i] = (int)i;
+        if (rank[aw.items[i].tile] < 0) rank[aw.items[i].tile] = ranks++;
+    }
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return rank[aw.items[a].tile] < rank[aw.items[b].tile]; });
+    std::vector<AdjItem> by_tile;
+    std::vector<float> cost;
+    std::vector<int> tile;
+    for (const int i : order) {
+        by_tile.push_back(aw.items[i]);
+        cost.push_back(aw.cost[i]);
+        tile.push_back(aw.items[i].tile);
+    }
+    aw.items.swap(by_tile);
     std::vector<AdjRec> recs;
     std::vector<AdjWorkItem> items;
     adjoint_records(dd, pt, aw, recs, items);
@@ -870,7 +887,8 @@ static int install_adjoint_plan(pat_geometry* g, const PointTables& pt, int wave
     g->adj_tiles = aw.tiles;
     g->adj_wtiles_x = aw.wtiles_x;
     g->adj_candidates = aw.candidates;
-    g->adj_item_cost = aw.cost;
+    g->adj_item_cost = cost;
+    g->adj_item_tile = tile;
     g->adj_items = (int)items.size();
     g->shapes.adjoint_waves = waves;
     return PAT_OK;

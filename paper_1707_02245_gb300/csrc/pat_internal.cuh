@@ -167,6 +167,7 @@ struct pat_geometry {
     int adj_tiles_x = 0, adj_tiles = 0, adj_items = 0;   // scale tiles (ATILE) per row, in all; items
     int adj_wtiles_x = 0;              // work tiles (WTILE) per row
     long long adj_candidates = 0;     // candidate points of one K^T application
+    std::vector<int> adj_item_tile;    // work tile per work item; the items of a tile are neighbours (host)
     std::vector<float> adj_item_cost;  // estimated cost per work item (host)
     int4* fwd_units = nullptr;         // K work units (see GeomView)
     int4* fwd_ctas = nullptr;          // K CTAs
@@ -352,7 +353,16 @@ struct AdjGeom {
     float dr_f, rh_f;
 };
 
-struct AdjArgs {       // fixed-point K^T y, one work item per block
+// An entry of K^T's launch map: problem, first work item and how many of them (1 to 128, all of
+// one tile) a CTA takes.
+inline int2 adj_map_entry(int problem, int item, int count) { return make_int2(problem | (count - 1) << 24, item); }
+__device__ __forceinline__ int adj_map_problem(int2 pm) { return pm.x & 0xffffff; }
+__device__ __forceinline__ int adj_map_count(int2 pm) { return 1 + (int)((unsigned)pm.x >> 24); }
+constexpr int ADJ_MAP_ITEMS = 128;
+// The map of B problems' K^T: every work item of every problem, heaviest entries first.
+std::vector<int2> adjoint_map(const pat_geometry* const* g, int B);
+
+struct AdjArgs {       // fixed-point K^T y
     AdjGeom g;
     const float* y;          // data rows, or data rows times the arc weights (premul)
     int premul;

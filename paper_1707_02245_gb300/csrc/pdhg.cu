@@ -949,19 +949,15 @@ static void build_iter_plan(const Prob* pr, int B, Arena& ar, IterPlan& ip, int*
     // maps: forward rows problem by problem; K^T items of all problems heaviest first;
     // update tiles grouped by regulariser
     std::vector<int2> upd[3][UPD_TILES];
-    std::vector<std::pair<float, int2>> adj;
+    std::vector<const pat_geometry*> gs;
     for (int b = 0; b < B; ++b) {
         const pat_geometry* g = pr[b].g;
-        for (int i = 0; i < g->adj_items; ++i) adj.push_back({g->adj_item_cost[i], make_int2(b, i)});
+        gs.push_back(g);
         const int tile = g->shapes.update_tile;
         const int N = g->desc.n, nt = ceil_div(N, upd_tx(tile)) * ceil_div(N, upd_ty(tile));
         for (int i = 0; i < nt; ++i) upd[pr[b].p.reg][tile].push_back(make_int2(b, i));
     }
-    std::stable_sort(adj.begin(), adj.end(), [](const std::pair<float, int2>& x, const std::pair<float, int2>& y) {
-        return x.first > y.first;
-    });
-    std::vector<int2> adjm;
-    for (auto& e : adj) adjm.push_back(e.second);
+    const std::vector<int2> adjm = adjoint_map(gs.data(), B);
     ip.map_adj = ar.put(adjm.data(), adjm.size());
     ip.n_adj = (int)adjm.size();
     for (int r = 0; r < 3; ++r)
@@ -1372,7 +1368,6 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
         std::vector<FwdArgs> fw[2], fg;
         std::vector<AdjArgs> ad[2];
         std::vector<FinalArgs> fi;
-        std::vector<std::pair<float, int2>> order;
         std::vector<Prob> prs(B);
         for (int b = 0; b < B; ++b) {
             InfoDev* in = inf(b);
@@ -1399,7 +1394,6 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
             fg.push_back(ga);
             fi.push_back(FinalArgs{(double*)buf(b, DPART), g[b]->fwd_n_ctas, (double*)buf(b, PPART), n_pix, p[b].alpha,
                                    0.0, p[b].box_u, p[b].box_v, p[b].tol, PAT_WAV, PAT_ADAPT_NONE, in, stopped});
-            for (int i = 0; i < g[b]->adj_items; ++i) order.push_back({g[b]->adj_item_cost[i], make_int2(b, i)});
             prs[b].g = g[b];
         }
         for (int par = 0; par < 2; ++par) {
@@ -1409,10 +1403,7 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
         fg_off = ar.put(fg.data(), fg.size());
         fi_off = ar.put(fi.data(), fi.size());
         forward_groups(prs.data(), B, ar, gp);
-        std::stable_sort(order.begin(), order.end(),
-                         [](const std::pair<float, int2>& x, const std::pair<float, int2>& y) { return x.first > y.first; });
-        std::vector<int2> am;
-        for (auto& e : order) am.push_back(e.second);
+        const std::vector<int2> am = adjoint_map(g, B);
         n_adj = (int)am.size();
         amap_off = ar.put(am.data(), am.size());
         rc = ar.upload(&dev, st);
@@ -2399,8 +2390,7 @@ static int gap_impl(const pat_geometry* g, const float* f, const pat_params* p, 
         forward_groups(&pr, 1, ar, gp);
         AdjArgs aa = make_adj_args(g, y, nullptr, &pr.ws.info->qmax_bits[0], pr.ws.kt[0], nullptr);
         const size_t adj_off = ar.put(&aa, 1);
-        std::vector<int2> amap(g->adj_items);
-        for (int i = 0; i < g->adj_items; ++i) amap[i] = make_int2(0, i);
+        const std::vector<int2> amap = adjoint_map(&g, 1);
         const size_t amap_off = ar.put(amap.data(), amap.size());
         FwdArgs fa = make_fwd_args(g, x);
         fa.q = const_cast<float*>(y);   // read only by the gap epilogue
@@ -2415,7 +2405,7 @@ static int gap_impl(const pat_geometry* g, const float* f, const pat_params* p, 
         rc = ar.upload(&dev, st);
         if (!rc) {
             char* b = (char*)dev;
-            rc = launch_adjoint_b((const AdjArgs*)(b + adj_off), (const int2*)(b + amap_off), g->adj_items, false, st);
+            rc = launch_adjoint_b((const AdjArgs*)(b + adj_off), (const int2*)(b + amap_off), (int)amap.size(), false, st);
             if (!rc)
                 rc = launch_gap_phase((const FwdArgs*)(b + fa_off), (const GapArgs*)(b + ga_off),
                                       (const FinalArgs*)(b + fi_off), gp, b, st);
