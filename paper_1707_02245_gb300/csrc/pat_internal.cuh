@@ -78,7 +78,8 @@ struct GeomView {
     // units {detector, window 0, window 1, (k group << 16) | row group's index in its
     // round}; a window is m_first | count << 16.  A CTA's units are stored round by round.
     const int4* units;
-    const int4* ctas;    // per K CTA (cluster-major, rank-minor): {first entry in rgs, row groups, first entry in roff, 0}
+    const int4* ctas;    // per K CTA (cluster-major, rank-minor): {first entry in rgs, row groups, first entry in roff, 0};
+                         // then zeros for a gap's CTAs that only take pixels
     const int* roff;     // per CTA: unit offsets of its rounds (rounds + 1 entries)
     const int* rgs;      // per cluster: its row groups in processing order
 };
@@ -174,6 +175,7 @@ struct pat_geometry {
     int* fwd_roff = nullptr;           // per CTA: unit offsets of its rounds
     int* fwd_rgs = nullptr;            // per cluster: its row groups
     int fwd_n_ctas = 0, fwd_smem = 0;  // K CTAs of one application (clusters x S); dynamic shared memory
+    int gap_ctas = 0;                  // ... and of a gap evaluation
     long long fwd_evaluated = 0;       // quadrature points inside the units' windows
     std::vector<float> fwd_cluster_cost; // points each K cluster's slowest CTA evaluates (host)
     std::vector<double> det_xy;        // detector positions (host copy, 2 per detector)
@@ -340,8 +342,7 @@ struct FwdArgs {
     float* qw;             // rows of row_stride(T)
     unsigned* qmax_bits;
     double* partials;      // FWD_GAP: term c of CTA i at [c * n_part + i]
-    int n_part;            // FWD_GAP: CTAs of the problem; those from n_ctas on only take pixels
-    int n_ctas;            // CTAs of the plan
+    int n_part;            // FWD_GAP: CTAs of the problem
     const int* stop;
 };
 

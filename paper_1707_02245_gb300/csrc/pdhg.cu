@@ -600,22 +600,10 @@ void solve_pool_users(int dev, int change) {
 
 static int pix_blocks(int N) { return std::min(4 * sm_count(), ceil_div((long long)N * N, 256)); }
 
-// CTAs of a gap evaluation: those of K's plan, and more that take pixels only (in whole clusters)
-// where K's would leave a thread several pixels while SMs idle: K has one cluster for eight radii
-// of a detector at most, so with few data a few CTAs would pass over the whole image, in one long
-// FP32 sum per thread.  As many as one pixel per thread asks for, within one wave (the partition of
-// a pixel pass of its own).  Solves of 100 iterations, gap every 10th, one detector of 16 samples,
-// TV / TGV: 1024^2 15.9 / 39.2 -> 5.4 / 7.8 ms, 512^2 6.2 / 9.9 -> 3.8 / 4.1 ms.
-static int gap_ctas(const pat_geometry* g) {
-    const int nt = forward_threads(g->fwd_smem), S = g->view.n_slabs;
-    const int wave = sm_count() * (nt == FWD_THREADS ? 2 : 1);
-    return std::max(g->fwd_n_ctas, std::min(ceil_div((long long)g->desc.n * g->desc.n, nt), wave) / S * S);
-}
-
 static int alloc_workspace(const pat_geometry* g, int reg, Workspace& ws, cudaStream_t st) {
     const size_t N = g->desc.n, NN = N * N, S = (size_t)g->desc.n_det * g->desc.n_t;
     const size_t nx = NN * (reg == PAT_TGV ? 3 : 1), ny = NN * (reg == PAT_TGV ? 5 : 2);
-    ws.n_part = gap_ctas(g);
+    ws.n_part = g->gap_ctas;
     size_t off[16];
     size_t sz[16] = {nx * 4, nx * 4, ny * 4, ny * 4, S * 4, NN * 4, NN * 4 * 2,
                      (reg == PAT_TGV ? 2 * NN : 1) * 4,

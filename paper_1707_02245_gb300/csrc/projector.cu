@@ -286,9 +286,8 @@ __device__ __forceinline__ void forward_cta(const FwdArgs& a, const int2 pm, con
     const GeomView& g = a.g;
     const int N = g.n, T = g.n_t, S = g.n_slabs, M = g.quad_m, D = g.n_det;
     const unsigned rank = S > 1 ? cluster_rank() : 0u;
-    // (whole clusters of a gap launch may have no row groups: see gap_ctas)
-    const bool pixels_only = EPI == FWD_GAP && pm.y >= a.n_ctas;
-    const int4 cta = pixels_only ? make_int4(0, 0, 0, 0) : __ldg(&g.ctas[pm.y]);
+    // (whole clusters of a gap launch may have no row groups and only take pixels: see gap_ctas)
+    const int4 cta = __ldg(&g.ctas[pm.y]);
     const int rg0 = cta.x, n_rg = cta.y;
     const int* roff = g.roff + cta.z;
     const bool smem_img = g.slab_rows > 0;
@@ -297,7 +296,7 @@ __device__ __forceinline__ void forward_cta(const FwdArgs& a, const int2 pm, con
     int4* s_units = reinterpret_cast<int4*>(smem + L.units);
     const int jlo = smem_img ? (int)rank * g.slab_rows - 1 : -1;
     const int reff = smem_img ? min(g.slab_rows, N - jlo) : N + 1;
-    if (smem_img && !pixels_only) {
+    if (smem_img && (EPI != FWD_GAP || n_rg > 0)) {
         float2* s_cs = reinterpret_cast<float2*>(smem + L.cs);
         float2* s_det = reinterpret_cast<float2*>(smem + L.det);
         for (int i = threadIdx.x; i < 2 * M; i += NT) s_cs[i] = __ldg(&g.cs[i < M ? i : i - M]);
@@ -308,7 +307,7 @@ __device__ __forceinline__ void forward_cta(const FwdArgs& a, const int2 pm, con
     // (every CTA of a cluster reads the same flag, so a stopped problem's clusters leave
     // together, before any cluster barrier)
     if (a.stop && *(volatile const int*)a.stop) return;
-    if (smem_img && !pixels_only)
+    if (smem_img && (EPI != FWD_GAP || n_rg > 0))
         stage_slab<NT>(a.img, N, g.slab_stride, jlo, reff + 1, reinterpret_cast<float*>(smem + L.slab));
     if (threadIdx.x == 0) s_qmax = 0u;
     const int lane = threadIdx.x & 31;
@@ -502,7 +501,6 @@ FwdArgs make_fwd_args(const pat_geometry* g, const float* img) {
     memset(&a, 0, sizeof a);
     a.g = g->view;
     a.img = img;
-    a.n_ctas = g->fwd_n_ctas;
     return a;
 }
 
