@@ -137,14 +137,13 @@ __device__ __forceinline__ unsigned max_of_slots(const unsigned* slots, int n) {
     return m;
 }
 
-// n_items work items of one tile, from item_index on, whose records follow one another.  max |y|
-// comes from a.ymax_bits, or (n_slots > 0) is the maximum of that many block maxima.
-template <bool PREMUL>
-__device__ __forceinline__ void adjoint_items(const AdjArgs& a, int item_index, int n_items, const unsigned* slots = nullptr,
-                                              int n_slots = 0) {
+// n_items work items of one tile: item (with SEVERAL: items[0], items[1], ...).  max |y| comes from
+// a.ymax_bits, or (n_slots > 0) is the maximum of that many block maxima.
+template <bool PREMUL, bool SEVERAL>
+__device__ __forceinline__ void adjoint_items(const AdjArgs& a, int item_index, const int* __restrict__ items, int n_items,
+                                              const unsigned* slots = nullptr, int n_slots = 0) {
     const int N = a.g.n;
-    const int4* __restrict__ items = reinterpret_cast<const int4*>(a.items + item_index);
-    int4 item = __ldg(items);
+    int4 item = __ldg(reinterpret_cast<const int4*>(a.items + (SEVERAL ? __ldg(items) : item_index)));
     const int tile = item.x;
     int nrec = item.z, split = item.w;
     const int x0 = (tile % a.wtiles_x) * WTILE, y0 = (tile / a.wtiles_x) * WTILE;
@@ -194,9 +193,9 @@ __device__ __forceinline__ void adjoint_items(const AdjArgs& a, int item_index, 
                 advance(geo, seg);
                 adjoint_segment<PREMUL, true>(ac, geo, seg, y, sub2, by, bx, cells + AKIND);
             }
-            if (--n_items == 0) break;
-            recs += 2 * nrec;
-            item = __ldg(++items);
+            if (!SEVERAL || --n_items == 0) break;
+            item = __ldg(reinterpret_cast<const int4*>(a.items + __ldg(++items)));
+            recs = reinterpret_cast<const float4*>(a.recs + item.y);
             nrec = item.z;
             split = item.w;
             first = warp * AROWS;
@@ -235,7 +234,7 @@ template <bool PREMUL>
 __global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles(const __grid_constant__ AdjArgs a,
                                                                             const unsigned* __restrict__ slots, int n_slots,
                                                                             unsigned* __restrict__ ymax_out) {
-    adjoint_items<PREMUL>(a, blockIdx.x, 1, slots, n_slots);
+    adjoint_items<PREMUL, false>(a, blockIdx.x, nullptr, 1, slots, n_slots);
     if (blockIdx.x == 0) {
         const unsigned m = max_of_slots(slots, n_slots);
         if (threadIdx.x == 0) *ymax_out = m;
@@ -276,12 +275,13 @@ __global__ void __launch_bounds__(512) k_adjoint_prep(const float* __restrict__ 
     dependents_may_start();
 }
 
-template <bool PREMUL>
+template <bool PREMUL, bool SEVERAL>
 __global__ void __launch_bounds__(ATHREADS, ADJ_MIN_BLOCKS) k_adjoint_tiles_b(const AdjArgs* __restrict__ args,
-                                                            const int2* __restrict__ map) {
+                                                                              const int2* __restrict__ map,
+                                                                              const int* __restrict__ list) {
     const int2 pm = map[blockIdx.x];
     const AdjArgs& a = args[adj_map_problem(pm)];   // (a shared copy would be reloaded after every shared atomic)
-    adjoint_items<PREMUL>(a, pm.y, adj_map_count(pm));
+    adjoint_items<PREMUL, SEVERAL>(a, pm.y, list + pm.y, adj_map_count(pm));
 }
 
 // out = the fixed-point K^T image in floating point
@@ -324,7 +324,7 @@ AdjArgs make_adj_args(const pat_geometry* g, const float* y, const float* premul
 
 int adjoint_blocks_per_sm() {
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_adjoint_tiles_b<true>, ATHREADS, 0) != cudaSuccess || n < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_adjoint_tiles_b<true, true>, ATHREADS, 0) != cudaSuccess || n < 1) {
         cudaGetLastError();
         n = 4;
     }
@@ -334,38 +334,44 @@ int adjoint_blocks_per_sm() {
 // Waves of CTAs a batch's K^T keeps.  A geometry's items fill one wave, so a batch of B has B waves
 // of them, and with few candidates an item is mostly its CTA's fixed cost: the chain of loads before
 // the first point, and clearing, merging and flushing the accumulators.  Beyond this many waves a
-// CTA takes several items of a tile.  us per launch with one item each, with 3 waves, (2, 8): 64
-// problems of 64^2 with 64 detectors 203, 87 (91, 90); 8 of them 26.7, 18.6 (15.1, 26.7); 16 of
-// 256^2 with 128 139, 120 (123, 127); 4 of 256^2 with 256 62.4, 62.4 (65.3, 62.4); 8 uneven ones
-// 61.4, 55.9 (53.0, 61.4).
+// CTA takes several items of a tile.  us per launch with one item a CTA and with this rule: 64
+// problems of 64^2 with 64 detectors 204, 91; 8 of them 26.8, 19.2; 64 of 32^2 with 16 44, 25; 8 of
+// 96^2 with 330 171, 74; 16 of 256^2 with 128 139, 121; 8 uneven ones 61.6, 57.0.  2 waves cost 4
+// problems of 256^2 with 256 detectors 65.3 against 62.4; 8 waves left the 8 of 64^2 at 26.7.
 constexpr int ADJ_BATCH_WAVES = 3;
 
-std::vector<int2> adjoint_map(const pat_geometry* const* g, int B) {
+AdjMap adjoint_map(const pat_geometry* const* g, int B) {
     long long total = 0;
     for (int b = 0; b < B; ++b) total += g[b]->adj_items;
-    const long long slots = (long long)sm_count() * adjoint_blocks_per_sm();
-    const int most = (int)std::min<long long>(ADJ_MAP_ITEMS, std::max<long long>(1, total / (ADJ_BATCH_WAVES * slots)));
+    const int most = (int)std::min<long long>(ADJ_MAP_ITEMS, std::max<long long>(1, total / (ADJ_BATCH_WAVES * g[0]->adj_slots)));
+    AdjMap map;
+    map.several = most > 1;
     std::vector<std::pair<float, int2>> v;
     for (int b = 0; b < B; ++b) {
-        const std::vector<int>& tile = g[b]->adj_item_tile;
-        for (int i = 0, n; i < g[b]->adj_items; i += n) {
-            for (n = 1; i + n < g[b]->adj_items && tile[i + n] == tile[i]; ++n) {}
+        const std::vector<float>& cost = g[b]->adj_item_cost;
+        const std::vector<int>&tile = g[b]->adj_item_tile, &by_tile = g[b]->adj_by_tile;
+        const int items = g[b]->adj_items;
+        for (int i = 0; !map.several && i < items; ++i) v.push_back({cost[i], adj_map_entry(b, i, 1)});
+        for (int i = 0, n; map.several && i < items; i += n) {
+            for (n = 1; i + n < items && tile[by_tile[i + n]] == tile[by_tile[i]]; ++n) {}
             const int parts = ceil_div(n, most);
             for (int p = 0; p < parts; ++p) {
                 const int i0 = i + n * p / parts, i1 = i + n * (p + 1) / parts;
-                float cost = 0.f;
-                for (int k = i0; k < i1; ++k) cost += g[b]->adj_item_cost[k];
-                v.push_back({cost, adj_map_entry(b, i0, i1 - i0)});
+                float sum = 0.f;
+                for (int k = i0; k < i1; ++k) sum += cost[by_tile[k]];
+                v.push_back({sum, adj_map_entry(b, (int)map.list.size(), i1 - i0)});
+                map.list.insert(map.list.end(), by_tile.begin() + i0, by_tile.begin() + i1);
             }
         }
     }
-    std::stable_sort(v.begin(), v.end(), [](const std::pair<float, int2>& x, const std::pair<float, int2>& y) { return x.first > y.first; });
-    std::vector<int2> map;
-    for (const auto& e : v) map.push_back(e.second);
+    if (B > 1 || map.several)   // (a geometry's items are heaviest first)
+        std::stable_sort(v.begin(), v.end(), [](const std::pair<float, int2>& x, const std::pair<float, int2>& y) { return x.first > y.first; });
+    for (const auto& e : v) map.entries.push_back(e.second);
     return map;
 }
 
-int launch_adjoint_b(const AdjArgs* args, const int2* map, int nblocks, bool premul, cudaStream_t st) {
+int launch_adjoint_b(const AdjArgs* args, const int2* map, const int* list, int nblocks, bool several, bool premul,
+                     cudaStream_t st) {
     if (nblocks <= 0) return PAT_OK;
     prof_mark(PAT_PHASE_ADJOINT, st, true);
     cudaLaunchConfig_t cfg = {};
@@ -376,8 +382,9 @@ int launch_adjoint_b(const AdjArgs* args, const int2* map, int nblocks, bool pre
     set_dependent_launch(attr[0]);
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = premul ? cudaLaunchKernelEx(&cfg, k_adjoint_tiles_b<true>, args, map)
-                                 : cudaLaunchKernelEx(&cfg, k_adjoint_tiles_b<false>, args, map);
+    auto kernel = premul ? (several ? k_adjoint_tiles_b<true, true> : k_adjoint_tiles_b<true, false>)
+                         : (several ? k_adjoint_tiles_b<false, true> : k_adjoint_tiles_b<false, false>);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args, map, list);
     if (e != cudaSuccess) return cuda_fail(e, "k_adjoint_tiles_b");
     PAT_LAUNCH_CHECK("k_adjoint_tiles_b");
     prof_mark(PAT_PHASE_ADJOINT, st, false);

@@ -534,7 +534,7 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
     const std::vector<float2>& cs = pt.cs;
     // K^T candidate boxes: for every WTILE x WTILE work tile and detector, the (k, m)
     // polar box of the tile's tap region (points with i0 in [x0-1, x0+WTILE-1], same in
-    // y), with one index of margin on every WTILE; FP64 on the host
+    // y), with one index of margin on every side; FP64 on the host
     w.tiles_x = (N + ATILE - 1) / ATILE;
     w.tiles = w.tiles_x * w.tiles_x;
     const int tiles_x = (N + WTILE - 1) / WTILE, tiles = tiles_x * tiles_x;
@@ -717,9 +717,9 @@ static int adjoint_worklist(const pat_geometry_desc& d, const PointTables& pt, d
 // lies in its share [c0, c1), so segments stay whole.  Neighbouring records go to the lanes
 // of one warp, so each kind is sorted longest first and the first kind is filled up to whole
 // warps with empty records.
-static void adjoint_records(const pat_geometry_desc& d, const PointTables& pt, const AdjWork& w,
-                            std::vector<AdjRec>& recs, std::vector<AdjWorkItem>& items) {
-    const int Tp = row_stride(d.n_t);
+static int adjoint_records(const pat_geometry_desc& d, const PointTables& pt, const AdjWork& w,
+                           std::vector<AdjRec>& recs, std::vector<AdjWorkItem>& items) {
+    const long long Tp = row_stride(d.n_t);
     auto longest = [](const AdjRec& a, const AdjRec& b) { return a.n > b.n; };
     recs.reserve(w.rays.size() + w.items.size() * AROWS);
     std::vector<AdjRec> kind[2];
@@ -739,10 +739,21 @@ static void adjoint_records(const pat_geometry_desc& d, const PointTables& pt, c
         std::stable_sort(kind[0].begin(), kind[0].end(), longest);
         std::stable_sort(kind[1].begin(), kind[1].end(), longest);
         while (kind[0].size() % AROWS) kind[0].push_back(AdjRec{});
+        if (recs.size() + kind[0].size() + kind[1].size() > (size_t)((1LL << 31) - 1))
+            return fail(PAT_ERR_INVALID_ARG, "pat_create_geometry: K^T work list too large");
         items.push_back(AdjWorkItem{it.tile, (int)recs.size(), (int)(kind[0].size() + kind[1].size()), (int)kind[0].size()});
         recs.insert(recs.end(), kind[0].begin(), kind[0].end());
         recs.insert(recs.end(), kind[1].begin(), kind[1].end());
     }
+    return PAT_OK;
+}
+
+// What the K^T kernel reads, for a GPU that holds `slots` K^T CTAs: the work list w of whole
+// segments, in `waves` waves of items, and its records.
+static int adjoint_plan(const pat_geometry_desc& d, const PointTables& pt, double slots, int waves, AdjWork& w,
+                        std::vector<AdjRec>& recs, std::vector<AdjWorkItem>& items) {
+    const int rc = adjoint_worklist(d, pt, slots, w, 1 << 30, waves);
+    return rc ? rc : adjoint_records(d, pt, w, recs, items);
 }
 
 // Angular windows of every (detector, group of KGRP radii): the smallest circular interval
@@ -860,28 +871,11 @@ static int install_adjoint_plan(pat_geometry* g, const PointTables& pt, int wave
     pat_geometry_desc dd = g->desc;
     dd.det_xy_host = g->det_xy.data();
     AdjWork aw;
-    const int rc = adjoint_worklist(dd, pt, (double)sm_count() * adjoint_blocks_per_sm(), aw, 1 << 30, waves);
-    if (rc) return rc;
-    // the items of a tile together, the tile with the heaviest item first
-    std::vector<int> rank(aw.wtiles, -1), order(aw.items.size());
-    int ranks = 0;
-    for (size_t i = 0; i < order.size(); ++i) {
-        order[i] = (int)i;
-        if (rank[aw.items[i].tile] < 0) rank[aw.items[i].tile] = ranks++;
-    }
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return rank[aw.items[a].tile] < rank[aw.items[b].tile]; });
-    std::vector<AdjItem> by_tile;
-    std::vector<float> cost;
-    std::vector<int> tile;
-    for (const int i : order) {
-        by_tile.push_back(aw.items[i]);
-        cost.push_back(aw.cost[i]);
-        tile.push_back(aw.items[i].tile);
-    }
-    aw.items.swap(by_tile);
     std::vector<AdjRec> recs;
     std::vector<AdjWorkItem> items;
-    adjoint_records(dd, pt, aw, recs, items);
+    const long long slots = (long long)sm_count() * adjoint_blocks_per_sm();
+    const int rc = adjoint_plan(dd, pt, (double)slots, waves, aw, recs, items);
+    if (rc) return rc;
     AdjRec* r_dev = nullptr;
     AdjWorkItem* it_dev = nullptr;
     cudaError_t e = cudaMalloc(&r_dev, sizeof(AdjRec) * std::max<size_t>(recs.size(), 1));
@@ -901,8 +895,15 @@ static int install_adjoint_plan(pat_geometry* g, const PointTables& pt, int wave
     g->adj_tiles = aw.tiles;
     g->adj_wtiles_x = aw.wtiles_x;
     g->adj_candidates = aw.candidates;
-    g->adj_item_cost = cost;
-    g->adj_item_tile = tile;
+    g->adj_item_cost = aw.cost;
+    g->adj_item_tile.clear();
+    g->adj_by_tile.clear();
+    for (const AdjWorkItem& it : items) {
+        g->adj_by_tile.push_back((int)g->adj_by_tile.size());
+        g->adj_item_tile.push_back(it.tile);
+    }
+    std::stable_sort(g->adj_by_tile.begin(), g->adj_by_tile.end(), [&](int a, int b) { return items[a].tile < items[b].tile; });
+    g->adj_slots = slots;
     g->adj_items = (int)items.size();
     g->shapes.adjoint_waves = waves;
     return PAT_OK;

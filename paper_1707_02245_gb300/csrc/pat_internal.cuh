@@ -164,11 +164,13 @@ struct pat_geometry {
     float* wk = nullptr;
     int2* win = nullptr;
     pat::AdjRec* adj_rec = nullptr;        // K^T ray segments of the work items
-    pat::AdjWorkItem* adj_item = nullptr;  // K^T work items, one CTA each
+    pat::AdjWorkItem* adj_item = nullptr;  // K^T work items, heaviest first
     int adj_tiles_x = 0, adj_tiles = 0, adj_items = 0;   // scale tiles (ATILE) per row, in all; items
     int adj_wtiles_x = 0;              // work tiles (WTILE) per row
     long long adj_candidates = 0;     // candidate points of one K^T application
-    std::vector<int> adj_item_tile;    // work tile per work item; the items of a tile are neighbours (host)
+    std::vector<int> adj_item_tile;    // work tile per work item (host)
+    std::vector<int> adj_by_tile;      // the work items, those of a tile together (host)
+    long long adj_slots = 1;           // K^T CTAs that the device holds at once
     std::vector<float> adj_item_cost;  // estimated cost per work item (host)
     int4* fwd_units = nullptr;         // K work units (see GeomView)
     int4* fwd_ctas = nullptr;          // K CTAs
@@ -354,14 +356,19 @@ struct AdjGeom {
     float dr_f, rh_f;
 };
 
-// An entry of K^T's launch map: problem, first work item and how many of them (1 to 128, all of
-// one tile) a CTA takes.
+// An entry of K^T's launch map: problem, and the work item of a CTA; or, where CTAs take several (1 to
+// 128, of one tile), their number and the first one's place in the map's list of items.
 inline int2 adj_map_entry(int problem, int item, int count) { return make_int2(problem | (count - 1) << 24, item); }
 __device__ __forceinline__ int adj_map_problem(int2 pm) { return pm.x & 0xffffff; }
 __device__ __forceinline__ int adj_map_count(int2 pm) { return 1 + (int)((unsigned)pm.x >> 24); }
 constexpr int ADJ_MAP_ITEMS = 128;
 // The map of B problems' K^T: every work item of every problem, heaviest entries first.
-std::vector<int2> adjoint_map(const pat_geometry* const* g, int B);
+struct AdjMap {
+    std::vector<int2> entries;
+    std::vector<int> list;
+    bool several = false;   // entries refer to the list
+};
+AdjMap adjoint_map(const pat_geometry* const* g, int B);
 
 struct AdjArgs {       // fixed-point K^T y
     AdjGeom g;
@@ -393,7 +400,8 @@ int launch_forward_b(int epi, const FwdArgs* args, const int2* map, int nblocks,
 int forward_smem_bytes(int rows, int stride, int M, int D, bool staged);
 int forward_clusters_per_gpu(int cluster, int smem);   // K clusters the GPU holds at once
 int forward_threads(int smem);                         // threads of a K CTA with this shared memory
-int launch_adjoint_b(const AdjArgs* args, const int2* map, int nblocks, bool premul, cudaStream_t st);
+int launch_adjoint_b(const AdjArgs* args, const int2* map, const int* list, int nblocks, bool several, bool premul,
+                     cudaStream_t st);
 // CTAs of the K^T kernel that one SM holds at once (sizes the work items)
 int adjoint_blocks_per_sm();
 

@@ -886,6 +886,8 @@ struct IterPlan {
     size_t fin = 0, map_adj = 0;
     size_t map_upd[3][UPD_TILES] = {};
     int n_adj = 0;
+    bool adj_several = false;
+    size_t adj_list = 0;
     int n_upd[3][UPD_TILES] = {};
     GapPlan gp;
 };
@@ -945,9 +947,11 @@ static void build_iter_plan(const Prob* pr, int B, Arena& ar, IterPlan& ip, int*
         const int N = g->desc.n, nt = ceil_div(N, upd_tx(tile)) * ceil_div(N, upd_ty(tile));
         for (int i = 0; i < nt; ++i) upd[pr[b].p.reg][tile].push_back(make_int2(b, i));
     }
-    const std::vector<int2> adjm = adjoint_map(gs.data(), B);
-    ip.map_adj = ar.put(adjm.data(), adjm.size());
-    ip.n_adj = (int)adjm.size();
+    const AdjMap adjm = adjoint_map(gs.data(), B);
+    ip.map_adj = ar.put(adjm.entries.data(), adjm.entries.size());
+    ip.n_adj = (int)adjm.entries.size();
+    ip.adj_several = adjm.several;
+    ip.adj_list = ar.put(adjm.list.data(), adjm.list.size());
     for (int r = 0; r < 3; ++r)
         for (int t = 0; t < UPD_TILES; ++t) {
             ip.map_upd[r][t] = ar.put(upd[r][t].data(), upd[r][t].size());
@@ -960,7 +964,8 @@ static int enqueue_iteration(const IterPlan& ip, const char* base, int it, bool 
     const int par = it & 1;
     int rc = launch_forward_groups(FWD_PROX, (const FwdArgs*)(base + ip.fwd[par]), ip.gp, base, st);
     if (rc) return rc;
-    rc = launch_adjoint_b((const AdjArgs*)(base + ip.adj[par]), (const int2*)(base + ip.map_adj), ip.n_adj, true, st);
+    rc = launch_adjoint_b((const AdjArgs*)(base + ip.adj[par]), (const int2*)(base + ip.map_adj),
+                          (const int*)(base + ip.adj_list), ip.n_adj, ip.adj_several, true, st);
     if (rc) return rc;
     const UpdateArgs* ua = (const UpdateArgs*)(base + ip.upd[par][gap_due ? 1 : 0]);
     for (int r = 0; r < 3; ++r)
@@ -1352,6 +1357,8 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
     size_t fw_off[2] = {0, 0}, ad_off[2] = {0, 0}, fg_off = 0, fi_off = 0, amap_off = 0;
     GapPlan gp;
     int n_adj = 0;
+    bool adj_several = false;
+    size_t alist_off = 0;
     if (!rc) {
         std::vector<FwdArgs> fw[2], fg;
         std::vector<AdjArgs> ad[2];
@@ -1391,9 +1398,11 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
         fg_off = ar.put(fg.data(), fg.size());
         fi_off = ar.put(fi.data(), fi.size());
         forward_groups(prs.data(), B, ar, gp);
-        const std::vector<int2> am = adjoint_map(g, B);
-        n_adj = (int)am.size();
-        amap_off = ar.put(am.data(), am.size());
+        const AdjMap am = adjoint_map(g, B);
+        n_adj = (int)am.entries.size();
+        adj_several = am.several;
+        alist_off = ar.put(am.list.data(), am.list.size());
+        amap_off = ar.put(am.entries.data(), am.entries.size());
         rc = ar.upload(&dev, st);
     }
     const char* base = (const char*)dev;
@@ -1416,7 +1425,8 @@ static int run_wavelet(int B, const pat_geometry* const* g, const float* const* 
             if (!e) e = launch_wav_dual(r, wb, sigr, in->step_mul, scal, NN, &in->stop, s, B, ps);
         }
         if (!e)
-            e = launch_adjoint_b((const AdjArgs*)(base + ad_off[par]), (const int2*)(base + amap_off), n_adj, true, s);
+            e = launch_adjoint_b((const AdjArgs*)(base + ad_off[par]), (const int2*)(base + amap_off),
+                                 (const int*)(base + alist_off), n_adj, adj_several, true, s);
         if (cwt) {
             if (!e) e = launch_cwt_synthesis(scrt, N, J, wm.bank, wtr, scr, &in->stop, s, B, ps);
         } else {
@@ -1717,8 +1727,8 @@ static int time_phases(int B, const pat_geometry* const* g, const float* const* 
             if (ph == PAT_PHASE_FORWARD_PROX)
                 return launch_forward_groups(FWD_PROX, (const FwdArgs*)(base + ip.fwd[0]), ip.gp, base, ls);
             if (ph == PAT_PHASE_ADJOINT)
-                return launch_adjoint_b((const AdjArgs*)(base + ip.adj[0]), (const int2*)(base + ip.map_adj), ip.n_adj,
-                                        true, ls);
+                return launch_adjoint_b((const AdjArgs*)(base + ip.adj[0]), (const int2*)(base + ip.map_adj),
+                                        (const int*)(base + ip.adj_list), ip.n_adj, ip.adj_several, true, ls);
             if (ph == PAT_PHASE_UPDATE) {
                 const UpdateArgs* ua = (const UpdateArgs*)(base + ip.upd[0][0]);
                 for (int r = 0; r < 3; ++r)
@@ -2378,8 +2388,9 @@ static int gap_impl(const pat_geometry* g, const float* f, const pat_params* p, 
         forward_groups(&pr, 1, ar, gp);
         AdjArgs aa = make_adj_args(g, y, nullptr, &pr.ws.info->qmax_bits[0], pr.ws.kt[0], nullptr);
         const size_t adj_off = ar.put(&aa, 1);
-        const std::vector<int2> amap = adjoint_map(&g, 1);
-        const size_t amap_off = ar.put(amap.data(), amap.size());
+        const AdjMap amap = adjoint_map(&g, 1);
+        const size_t amap_off = ar.put(amap.entries.data(), amap.entries.size());
+        const size_t alist_off = ar.put(amap.list.data(), amap.list.size());
         FwdArgs fa = make_fwd_args(g, x);
         fa.q = const_cast<float*>(y);   // read only by the gap epilogue
         fa.f = f;
@@ -2393,7 +2404,8 @@ static int gap_impl(const pat_geometry* g, const float* f, const pat_params* p, 
         rc = ar.upload(&dev, st);
         if (!rc) {
             char* b = (char*)dev;
-            rc = launch_adjoint_b((const AdjArgs*)(b + adj_off), (const int2*)(b + amap_off), (int)amap.size(), false, st);
+            rc = launch_adjoint_b((const AdjArgs*)(b + adj_off), (const int2*)(b + amap_off),
+                                  (const int*)(b + alist_off), (int)amap.entries.size(), amap.several, false, st);
             if (!rc)
                 rc = launch_gap_phase((const FwdArgs*)(b + fa_off), (const GapArgs*)(b + ga_off),
                                       (const FinalArgs*)(b + fi_off), gp, b, st);
