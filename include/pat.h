@@ -399,7 +399,7 @@ int  pat_adjoint_worklist(const pat_geometry_desc* desc, int slots, int* rays_ho
  * units' windows, dynamic shared memory of a CTA in bytes, round offsets}.  When not NULL:
  *   units_host: 4 ints per unit {detector, window 0, window 1, (k / 8) << 16 | the row
  *     group's index in its round}; a window is m_first | count << 16, a circular range of
- *     angles;
+ *     angles (with T > 2^19 this format does not hold k / 8: PAT_ERR_INVALID_ARG);
  *   ctas_host: 4 ints per CTA, cluster-major and rank-minor {first entry in rgs, row
  *     groups of the cluster, first entry in roff, 0};
  *   roff_host: per CTA, unit offsets of its rounds (rounds + 1 entries);

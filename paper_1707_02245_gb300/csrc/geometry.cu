@@ -333,7 +333,7 @@ static void cover_two(const unsigned char* mask, int M, unsigned& w0, unsigned& 
 
 struct SlabPlan {
     int slabs = 1, rows = 0, stride = 0, smem = 0;
-    std::vector<int4> units;     // per CTA, round by round: {detector, window 0, window 1, k group << 16 | index}
+    std::vector<int4> units;     // per CTA, round by round: {detector, window 0, window 1, k group * FWD_ROUND + index}
     std::vector<int4> ctas;      // per CTA (cluster-major, rank-minor): {first rg entry, row groups, first roff entry, 0}
     std::vector<int> roff;       // per CTA: unit offsets of its rounds
     std::vector<int> rgs;        // per cluster: its row groups in processing order
@@ -503,7 +503,7 @@ static void build_slab_plan(const pat_geometry_desc& d, const PointTables& pt, c
                     const int rg = mem[e.second];
                     const U& u = units[(size_t)rg * S + s];
                     const int dd = rg / n_kgrp, kg = rg - dd * n_kgrp;
-                    sp.units.push_back(make_int4(dd, (int)u.w0, (int)u.w1, (kg << 16) | (e.second - rd * FWD_ROUND)));
+                    sp.units.push_back(make_int4(dd, (int)u.w0, (int)u.w1, (int)((unsigned)kg * FWD_ROUND + (unsigned)(e.second - rd * FWD_ROUND))));
                     tot += e.first;
                 }
             }
@@ -1034,11 +1034,14 @@ extern "C" int pat_forward_plan(const pat_geometry_desc* desc, int budget_bytes,
     if ((units_host && units_cap < info8_host[3]) || (ctas_host && ctas_cap < info8_host[4]) ||
         (roff_host && roff_cap < info8_host[7]) || (rgs_host && rgs_cap < (long long)sp.rgs.size()))
         return fail(PAT_ERR_INVALID_ARG, "pat_forward_plan: output capacity too small");
+    if (units_host && desc->n_t > (KGRP << 16))
+        return fail(PAT_ERR_INVALID_ARG, "pat_forward_plan: the units' format holds 65536 groups of radii");
     for (size_t i = 0; units_host && i < sp.units.size(); ++i) {
         units_host[4 * i] = sp.units[i].x;
         units_host[4 * i + 1] = sp.units[i].y;
         units_host[4 * i + 2] = sp.units[i].z;
-        units_host[4 * i + 3] = sp.units[i].w;
+        const unsigned w = (unsigned)sp.units[i].w;
+        units_host[4 * i + 3] = (int)((w / FWD_ROUND) << 16 | w % FWD_ROUND);
     }
     for (size_t i = 0; ctas_host && i < sp.ctas.size(); ++i) {
         ctas_host[4 * i] = sp.ctas[i].x;

@@ -75,7 +75,7 @@ struct GeomView {
     int slab_rows;       // R (0: global-memory variant)
     int slab_stride;     // shared-memory row stride in floats (W = 4 mod 8, >= N + 6)
     int smem_bytes;      // dynamic shared memory of a K CTA of this plan
-    // units {detector, window 0, window 1, (k group << 16) | row group's index in its
+    // units {detector, window 0, window 1, k group * FWD_ROUND + row group's index in its
     // round}; a window is m_first | count << 16.  A CTA's units are stored round by round.
     const int4* units;
     const int4* ctas;    // per K CTA (cluster-major, rank-minor): {first entry in rgs, row groups, first entry in roff, 0};

@@ -235,14 +235,14 @@ __device__ __forceinline__ void forward_units(const FwdArgs& a, int ub, int ue, 
         if (u >= ue) break;
         const int4 un = s_units[u - ub];
         const int d = un.x;
-        const int k = (un.w >> 16) * KGRP + kl;
+        const int k = (int)((unsigned)un.w / FWD_ROUND) * KGRP + kl;
         const bool valid = k < T;
         const float r = radius(valid ? k : 0, dr_f, rh_f);   // = rk[k], bit for bit
         const float2 det = SMEM ? s_det[d] : __ldg(&g.det[d]);
         const float acc = unit_partial<SMEM>(g, cs_s, a.img, img_s, jlo, reff, (unsigned)un.y, (unsigned)un.z, det, r,
                                              valid, ph);
         const float sum = phase_sum(acc);
-        if (ph == 0) s_acc[(un.w & 0xffff) * KGRP + kl] = sum;
+        if (ph == 0) s_acc[((unsigned)un.w % FWD_ROUND) * KGRP + kl] = sum;
     }
 }
 
