@@ -385,6 +385,19 @@ int  pat_geometry_info(const pat_geometry* g, long long* out6_host);
 int  pat_adjoint_worklist(const pat_geometry_desc* desc, int slots, int* rays_host, long long rays_cap,
                           int* items_host, long long items_cap, long long* counts3_host);
 
+/* Host only (no CUDA call): what the K^T kernel reads of that work list.  counts2_host =
+ * {records, work items}.  A record (8 four-byte words) is a ray segment of a tile: floats {dm, ds,
+ * cm, cs}, the detector coordinate and direction (in pixels) along the ray's faster axis (m) and the
+ * other one (s); unsigned {index of its first datum in rows of T padded to an even length, the same
+ * in rows of T}; float: its first radius index, even (past 2^24 a multiple of 16, and 16 points at
+ * most); int: its number of points from there.
+ * A work item (4 ints: tile, first record, records, split) holds the segments that begin in its
+ * share: those that advance faster along x, then, from record `split` on, those along y, each kind
+ * longest first and the first kind filled up to a multiple of 4 with empty records.  Outputs and
+ * capacities as above; slots must be at least 1. */
+int  pat_adjoint_records(const pat_geometry_desc* desc, int slots, void* recs_host, long long recs_cap,
+                         int* items_host, long long items_cap, long long* counts2_host);
+
 /* Host only: the work plan of the forward projector K (Sec. 3.3.1, eq. (K_def)) that
  * pat_create_geometry builds for `desc`.  Row group rg = d * ceil(T/8) + k/8 holds 8
  * consecutive radii of one detector.  The image is cut into S horizontal slabs of R rows

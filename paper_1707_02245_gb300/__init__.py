@@ -34,7 +34,7 @@ EXPORTED = [
     "pat_create_geometry", "pat_destroy_geometry", "pat_forward", "pat_adjoint",
     "pat_direction_field", "pat_params_default", "pat_reconstruct", "pat_reconstruct_batched",
     "pat_steps", "pat_duality_gap", "pat_error_string", "pat_last_error", "pat_geometry_info",
-    "pat_adjoint_worklist",
+    "pat_adjoint_records", "pat_adjoint_worklist",
     "pat_profile_enable", "pat_profile_read", "pat_kernel_launches", "pat_adjoint_noalloc",
     "pat_tune_step_ratio", "pat_tune_step_ratio_batched", "pat_preprocess", "pat_wavelet_transform",
     "pat_dtcwt_transform",
@@ -103,6 +103,9 @@ class pat_info(ctypes.Structure):
         return {k: getattr(self, k) for k, _ in self._fields_}
 
 
+ADJ_RECORD = np.dtype([("dm", "f4"), ("ds", "f4"), ("cm", "f4"), ("cs", "f4"), ("ypad", "u4"), ("yraw", "u4"),
+                       ("k", "f4"), ("n", "i4")])
+
 _lib = None
 
 
@@ -151,6 +154,8 @@ def load(path: str | None = None) -> ctypes.CDLL:
         "pat_geometry_info": (i, [vp, ctypes.POINTER(ctypes.c_longlong)]),
         "pat_adjoint_worklist": (i, [ctypes.POINTER(pat_geometry_desc), i, vp, ctypes.c_longlong, vp,
                                      ctypes.c_longlong, ctypes.POINTER(ctypes.c_longlong)]),
+        "pat_adjoint_records": (i, [ctypes.POINTER(pat_geometry_desc), i, vp, ctypes.c_longlong, vp,
+                                    ctypes.c_longlong, ctypes.POINTER(ctypes.c_longlong)]),
         "pat_forward_plan": (i, [ctypes.POINTER(pat_geometry_desc), i, i, vp, ctypes.c_longlong, vp,
                                  ctypes.c_longlong, vp, ctypes.c_longlong, vp, ctypes.c_longlong,
                                  ctypes.POINTER(ctypes.c_longlong)]),
@@ -239,6 +244,21 @@ def pat_adjoint_worklist(n: int, det_xy, n_t: int, r0: float, dr: float, quad_m:
     _check(lib.pat_adjoint_worklist(ctypes.byref(desc), slots, rays.ctypes.data, cnt[0], items.ctypes.data, cnt[1],
                                     cnt), "pat_adjoint_worklist")
     return {"rays": rays, "items": items, "candidates": int(cnt[2])}
+
+
+def pat_adjoint_records(n: int, det_xy, n_t: int, r0: float, dr: float, quad_m: int, slots: int,
+                        extent=(-1.0, 1.0, -1.0, 1.0)) -> dict:
+    """What the K^T kernel reads of its work list (host only; see include/pat.h): records (a
+    structured array) and items (I x 4: tile, first record, records, split)."""
+    lib = load()
+    desc, _det = _geometry_desc(n, det_xy, n_t, r0, dr, quad_m, extent)
+    cnt = (ctypes.c_longlong * 2)()
+    _check(lib.pat_adjoint_records(ctypes.byref(desc), slots, None, 0, None, 0, cnt), "pat_adjoint_records")
+    recs = np.zeros(cnt[0], dtype=ADJ_RECORD)
+    items = np.zeros((cnt[1], 4), dtype=np.int32)
+    _check(lib.pat_adjoint_records(ctypes.byref(desc), slots, recs.ctypes.data, cnt[0], items.ctypes.data, cnt[1], cnt),
+           "pat_adjoint_records")
+    return {"records": recs, "items": items}
 
 
 def pat_forward_plan(n: int, det_xy, n_t: int, r0: float, dr: float, quad_m: int, sms: int,

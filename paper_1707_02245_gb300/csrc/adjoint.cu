@@ -86,7 +86,7 @@ __device__ __forceinline__ void adjoint_segment(const AdjConst& a, const float4 
         if (PREMUL) {
             yv = __ldg(reinterpret_cast<const float2*>(yp + p));
         } else {   // (the caller's array may lie on any 4-byte boundary and its rows have no padding)
-            const int k = (int)seg.z + p;
+            const int k = min((int)seg.z + p, a.T - 1);   // (seg.z may be rounded beyond 2^28)
             yv = make_float2(__ldg(yp + p) * __ldg(a.wk + k), k + 1 < a.T ? __ldg(yp + p + 1) * __ldg(a.wk + k + 1) : 0.f);
         }
         const float2 c = __fmul2_rn(yv, a.scale);

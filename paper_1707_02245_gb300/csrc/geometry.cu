@@ -731,10 +731,21 @@ static int adjoint_records(const pat_geometry_desc& d, const PointTables& pt, co
             if (ray.w < it.c0) continue;   // begins in the item before
             const float2 det = pt.det[ray.x], cs = pt.cs[ray.y];
             const bool fast_y = std::fabs(cs.y) > std::fabs(cs.x);
-            const int k0 = ray.z & ~1, n = ray.z - k0 + w.rays[r + 1].w - ray.w;
-            AdjRec q{fast_y ? det.y : det.x, fast_y ? det.x : det.y, fast_y ? cs.y : cs.x, fast_y ? cs.x : cs.y,
-                     (unsigned)((long long)ray.x * Tp + k0), (unsigned)((long long)ray.x * d.n_t + k0), (float)k0, n};
-            kind[fast_y].push_back(q);
+            // Past AEXACT the index is rounded.  There a record holds one step of its lanes, from a
+            // multiple of that step: its own index is exact (to 2^28), and its lanes' are rounded once,
+            // as K's are.
+            constexpr int STEP = 2 * ALANES;
+            const int len = w.rays[r + 1].w - ray.w;
+            const bool exact = len <= AEXACT - ray.z;
+            const int k0 = ray.z & ~(exact ? 1 : STEP - 1), n = ray.z - k0 + len, most = exact ? n : STEP;
+            AdjRec q{fast_y ? det.y : det.x, fast_y ? det.x : det.y, fast_y ? cs.y : cs.x, fast_y ? cs.x : cs.y, 0u, 0u, 0.f, 0};
+            for (int i = 0; i < n; i += most) {
+                q.kf = (float)(k0 + i);
+                q.n = std::min(most, n - i);
+                q.ypad = (unsigned)(ray.x * Tp + k0 + i);
+                q.yraw = (unsigned)((long long)ray.x * d.n_t + k0 + i);
+                kind[fast_y].push_back(q);
+            }
         }
         std::stable_sort(kind[0].begin(), kind[0].end(), longest);
         std::stable_sort(kind[1].begin(), kind[1].end(), longest);
@@ -1094,6 +1105,26 @@ extern "C" int pat_adjoint_worklist(const pat_geometry_desc* desc, int slots, in
             o[3] = it.c0;
             o[4] = it.c1;
         }
+    return PAT_OK;
+}
+
+extern "C" int pat_adjoint_records(const pat_geometry_desc* desc, int slots, void* recs_host, long long recs_cap,
+                                   int* items_host, long long items_cap, long long* counts2_host) {
+    if (!desc || !counts2_host || slots < 1) return fail(PAT_ERR_INVALID_ARG, "pat_adjoint_records: bad argument");
+    const int vrc = check_desc(*desc);
+    if (vrc) return vrc;
+    AdjWork aw;
+    std::vector<AdjRec> recs;
+    std::vector<AdjWorkItem> items;
+    const int rc = adjoint_plan(*desc, point_tables(*desc), (double)slots, ADJ_WAVES, aw, recs, items);
+    if (rc) return rc;
+    counts2_host[0] = (long long)recs.size();
+    counts2_host[1] = (long long)items.size();
+    if ((recs_host && recs_cap < counts2_host[0]) || (items_host && items_cap < counts2_host[1]))
+        return fail(PAT_ERR_INVALID_ARG, "pat_adjoint_records: output capacity too small");
+    static_assert(sizeof(AdjRec) == 32 && sizeof(AdjWorkItem) == 16, "as the header says");
+    if (recs_host && !recs.empty()) memcpy(recs_host, recs.data(), recs.size() * sizeof(AdjRec));
+    if (items_host) memcpy(items_host, items.data(), items.size() * sizeof(AdjWorkItem));
     return PAT_OK;
 }
 

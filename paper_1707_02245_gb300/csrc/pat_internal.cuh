@@ -106,6 +106,7 @@ static_assert(ATILE % WTILE == 0, "work tiles nest in scale tiles");
 constexpr int ARAYS = 1024;    // most ray segments a work item of the exported work list holds
 constexpr int ALANES = 8;            // lanes of a warp that share one K^T ray segment (8: 18.8 us per launch, 16: 22.3)
 constexpr int AROWS = 32 / ALANES;   // ray segments a warp walks at once
+constexpr int AEXACT = 1 << 24;      // radius indexes up to here, and sums of them, are exact in FP32
 #ifndef PAT_ADJ_WAVES
 #define PAT_ADJ_WAVES 1
 #endif
