@@ -142,7 +142,8 @@ struct __align__(16) AdjRec {
 
 // Row length of the data times arc weights that K hands to K^T: T rounded up to even (the
 // odd entry is zero), so that pairs of data are 8-byte aligned.
-__host__ __device__ __forceinline__ int row_stride(int n_t) { return (n_t + 1) & ~1; }
+__host__ __device__ constexpr unsigned row_stride(int n_t) { return ((unsigned)n_t + 1u) & ~1u; }
+static_assert(row_stride(1) == 2 && row_stride(2) == 2 && row_stride(2147483647) == 2147483648u, "every n_t");
 
 struct PrecondCache {
     float* krow = nullptr;      // K 1 per data row (S), summed in FP64
