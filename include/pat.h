@@ -209,9 +209,13 @@ void pat_params_default(pat_params* p);
  *   ubar <- u+ + theta (u+ - u),  vbar <- v+ + theta (v+ - v)
  * with the box-restricted duality gap and residual of Sec. 3.3.3 evaluated in FP64 on
  * the device.  f_dev: D*T floats; u_dev: N*N floats, receives the final u.  *info
- * (host) is filled after the call synchronises `stream`.  Workspace is allocated from
- * the stream-ordered pool and released before returning.  Returns PAT_ERR_NONFINITE
- * (status DIVERGED) when the gap stops being finite. */
+ * (host) is filled after the call synchronises `stream`.  Returns PAT_ERR_NONFINITE
+ * (status DIVERGED) when the gap stops being finite.
+ * Device memory: the workspace is allocated in stream order and released before returning.  It
+ * comes from a stream-ordered pool of the library's own, one per device, which keeps up to
+ * 64 MiB of released memory for the next solve as long as a geometry lives on the device; the
+ * pat_destroy_geometry of the last one gives it back.  Where the application has set a pool for
+ * the device (cudaDeviceSetMemPool), that pool is used instead and the library keeps nothing. */
 int  pat_reconstruct(const pat_geometry* g, const float* f_dev, const pat_params* p,
                      float* u_dev, pat_info* info, void* stream);
 
@@ -236,7 +240,7 @@ int  pat_steps(const pat_geometry* g, const pat_params* p, float* sig_q_dev, flo
  * smallest relative gap after the probe wins.  best_host receives its s, and rel_gaps_host
  * (may be NULL) each probe's relative gap.  p's iters, tol, gap_every, adapt and outputs
  * are ignored; nothing is written to the caller's buffers.  The call synchronises
- * `stream`.  Scratch comes from the stream-ordered pool. */
+ * `stream`.  Scratch comes from the pool of pat_reconstruct. */
 int  pat_tune_step_ratio(const pat_geometry* g, const float* f_dev, const pat_params* p,
                          const double* candidates_host, int n_candidates, int probe_iters,
                          double* best_host, double* rel_gaps_host, void* stream);

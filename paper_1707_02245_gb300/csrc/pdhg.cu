@@ -559,19 +559,21 @@ struct Workspace {
 // default pool gives all its free memory back to the driver, so each solve mapped its workspace
 // anew (190 us a call: 200 TV iterations at 64^2 4.00 -> 3.82 ms, directional TV at 256^2 with 32
 // detectors 5.15 -> 4.96).  The library's own pool keeps up to 64 MiB (a 256^2 solve takes 10 to 20)
-// between solves while geometries live on the device, and gives it back with the last of them.
+// between solves while geometries live on the device, and gives it back with the last of them.  An
+// application that has set a pool of its own for the device (cudaDeviceSetMemPool) is served from that.
 // Allocations and frees are ordered by their streams, as in the default pool, from any thread.
 constexpr int POOL_DEVICES = 64;
 constexpr unsigned long long POOL_KEEP = 64ull << 20;
 static std::mutex g_pool_mtx;
-static cudaMemPool_t g_pool[POOL_DEVICES];
+static cudaMemPool_t g_pool[POOL_DEVICES], g_default_pool[POOL_DEVICES];
 static int g_pool_users[POOL_DEVICES];   // geometries alive
 
 static cudaError_t solve_alloc(void** ptr, size_t bytes, cudaStream_t st) {
     int dev = 0;
-    cudaMemPool_t pool = nullptr;
-    if (cudaGetDevice(&dev) == cudaSuccess && dev < POOL_DEVICES) {
+    cudaMemPool_t pool = nullptr, current = nullptr;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev < POOL_DEVICES && cudaDeviceGetMemPool(&current, dev) == cudaSuccess) {
         std::lock_guard<std::mutex> lock(g_pool_mtx);
+        if (!g_default_pool[dev] && cudaDeviceGetDefaultMemPool(&g_default_pool[dev], dev) != cudaSuccess) cudaGetLastError();
         if (!g_pool[dev]) {
             cudaMemPoolProps props = {};
             props.allocType = cudaMemAllocationTypePinned;
@@ -582,11 +584,12 @@ static cudaError_t solve_alloc(void** ptr, size_t bytes, cudaStream_t st) {
                 cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
                 g_pool[dev] = pool;
             } else {
-                cudaGetLastError();   // no pool of its own: the default one serves
-                pool = nullptr;
+                cudaGetLastError();   // no pool of its own: the device's serves
             }
         }
-        pool = g_pool[dev];
+        pool = current == g_default_pool[dev] ? g_pool[dev] : nullptr;
+    } else {
+        cudaGetLastError();
     }
     return pool ? cudaMallocFromPoolAsync(ptr, bytes, pool, st) : cudaMallocAsync(ptr, bytes, st);
 }
