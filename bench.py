@@ -355,7 +355,9 @@ def run_gb300(args) -> int:
         e2e_ms = e2e_ms[1:]
         e2e_s, e2e_units = aggregate(dist, sum(e2e_ms) / 1e3, float(iters * e2e_steps), device)
         e2e = {"value": e2e_units / e2e_s, "unit": UNIT, "h2d_bytes_per_step": f.numel() * 4,
-               "d2h_bytes_per_step": u.numel() * 4, "steps": e2e_steps}
+               "d2h_bytes_per_step": u.numel() * 4, "steps": e2e_steps,
+               # this rank's steps: a single slow one shows beside the median
+               "ms_median": sorted(e2e_ms)[len(e2e_ms) // 2], "ms_min": min(e2e_ms), "ms_max": max(e2e_ms)}
 
     # ---- time to relative gap 1e-4 (cold start): the paper's steps, and the balance s
     # chosen by the probe tuner (probe time included) ----
