@@ -28,15 +28,15 @@ namespace pat {
 // (in any order) into one image with integer atomics.
 //
 // Bound: issue slots and the shared-memory atomics together.  At 256^2 with 256 detectors
-// (8.4 M points): 18.8 us per launch, against 26.5 us for a kernel whose threads walked
+// (8.4 M points): 18.2 us per launch, against 26.5 us for a kernel whose threads walked
 // contiguous runs of the candidate list one point at a time: there nearly every step of a
 // warp held some lane's segment change, and its lanes' pixels lay on random banks (3.6
 // wavefronts per atomic, 19 M warp instructions).  64^2 with 64 detectors: 6.0 -> 5.2 us;
-// an uneven batch of 8: 77 -> 63 us.  Tiles of 64 pixels with 16 lanes to a segment: 19.2 us.
+// an uneven batch of 8: 77 -> 57 us.  Tiles of 64 pixels with 16 lanes to a segment: 19.2 us.
 // ---------------------------------------------------------------------------------
 // Threads of a K^T CTA and resident CTAs per SM.  Fewer, larger CTAs zero and flush fewer tile
-// copies; the 64 registers of 2 x 512 threads hold the loop without spills (measured at 256^2
-// on 64-pixel tiles: 2 x 512 19.2 us, 1 x 1024 19.9, 4 x 256 20.5, 3 x 512 with spills 30).
+// copies; the 64 registers of 2 x 512 threads hold the loop without spills (us per launch at
+// 256^2 / 64^2: 2 x 512 18.2 / 4.8, 1 x 1024 19.3 / 4.6, 4 x 256 18.7 / 5.3, 3 x 384 18.7 / 5.3).
 constexpr int ATHREADS = 512;
 constexpr int ADJ_MIN_BLOCKS = 2;
 constexpr int ACELL = WTILE + 3;     // cells per axis: the tile, its ring and one more for points outside

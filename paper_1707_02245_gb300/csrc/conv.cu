@@ -736,7 +736,8 @@ __global__ void __launch_bounds__(H_THREADS, 1)
         if (lane == 0) {
             // ---- MMA issuer ----
             const uint32_t idesc = tc_idesc(TBM, a.bn);
-            constexpr uint32_t layout = CB == 16 ? 6u : CB == 32 ? 4u : 2u;
+            static_assert(CB == 32 || CB == 64, "boxes of 64 or 128 bytes");
+            constexpr uint32_t layout = CB == 32 ? 4u : 2u;
             constexpr uint32_t row = CB * 2;   // bytes of a pixel (and of an output channel) in a box
             const uint64_t da = tc_desc(0, 16, HPX * row, layout), db = tc_desc(0, 16, 8 * row, layout) + (sB >> 4);
             const uint32_t b16 = b_reg >> 4;

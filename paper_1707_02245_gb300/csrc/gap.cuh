@@ -45,7 +45,7 @@ struct GapArgs {
 };
 
 // Adds the terms of pixels first, first + step, ... to acc: per-thread sums in FP32 (a thread
-// covers few pixels; the block's sums are FP32 pairs per warp and FP64 across warps, since
+// covers few pixels, see gap_ctas; the block's sums are FP32 pairs per warp and FP64 across warps, since
 // GB300's FP64 pipe runs at 1/64 of FP32).  The last term is the dual residual of the
 // regulariser duals (distance of their argument from the normal cone of the ball at r and s),
 // for the adaptive balance.

@@ -104,7 +104,7 @@ constexpr int ATILE = 32;      // side of the pixel tiles that share one K^T fix
 constexpr int WTILE = 32;      // side of the pixel tiles one K^T work item accumulates
 static_assert(ATILE % WTILE == 0, "work tiles nest in scale tiles");
 constexpr int ARAYS = 1024;    // most ray segments a work item of the exported work list holds
-constexpr int ALANES = 8;            // lanes of a warp that share one K^T ray segment (8: 18.8 us per launch, 16: 22.3)
+constexpr int ALANES = 8;            // lanes of a warp that share one K^T ray segment (8: 18.2 us per launch, 16: 22.3)
 constexpr int AROWS = 32 / ALANES;   // ray segments a warp walks at once
 constexpr int AEXACT = 1 << 24;      // radius indexes up to here, and sums of them, are exact in FP32
 #ifndef PAT_ADJ_WAVES
@@ -243,9 +243,9 @@ struct KtView {
 constexpr float FLOOR_MAGIC = 12582912.0f;   // 1.5 * 2^23, bits 0x4B400000
 constexpr int FLOOR_MAGIC_BITS = 0x4B400000;
 
-// Taps of a point without the grid test (callers that test a tile window instead).  The
-// floors are floorf (K's shared-memory loop takes the same floors by the exact round-down
-// add above; here floorf measured faster: K^T 26.3 against 29.4 us at 256^2).
+// Taps of a point without the grid test (K's loop over global taps adds its own).
+// The floors are floorf; K's shared-memory loop and K^T take the same floors by the exact
+// round-down add above, two points an instruction.
 template <class G>
 __device__ __forceinline__ void point_coords(const G& g, float2 det, float r, float2 cs, Taps& t) {
     const float fx = fmaf(r, cs.x, det.x);
@@ -330,9 +330,9 @@ __device__ __forceinline__ const T& stage_args(const T* __restrict__ args, int p
 // K applied to an N*N image for every row group of one problem, with one of three
 // epilogues on the finished rows: FWD_Y writes y = K img; FWD_PROX performs the data prox
 // q <- (q + sigma (K ubar - f)) / (1 + sigma) and records q w_k and max |q| for the K^T
-// that follows; FWD_GAP writes the per-row-group sums of the gap's data terms.
+// that follows; FWD_GAP writes each CTA's sums of the gap's terms.
 enum { FWD_Y = 0, FWD_PROX = 1, FWD_GAP = 2 };
-constexpr int GAP_DATA_TERMS = 4;   // per-row-group sums of the data pass: |Ku-f|^2, |q|^2, <q,f>, |q-(Ku-f)|_1
+constexpr int GAP_DATA_TERMS = 4;   // sums over data: |Ku-f|^2, |q|^2, <q,f>, |q-(Ku-f)|_1
 
 struct FwdArgs {
     GeomView g;
@@ -346,7 +346,7 @@ struct FwdArgs {
     float* qw;             // rows of row_stride(T)
     unsigned* qmax_bits;
     double* partials;      // FWD_GAP: term c of CTA i at [c * n_part + i]
-    int n_part;            // FWD_GAP: CTAs of the problem
+    int n_part;            // FWD_GAP: CTAs of the problem's gap evaluation
     const int* stop;
 };
 

@@ -113,7 +113,7 @@ __device__ __forceinline__ float unit_partial(const GeomView& g, unsigned cs_s, 
                     const float2 cs = lds2(vj ? csp + 8u * NPH * e : csp);
                     // position and taps; the FP32 arithmetic of the transpose (fx = fmaf(r, cs.x, det.x))
                     const float2 fp = __ffma2_rn(rr, cs, det);
-                    // exact floor (see point_coords): tp = floor(fp) + 1.5 * 2^23
+                    // exact floor (see FLOOR_MAGIC): tp = floor(fp) + 1.5 * 2^23
                     const float2 tp = __fadd2_rd(fp, magic);
                     const int li = __float_as_int(tp.x) - lbias, lj = __float_as_int(tp.y) - jbias;
                     const bool in = ((unsigned)lj < (unsigned)reff) & ((unsigned)li <= (unsigned)N) & vj;
@@ -256,8 +256,8 @@ struct GapShared {
 // The gap's pixel terms of pixels first, first + step, ... into t[GAP_DATA_TERMS..].  K's CTAs
 // take the pixels between them while their slabs are on the way, and the last CTA of the
 // problem adds up: one launch per gap evaluation.  With a pixel kernel of its own after K, an
-// evaluation took 30.0 us at 64^2 (64 detectors) and 47.0 us at 256^2 (256), now 17.4 and
-// 31.5, and 177 instead of 244 us for an uneven batch of 8.  What is left beside K is latency:
+// evaluation took 30.0 us at 64^2 (64 detectors) and 47.0 us at 256^2 (256), now 16.2 and
+// 32.6, and 177 instead of 244 us for an uneven batch of 8.  What is left beside K is latency:
 // the ticket, the loads of the partial sums and the FP64 pipe of one SM.
 __device__ __forceinline__ void gap_pixel_share(const GapArgs& g, int first, int step, float (&t)[GAP_TERMS]) {
     float acc[GAP_PIX_TERMS];
