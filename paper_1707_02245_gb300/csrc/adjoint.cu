@@ -428,10 +428,14 @@ int launch_adjoint(const pat_geometry* g, const float* y, float* out, cudaStream
     if (rc) return rc;
     char* scratch = nullptr;
     const size_t head = 4096, acc = ((size_t)g->desc.n * g->desc.n * sizeof(int) + 255) & ~(size_t)255;
-    const size_t bytes = head + acc + (size_t)g->desc.n_det * row_stride(g->desc.n_t) * sizeof(float);
-    PAT_CUDA(cudaMallocAsync((void**)&scratch, bytes, st));
+    const size_t weighted = (size_t)g->desc.n_det * row_stride(g->desc.n_t) * sizeof(float);
+    bool qw = cudaMallocAsync((void**)&scratch, head + acc + weighted, st) == cudaSuccess;
+    if (!qw) {   // no room for the weighted data: the kernel weights them itself
+        cudaGetLastError();
+        PAT_CUDA(cudaMallocAsync((void**)&scratch, head + acc, st));
+    }
     rc = launch_adjoint_into(g, y, (unsigned*)scratch, (int)(head / 4) - 1, (int*)(scratch + head),
-                             (float*)(scratch + head + acc), out, st);
+                             qw ? (float*)(scratch + head + acc) : nullptr, out, st);
     cudaFreeAsync(scratch, st);
     return rc;
 }
