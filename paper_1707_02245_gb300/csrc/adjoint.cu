@@ -346,7 +346,13 @@ AdjMap adjoint_map(const pat_geometry* const* g, int B) {
     const int most = (int)std::min<long long>(ADJ_MAP_ITEMS, std::max<long long>(1, total / (ADJ_BATCH_WAVES * g[0]->adj_slots)));
     AdjMap map;
     map.several = most > 1;
+    if (B == 1 && !map.several) {   // (a geometry's items are heaviest first)
+        map.entries.resize(g[0]->adj_items);
+        for (int i = 0; i < g[0]->adj_items; ++i) map.entries[i] = adj_map_entry(0, i, 1);
+        return map;
+    }
     std::vector<std::pair<float, int2>> v;
+    v.reserve((size_t)total);
     for (int b = 0; b < B; ++b) {
         const std::vector<float>& cost = g[b]->adj_item_cost;
         const std::vector<int>&tile = g[b]->adj_item_tile, &by_tile = g[b]->adj_by_tile;
@@ -364,8 +370,8 @@ AdjMap adjoint_map(const pat_geometry* const* g, int B) {
             }
         }
     }
-    if (B > 1 || map.several)   // (a geometry's items are heaviest first)
-        std::stable_sort(v.begin(), v.end(), [](const std::pair<float, int2>& x, const std::pair<float, int2>& y) { return x.first > y.first; });
+    std::stable_sort(v.begin(), v.end(), [](const std::pair<float, int2>& x, const std::pair<float, int2>& y) { return x.first > y.first; });
+    map.entries.reserve(v.size());
     for (const auto& e : v) map.entries.push_back(e.second);
     return map;
 }
